@@ -96,14 +96,33 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   const int64_t N = d.n_max, M = d.m_max, P = d.brute ? 0 : d.p_max;
   const size_t ncp = (size_t)d.grid.n_keys + 2;
   const size_t nb = d.brute ? 1 : (size_t)d.grid.n_buckets;
+  // what every build starts from zero, in one range from the header on
+  const int64_t tiles = (M + kWarp - 1) / kWarp;
   t.header = reinterpret_cast<DeviceHeader*>(take(sizeof(DeviceHeader)));
+  if (!d.brute) {
+    t.occ = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ((nb + 31) / 32)));
+    t.listed = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ((nb + 31) / 32)));
+    t.qbits = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ((ncp + 31) / 32)));
+  }
+  t.gpart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * gpart_words(N)));
+  t.qsort_ws = take(radix_sort_workspace_bytes(M, d.grid.key_bits));
+  t.osort_ws = take(radix_sort_workspace_bytes(N, d.grid.obits));
+  t.gsort_ws = take(radix_sort_workspace_bytes(P, d.grid.hash_bits));
+  if (d.split_items > 0)
+    t.xpart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tile_groups(tiles) + 1)));
+  if (d.grid.blevel >= 0) {
+    t.cocc = reinterpret_cast<uint32_t*>(
+        take(sizeof(uint32_t) * (((size_t)d.grid.cdx * d.grid.cdy * d.grid.cdz + 31) / 32)));
+    if (d.grid.fwords)
+      t.focc = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * focc_words(d.grid)));
+  }
+  t.clear_bytes = off;
   t.rec = reinterpret_cast<float*>(take(sizeof(float) * N * rec_stride(d.channels)));
   t.box = reinterpret_cast<uint4*>(take(sizeof(uint4) * N));
   t.gcount = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
   t.glive = reinterpret_cast<uint8_t*>(take(sizeof(uint8_t) * N));
-  t.gmask = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
+  t.gmask = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * N));
   t.qbox = reinterpret_cast<uint2*>(take(sizeof(uint2) * N));
-  t.goffset = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
   for (int k = 0; k < 2; ++k) {
     t.okey[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
     t.oval[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
@@ -112,6 +131,7 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
     t.qkey[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * M));
     t.qval[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * M));
   }
+  t.qpos = reinterpret_cast<float4*>(take(sizeof(float4) * M));
   t.qstart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ncp));
   t.qrec = reinterpret_cast<float*>(take(sizeof(float) * M * qrec_stride(d.channels)));
   // room for float64 sums (the gradient-check build of the backward)
@@ -122,25 +142,17 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
     t.gkey[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (P > 0 ? P : 1)));
     t.gval[k] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (P > 0 ? P : 1)));
   }
-  t.occ = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ((nb + 31) / 32)));
   t.brange = reinterpret_cast<uint2*>(take(sizeof(uint2) * nb));
   t.dec = d.bf16 ? reinterpret_cast<float*>(take(sizeof(float) * (10 + d.channels) * N)) : nullptr;
   if (d.split_items > 0) {
-    const int64_t tiles = (M + kWarp - 1) / kWarp;
     t.tparts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
-    t.xoff = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.xunit = reinterpret_cast<uint4*>(take(sizeof(uint4) * GPF_MAX_SPLIT_UNITS));
     t.xsum = reinterpret_cast<float*>(
         take(sizeof(float) * (size_t)GPF_MAX_SPLIT_UNITS * (d.channels + 1) * kWarp));
   }
   if (d.grid.blevel >= 0) {
-    const int64_t tiles = (M + kWarp - 1) / kWarp;
-    t.cocc = reinterpret_cast<uint32_t*>(
-        take(sizeof(uint32_t) * (((size_t)d.grid.cdx * d.grid.cdy * d.grid.cdz + 31) / 32)));
-    if (d.grid.fwords)
-      t.focc = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * focc_words(d.grid)));
     t.hparts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
-    t.hoff = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
+    t.hpart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tile_groups(tiles) + 1)));
     t.hitems = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.hunit = reinterpret_cast<uint4*>(take(sizeof(uint4) * GPF_MAX_SPLIT_UNITS));
     t.hsum = reinterpret_cast<float*>(
@@ -155,14 +167,10 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
     t.nbknn = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * std::max<int64_t>(M, 1) *
                                                GPF_MAX_KMIN));
     t.nbrange = reinterpret_cast<uint2*>(take(sizeof(uint2) * std::max<int64_t>(N, 1)));
-    t.nbsort_ws = take(radix_sort_workspace_bytes(d.nb_max));
+    t.nbsort_ws = take(radix_sort_workspace_bytes(d.nb_max, d.grid.id_bits));
     t.nbsorted = radix_sort_passes(d.grid.id_bits) % 2;
   }
-  t.scan_ws = take(scan_workspace_bytes(
-      std::max<int64_t>(std::max<int64_t>(std::max<int64_t>(N, 1), ncp), M + 2)));
-  t.qsort_ws = take(radix_sort_workspace_bytes(M > 0 ? M : 1));
-  t.gsort_ws = take(radix_sort_workspace_bytes(P > 0 ? P : 1));
-  t.osort_ws = take(radix_sort_workspace_bytes(N > 0 ? N : 1));
+  if (d.nb_max > 0) t.scan_ws = take(scan_workspace_bytes(M + 2));
   t.qsorted = radix_sort_passes(d.grid.key_bits) % 2;
   t.osorted = radix_sort_passes(d.grid.obits) % 2;
   t.gsorted = radix_sort_passes(d.grid.hash_bits) % 2;
@@ -741,7 +749,7 @@ gpf_status gpf_sort_pairs_workspace_size(int64_t n, size_t* bytes) {
   if (!bytes) return fail(GPF_ERR_INVALID_ARG, "bytes is NULL");
   if (n < 0 || n >= kMaxSortN)
     return fail(GPF_ERR_INVALID_ARG, "n = %lld outside [0, 2^30)", (long long)n);
-  *bytes = 256 + radix_sort_workspace_bytes(n > 0 ? n : 1);
+  *bytes = 256 + radix_sort_workspace_bytes(n > 0 ? n : 1, 32);
   return GPF_OK;
 }
 
@@ -767,8 +775,8 @@ gpf_status gpf_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, ui
   uint32_t* stalled = static_cast<uint32_t*>(workspace);
   cudaError_t e = cudaMemsetAsync(stalled, 0, sizeof(uint32_t), st);
   if (e == cudaSuccess && n > 0)
-    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, n, nullptr, bits,
-                         static_cast<char*>(workspace) + 256, stalled, st);
+    e = radix_sort_pairs(SortTask{keys, vals, keys_alt, vals_alt, n, nullptr, bits,
+                                  static_cast<char*>(workspace) + 256}, stalled, st);
   if (e != cudaSuccess) return cuda_fail(e, "gpf_sort_pairs");
   *result_in_alt = n > 0 ? radix_sort_passes(bits) % 2 : 0;
   return GPF_OK;

@@ -40,13 +40,14 @@ struct FwdArgs {
   Grid grid;
   const uint32_t* qkey;    // sorted query-level keys of hit points
   const uint32_t* qval;    // sorted hit point ids
+  const float4* qpos;      // sorted positions and ids of the active ones
   const DeviceHeader* header;
-  const float* x;          // [3,M]
   const float* albedo;     // [C,M] or null
   int64_t m;
   const float* rec;
   const uint4* box;
   const uint2* brange;     // [n_buckets] [start, end) of each bucket's list
+  const uint32_t* listed;  // [n_buckets / 32] set: the bucket has a list
   const uint32_t* gval;    // sorted entries (Gaussian ids)
   int64_t n;               // Gaussians (brute force)
   int mode;
@@ -317,9 +318,10 @@ fwd_kernel(FwdArgs a) {
 
   float px = 0.f, py = 0.f, pz = 0.f;
   if (active) {
-    px = a.x[q];
-    py = a.x[a.m + q];
-    pz = a.x[2 * a.m + q];
+    const float4 p = __ldg(a.qpos + k);
+    px = p.x;
+    py = p.y;
+    pz = p.z;
   }
   float L[C];
 #pragma unroll
@@ -364,7 +366,8 @@ fwd_kernel(FwdArgs a) {
     for (int lev = 0; lev < kMaxLevels; ++lev) {
       if (lev < G.levels && ((lmask >> lev) & 1u)) {
         uint2 rg = make_uint2(0u, 0u);
-        if (active) rg = __ldg(a.brange + cell_hash(G, lev, c0x >> lev, c0y >> lev, c0z >> lev).bucket);
+        if (active)
+          rg = bucket_list(a.listed, a.brange, bucket_of(G, lev, c0x >> lev, c0y >> lev, c0z >> lev));
         s_range[wib][lev][lane] = rg;
       }
     }
@@ -636,10 +639,11 @@ __global__ void fwd_split_combine_kernel(FwdArgs a) {
 // staged evaluation of their survivors by the whole warp; else the points'
 // own lists, counted 4 times for the points not sampled. Then the tile's
 // number of parts. Four tiles per warp, eight lanes each.
-__global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header, const float* __restrict__ x,
-                                 const uint32_t* __restrict__ qval, int64_t m,
-                                 const uint2* __restrict__ brange, int split_items,
-                                 uint32_t* __restrict__ tparts, uint32_t* __restrict__ xparts) {
+__global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
+                                 const float4* __restrict__ qpos, int64_t m,
+                                 const uint2* __restrict__ brange,
+                                 const uint32_t* __restrict__ listed, int split_items,
+                                 uint32_t* __restrict__ tparts, uint32_t* __restrict__ xpart) {
   const int lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t tile = gt >> 3;
@@ -652,16 +656,16 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header, const fl
   uint2 rg[kMaxLevels];
   const uint32_t lmask = header->level_mask;
   if (active) {
-    const uint32_t q = qval[k];
-    c0x = coord0(x[q], grid.ox, grid.inv_cell0, grid.max0x);
-    c0y = coord0(x[m + q], grid.oy, grid.inv_cell0, grid.max0y);
-    c0z = coord0(x[2 * m + q], grid.oz, grid.inv_cell0, grid.max0z);
+    const float4 p = __ldg(qpos + k);
+    c0x = coord0(p.x, grid.ox, grid.inv_cell0, grid.max0x);
+    c0y = coord0(p.y, grid.oy, grid.inv_cell0, grid.max0y);
+    c0z = coord0(p.z, grid.oz, grid.inv_cell0, grid.max0z);
   }
 #pragma unroll
   for (int lev = 0; lev < kMaxLevels; ++lev) {
     rg[lev] = make_uint2(0u, 0u);
     if (active && lev < grid.levels && ((lmask >> lev) & 1u))
-      rg[lev] = __ldg(brange + cell_hash(grid, lev, c0x >> lev, c0y >> lev, c0z >> lev).bucket);
+      rg[lev] = bucket_list(listed, brange, bucket_of(grid, lev, c0x >> lev, c0y >> lev, c0z >> lev));
   }
   uint32_t cost = 0;
 #pragma unroll
@@ -688,23 +692,44 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header, const fl
       parts = min((cost + (uint32_t)split_items - 1) / (uint32_t)split_items,
                   (uint32_t)GPF_MAX_TILE_PARTS);
     tparts[tile] = parts;
-    xparts[tile] = parts > 1 ? parts : 0u;
+    if (parts > 1) atomicAdd(&xpart[tile / kTileGroup], parts);
   }
 }
 
-// The split units: tile t's parts at xoff[t] .. xoff[t] + parts - 1 (the
-// exclusive scan of the parts of split tiles); a tile whose units would not
-// all fit under GPF_MAX_SPLIT_UNITS runs unsplit, and its slots below the
-// limit are marked empty.
-__global__ void tile_units_kernel(int64_t n_tiles, uint32_t* __restrict__ tparts,
-                                  const uint32_t* __restrict__ xoff, uint4* __restrict__ xunit,
-                                  uint32_t* n_units) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0) *n_units = min(xoff[n_tiles], (uint32_t)GPF_MAX_SPLIT_UNITS);
-  if (t >= n_tiles) return;
-  const uint32_t parts = tparts[t];
+// The split units: a split tile's parts follow those of the split tiles before
+// it (a block adds up the groups before its own: there is one word per 256
+// tiles, and most of them are zero); a tile whose units would not all fit
+// under GPF_MAX_SPLIT_UNITS runs unsplit, and its slots below the limit are
+// marked empty.
+__global__ void __launch_bounds__(kTileGroup)
+tile_units_kernel(int64_t n_tiles, uint32_t* __restrict__ tparts,
+                  const uint32_t* __restrict__ xpart, uint4* __restrict__ xunit,
+                  uint32_t* n_units) {
+  __shared__ uint32_t s_sum[kTileGroup / kWarp], s_warp[kTileGroup / kWarp];
+  const bool last = blockIdx.x == gridDim.x - 1;
+  if (xpart[blockIdx.x] == 0u && !last) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * kTileGroup + threadIdx.x;
+  uint32_t before = 0;
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kTileGroup) before += xpart[i];
+  before = __reduce_add_sync(kFullMask, before);
+  const uint32_t parts = t < n_tiles ? tparts[t] : 1u;
+  uint32_t incl = parts > 1 ? parts : 0u;
+#pragma unroll
+  for (int o = 1; o < kWarp; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(kFullMask, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 0) s_sum[warp] = before;
+  if (lane == kWarp - 1) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t o = incl - (parts > 1 ? parts : 0u), total = 0;
+  for (int w = 0; w < kTileGroup / kWarp; ++w) {
+    o += s_sum[w] + (w < warp ? s_warp[w] : 0u);
+    total += s_sum[w] + s_warp[w];
+  }
+  if (last && threadIdx.x == 0) *n_units = min(total, (uint32_t)GPF_MAX_SPLIT_UNITS);
   if (parts <= 1) return;
-  const uint32_t o = xoff[t];
   const bool fits = (uint64_t)o + parts <= (uint64_t)GPF_MAX_SPLIT_UNITS;
   if (!fits) tparts[t] = 1;
   for (uint32_t p = 0; p < parts && o + p < (uint32_t)GPF_MAX_SPLIT_UNITS; ++p)
@@ -713,12 +738,10 @@ __global__ void tile_units_kernel(int64_t n_tiles, uint32_t* __restrict__ tparts
 
 }  // namespace
 
-cudaError_t launch_split_units(int64_t n_tiles, uint32_t* tparts, uint32_t* xoff, uint4* xunit,
-                               uint32_t* n_units, void* scan_ws, cudaStream_t stream) {
-  cudaError_t e = exclusive_scan_u32(xoff, xoff, n_tiles + 1, nullptr, scan_ws, stream);
-  if (e != cudaSuccess) return e;
-  tile_units_kernel<<<(unsigned)((n_tiles + 256) / 256), 256, 0, stream>>>(n_tiles, tparts, xoff,
-                                                                           xunit, n_units);
+cudaError_t launch_split_units(int64_t n_tiles, uint32_t* tparts, const uint32_t* xpart,
+                               uint4* xunit, uint32_t* n_units, cudaStream_t stream) {
+  tile_units_kernel<<<(unsigned)tile_groups(n_tiles), kTileGroup, 0, stream>>>(
+      n_tiles, tparts, xpart, xunit, n_units);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -727,10 +750,9 @@ cudaError_t launch_tile_split(const IndexDims& d, const IndexBuffers& b, const g
                               cudaStream_t stream) {
   const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
   tile_cost_kernel<<<(unsigned)((n_tiles * 8 + 255) / 256), 256, 0, stream>>>(
-      d.grid, b.header, q.x, b.qval[b.qsorted], q.m, b.brange, d.split_items, b.tparts, b.xoff);
+      d.grid, b.header, b.qpos, q.m, b.brange, b.listed, d.split_items, b.tparts, b.xpart);
   note_launches(1);
-  return launch_split_units(n_tiles, b.tparts, b.xoff, b.xunit, &b.header->n_xunits, b.scan_ws,
-                            stream);
+  return launch_split_units(n_tiles, b.tparts, b.xpart, b.xunit, &b.header->n_xunits, stream);
 }
 
 cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_queries& q,
@@ -746,13 +768,14 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
   a.grid = d.grid;
   a.qkey = b.qkey[b.qsorted];
   a.qval = b.qval[b.qsorted];
+  a.qpos = b.qpos;
   a.header = b.header;
-  a.x = q.x;
   a.albedo = q.albedo;
   a.m = q.m;
   a.rec = b.rec;
   a.box = b.box;
   a.brange = b.brange;
+  a.listed = b.listed;
   a.gval = b.gval[b.gsorted];
   a.n = n;
   a.mode = p.mode;

@@ -70,12 +70,13 @@ constexpr uint32_t kHybSplitEntries = 512;
 struct HybArgs {
   Grid grid;
   const uint32_t* qval;
+  const float4* qpos;      // sorted positions and ids of the active hit points
   const DeviceHeader* header;
-  const float* x;
   const float* albedo;
   int64_t m;
   const float* rec;
   const uint2* brange;
+  const uint32_t* listed;
   const uint32_t* gval;
   const uint32_t* cocc;    // centre occupancy bits (Grid::cshift cells)
   const uint32_t* focc;    // and per centre cell (Grid::fwords > 0)
@@ -179,8 +180,9 @@ __device__ void lane_ball(const HybArgs& a, float px, float py, float pz, float 
   for (int cz = max(hz - 1, 0); cz <= min(hz + 1, mz); ++cz)
     for (int cy = max(hy - 1, 0); cy <= min(hy + 1, my); ++cy)
       for (int cx = max(hx - 1, 0); cx <= min(hx + 1, mx); ++cx) {
+        if (!centre_cell_occupied(a, cx, cy, cz)) continue;   // no mean: no list
         const CellHash h = cell_hash(G, Lb, cx, cy, cz, kCentreSalt);
-        const uint2 rg = __ldg(a.brange + h.bucket);
+        const uint2 rg = bucket_list(a.listed, a.brange, h.bucket);
         for (uint32_t e = rg.x; e < rg.y; ++e) {
           const uint32_t v = __ldg(a.gval + e);
           if ((v & ~G.id_mask) != h.tag) continue;
@@ -381,7 +383,7 @@ __device__ int warp_knn(const HybArgs& a, bool need, float px, float py, float p
               if (!(d2 > __uint_as_float(tmax)) && occupied) {
                 const CellHash h =
                     cell_hash(G, Lb, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz, kCentreSalt);
-                const uint2 rg = __ldg(a.brange + h.bucket);
+                const uint2 rg = bucket_list(a.listed, a.brange, h.bucket);
                 eb = rg.x;
                 cnt = rg.y - rg.x;
                 tag = h.tag;
@@ -548,8 +550,8 @@ hybrid_fwd_kernel(HybArgs a) {
     const int64_t k = tile * kWarp + lane;
     const bool in_range = k < a.m;
     const bool active = k < n_act;
-    const uint32_t q = in_range ? a.qval[k] : 0u;
     if (MODE == kHybSums && in_range && !active && !partial) {
+      const uint32_t q = a.qval[k];
 #pragma unroll
       for (int c = 0; c < C; ++c) a.out[(int64_t)c * a.m + q] = 0.0f;
       if (a.z) a.z[q] = 0.0f;
@@ -567,10 +569,13 @@ hybrid_fwd_kernel(HybArgs a) {
                                                (C + 1) * kWarp + lane]);
     }
     float px = 0.f, py = 0.f, pz = 0.f;
+    uint32_t q = 0;
     if (active) {
-      px = a.x[q];
-      py = a.x[a.m + q];
-      pz = a.x[2 * a.m + q];
+      const float4 p = __ldg(a.qpos + k);
+      px = p.x;
+      py = p.y;
+      pz = p.z;
+      q = __float_as_uint(p.w);
     }
     float L[C];
 #pragma unroll
@@ -631,7 +636,7 @@ hybrid_fwd_kernel(HybArgs a) {
           // skips the same cells)
           if (centre_cell_occupied(a, ccx, ccy, ccz)) {
             const CellHash h = cell_hash(G, Lb, ccx, ccy, ccz, kCentreSalt);
-            const uint2 rg = __ldg(a.brange + h.bucket);
+            const uint2 rg = bucket_list(a.listed, a.brange, h.bucket);
             eb = rg.x;
             len = rg.y - rg.x;
             tag = h.tag;
@@ -758,7 +763,7 @@ hybrid_fwd_kernel(HybArgs a) {
 // from them its parts (1: whole); one warp per tile.
 template <int C>
 __global__ void __launch_bounds__(kHybThreads)
-hyb_cost_kernel(HybArgs a, uint32_t* __restrict__ hparts, uint32_t* __restrict__ hoff,
+hyb_cost_kernel(HybArgs a, uint32_t* __restrict__ hparts, uint32_t* __restrict__ hpart,
                 uint32_t* __restrict__ hitems) {
   const int lane = threadIdx.x & 31;
   const int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -773,10 +778,10 @@ hyb_cost_kernel(HybArgs a, uint32_t* __restrict__ hparts, uint32_t* __restrict__
     const bool active = k < n_act;
     float px = 0.f, py = 0.f, pz = 0.f;
     if (active) {
-      const uint32_t q = a.qval[k];
-      px = a.x[q];
-      py = a.x[a.m + q];
-      pz = a.x[2 * a.m + q];
+      const float4 p = __ldg(a.qpos + k);
+      px = p.x;
+      py = p.y;
+      pz = p.z;
     }
     float b0 = active ? px : INFINITY, b1 = active ? py : INFINITY, b2 = active ? pz : INFINITY;
     float b3 = active ? px : -INFINITY, b4 = active ? py : -INFINITY, b5 = active ? pz : -INFINITY;
@@ -801,7 +806,8 @@ hyb_cost_kernel(HybArgs a, uint32_t* __restrict__ hparts, uint32_t* __restrict__
       for (uint32_t i = lane; i < (uint32_t)n_cells; i += kWarp) {
         const uint32_t cx = cx0 + i % nx, cy = cy0 + (i / nx) % ny, cz = cz0 + i / (nx * ny);
         if (!centre_cell_occupied(a, cx, cy, cz)) continue;
-        const uint2 rg = __ldg(a.brange + cell_hash(G, Lb, cx, cy, cz, kCentreSalt).bucket);
+        const uint2 rg = bucket_list(a.listed, a.brange,
+                                     cell_hash(G, Lb, cx, cy, cz, kCentreSalt).bucket);
         items += rg.y - rg.x;
       }
       items = __reduce_add_sync(kFullMask, items);
@@ -812,7 +818,7 @@ hyb_cost_kernel(HybArgs a, uint32_t* __restrict__ hparts, uint32_t* __restrict__
     if (items > kHybSplitEntries)
       parts = min((items + kHybSplitEntries - 1) / kHybSplitEntries, (uint32_t)GPF_MAX_TILE_PARTS);
     hparts[tile] = parts;
-    hoff[tile] = parts > 1 ? parts : 0u;
+    if (parts > 1) atomicAdd(&hpart[tile / kTileGroup], parts);
     hitems[tile] = items;
   }
 }
@@ -827,11 +833,12 @@ HybArgs hyb_args(const IndexDims& d, const IndexBuffers& b, const gpf_queries& q
   a.grid = d.grid;
   a.qval = b.qval[b.qsorted];
   a.header = b.header;
-  a.x = q.x;
+  a.qpos = b.qpos;
   a.albedo = q.albedo;
   a.m = q.m;
   a.rec = b.rec;
   a.brange = b.brange;
+  a.listed = b.listed;
   a.gval = b.gval[b.gsorted];
   a.cocc = b.cocc;
   a.focc = b.focc;
@@ -905,10 +912,13 @@ cudaError_t hyb_split_plan(HybArgs& a, const IndexDims& d, const IndexBuffers& b
                            const gpf_queries& q, cudaStream_t stream) {
   const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
   const unsigned blocks = (unsigned)((n_tiles + kHybWarps - 1) / kHybWarps);
+  cudaError_t e =
+      cudaMemsetAsync(b.hpart, 0, sizeof(uint32_t) * (tile_groups(n_tiles) + 1), stream);
+  if (e != cudaSuccess) return e;
   switch (d.channels) {
 #define GPF_HYB_COST(CC)                                                                      \
   case CC:                                                                                    \
-    hyb_cost_kernel<CC><<<blocks, kHybThreads, 0, stream>>>(a, b.hparts, b.hoff, b.hitems); \
+    hyb_cost_kernel<CC><<<blocks, kHybThreads, 0, stream>>>(a, b.hparts, b.hpart, b.hitems); \
     break;
     GPF_HYB_COST(1) GPF_HYB_COST(2) GPF_HYB_COST(3) GPF_HYB_COST(4)
     GPF_HYB_COST(5) GPF_HYB_COST(6) GPF_HYB_COST(7) GPF_HYB_COST(8)
@@ -917,8 +927,7 @@ cudaError_t hyb_split_plan(HybArgs& a, const IndexDims& d, const IndexBuffers& b
       return cudaErrorInvalidValue;
   }
   note_launches(1);
-  cudaError_t e = launch_split_units(n_tiles, b.hparts, b.hoff, b.hunit, &b.header->n_hunits,
-                                     b.scan_ws, stream);
+  e = launch_split_units(n_tiles, b.hparts, b.hpart, b.hunit, &b.header->n_hunits, stream);
   if (e != cudaSuccess) return e;
   a.hparts = b.hparts;
   a.hitems = b.hitems;
@@ -994,9 +1003,9 @@ cudaError_t launch_hybrid_pairs(const IndexDims& d, const IndexBuffers& b, const
   a.phase = kHybSplitFinish;
   if ((e = hyb_pass<kHybEmit>(a, d.channels, psi, stream)) != cudaSuccess) return e;
   // by Gaussian, stable: each Gaussian's hit points stay in increasing order
-  e = radix_sort_pairs(b.nbkey[0], b.nbval[0], b.nbkey[1], b.nbval[1], d.nb_max,
-                       &b.header->nb_pairs, d.grid.id_bits, b.nbsort_ws, &b.header->stalled,
-                       stream);
+  e = radix_sort_pairs(SortTask{b.nbkey[0], b.nbval[0], b.nbkey[1], b.nbval[1], d.nb_max,
+                                &b.header->nb_pairs, d.grid.id_bits, b.nbsort_ws},
+                       &b.header->stalled, stream);
   if (e != cudaSuccess) return e;
   nb_range_kernel<<<(unsigned)((d.nb_max + 255) / 256), 256, 0, stream>>>(
       b.nbkey[b.nbsorted], b.header, d.nb_max, b.nbrange);

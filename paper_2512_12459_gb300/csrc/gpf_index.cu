@@ -11,14 +11,17 @@
 // query-level cell of their mean, the order the backward walks them in.
 //
 // Kernels, in stream order:
-//   query_keys (hit point keys and per-cell counts, occupancy bits of every level)
+//   query_keys (hit point keys, occupancy bits of every level)
 //   preprocess (records, level boxes, entry counts, order keys, level mask)
-//   sort hit points, per-cell starts (scan of the counts)
-//   sort Gaussians into the backward's order
-//   scan of entry counts -> emit (bucket, Gaussian) entries -> sort -> bucket ranges
+//   emit (bucket, Gaussian) entries
+//   sorts, a pass of all three per launch: hit points by cell, Gaussians into
+//   the backward's order, entries by bucket
+//   ranges (per-cell starts of the hit points, bucket ranges of the entries)
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "gpf_internal.h"
 
@@ -29,7 +32,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kBlockWarps = kThreads / kWarp;
 
-// The sum over a block of kThreads threads of up to four per-thread counts,
+// The sum over a block of up to four per-thread counts,
 // each in [0, 2^32); thread 0 gets the sums. The header counters take one
 // atomic per block: atomics to one address are serialised, so per-warp
 // updates from 10^6 threads cost tens of microseconds.
@@ -46,7 +49,7 @@ __device__ __forceinline__ void block_counts(uint32_t (&v)[4], uint32_t (*s)[4])
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       uint32_t t = 0;
-      for (int w = 0; w < kBlockWarps; ++w) t += s[w][k];
+      for (int w = 0; w < (int)blockDim.x / kWarp; ++w) t += s[w][k];
       v[k] = t;
     }
   }
@@ -54,8 +57,67 @@ __device__ __forceinline__ void block_counts(uint32_t (&v)[4], uint32_t (*s)[4])
 // Boxes with more cells than this on their level are refused (overflow flag).
 constexpr int64_t kMaxBoxCells = int64_t(1) << 16;
 constexpr uint32_t kNoBox = 0xffffffffu;
-// gmask of a box of more than 31 cells: emit tests every cell's occupancy bit.
-constexpr uint32_t kMaskAll = 0xffffffffu;
+// Boxes of up to this many cells keep a bit mask of the occupied ones; emit
+// tests the cells of the others again.
+constexpr int64_t kMaskCells = 64;
+
+// Groups of Gaussians whose entry counts add up to one word of gpart, which
+// then holds one word per kSuper groups: the entry offset of a group is the
+// sum of at most kSuper groups and n / (kSuper * group) super-groups.
+constexpr int kSuper = 64;
+// Small fields take groups of 64 (preprocess blocks of 64 threads): 4,096
+// Gaussians are 16 blocks of 256.
+constexpr int64_t kSmallField = 65536;
+inline int group_size(int64_t n) { return n <= kSmallField ? 64 : kThreads; }
+__host__ __device__ __forceinline__ int64_t group_count(int64_t n, int group) {
+  return (n + group - 1) / group;
+}
+
+// Adds the digits of this lane's sort key (if ok) to the block's digit counts
+// cnt[pass * kSortBins + digit]: one atomic per run of lanes with equal digits
+// (hit points of neighbouring pixels share the high digits of their cell keys,
+// and atomics to one address are serialised). All lanes of the warp call it.
+__device__ __forceinline__ void count_digits(uint32_t key, bool ok, int passes, uint32_t* cnt) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t left = __shfl_up_sync(kFullMask, key, 1);
+  const uint32_t valid = __ballot_sync(kFullMask, ok);     // a prefix of the lanes
+  for (int p = 0; p < passes; ++p) {
+    const uint32_t d = (key >> (8 * p)) & 255u;
+    const bool head = ok && (lane == 0 || d != ((left >> (8 * p)) & 255u));
+    const uint32_t heads = __ballot_sync(kFullMask, head);
+    if (head) {
+      const uint32_t later = heads & ~((2u << lane) - 1u);
+      const int end = later ? __ffs(later) - 1 : __popc(valid);
+      atomicAdd(&cnt[p * kSortBins + d], (uint32_t)(end - lane));
+    }
+  }
+}
+__device__ __forceinline__ void flush_digits(const uint32_t* cnt, int passes,
+                                             uint32_t* __restrict__ out) {
+  for (int i = threadIdx.x; i < passes * kSortBins; i += blockDim.x)
+    if (cnt[i]) atomicAdd(&out[i], cnt[i]);
+}
+
+// Position of the j-th (from 0) set bit of m, which has more than j.
+__device__ __forceinline__ uint32_t nth_bit(unsigned long long m, uint32_t j) {
+  uint32_t w = (uint32_t)m, pos = 0;
+  const uint32_t lo = (uint32_t)__popc(w);
+  if (j >= lo) {
+    j -= lo;
+    w = (uint32_t)(m >> 32);
+    pos = 32;
+  }
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    const uint32_t c = (uint32_t)__popc(w & ((1u << h) - 1u));
+    if (j >= c) {
+      j -= c;
+      w >>= h;
+      pos += h;
+    }
+  }
+  return pos;
+}
 
 __device__ __forceinline__ bool occupied(const uint32_t* occ, uint32_t b) {
   return (occ[b >> 5] >> (b & 31u)) & 1u;
@@ -154,13 +216,22 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
                                   float* __restrict__ rec, int rs, uint4* __restrict__ box,
                                   const uint32_t* __restrict__ occ,
                                   uint32_t* __restrict__ gcount, uint8_t* __restrict__ glive,
-                                  uint32_t* __restrict__ gmask, uint2* __restrict__ qbox,
+                                  unsigned long long* __restrict__ gmask,
+                                  uint2* __restrict__ qbox,
                                   uint32_t* __restrict__ okey, uint32_t* __restrict__ oval,
-                                  DeviceHeader* header) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                                  int passes, uint32_t* __restrict__ digit_counts,
+                                  uint32_t* __restrict__ gpart, DeviceHeader* header) {
+  __shared__ uint32_t s_digits[kSortMaxPasses * kSortBins];   // of the order keys
+  for (int i = threadIdx.x; i < passes * kSortBins; i += blockDim.x) s_digits[i] = 0;
+  __syncthreads();
   const int64_t n = f.n;
-  uint32_t level_bit = 0;
+  const int64_t n_groups = group_count(n, (int)blockDim.x);
+  uint32_t level_bits = 0;
+  uint32_t v[4] = {0u, 0u, 0u, 0u};    // live, small, huge, bad of this thread
+  for (int64_t group = blockIdx.x; group < n_groups; group += gridDim.x) {
+  const int64_t g = group * blockDim.x + threadIdx.x;
   bool live = false, small = false, huge = false, bad = false;
+  uint32_t order_key = 0, entries = 0;
   if (g < n) {
     const float* mean = static_cast<const float*>(f.mean);
     const float* spec = static_cast<const float*>(f.spectrum);
@@ -229,10 +300,10 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
       } else {
         box[g] = make_uint4(lx | ((uint32_t)L << 20), ly, lz, sx | (sy << 8) | (sz << 16));
         rv[3] = rec_radius_with_level(rv[3], (uint32_t)L);
-        level_bit = 1u << L;
+        level_bits |= 1u << L;
         // bit c of the mask: the c-th cell of the box (x fastest) holds a
         // hit point; emit walks the set bits only
-        uint32_t mask = 0;
+        unsigned long long mask = 0;
         if (sx <= 2 && sy <= 2 && sz <= 2) {
           // at most 3 x 3 x 3 cells: the nine occupancy reads of a z slice
           // are independent and go out together
@@ -243,7 +314,20 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
               if (dy <= sy && dx <= sx &&
                   occupied(occ, bucket_of(grid, L, lx + dx, ly + dy, lz + dz))) {
                 ++cnt;
-                mask |= 1u << ((dz * (sy + 1) + dy) * (sx + 1) + dx);
+                mask |= 1ull << ((dz * (sy + 1) + dy) * (sx + 1) + dx);
+              }
+            }
+          }
+        } else if (sx <= 3 && sy <= 3 && sz <= 3) {
+          // the same for up to 4 x 4 x 4 cells
+          for (uint32_t dz = 0; dz <= sz; ++dz) {
+#pragma unroll
+            for (uint32_t j = 0; j < 16; ++j) {
+              const uint32_t dy = j / 4, dx = j % 4;
+              if (dy <= sy && dx <= sx &&
+                  occupied(occ, bucket_of(grid, L, lx + dx, ly + dy, lz + dz))) {
+                ++cnt;
+                mask |= 1ull << ((dz * (sy + 1) + dy) * (sx + 1) + dx);
               }
             }
           }
@@ -254,19 +338,21 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
               for (uint32_t ix = lx; ix <= lx + sx; ++ix, ++c)
                 if (occupied(occ, bucket_of(grid, L, ix, iy, iz))) {
                   ++cnt;
-                  if (c < 32) mask |= 1u << c;
+                  if (c < 64) mask |= 1ull << c;
                 }
         }
-        gmask[g] = vol <= 31 ? mask : kMaskAll;
+        gmask[g] = mask;
       }
       live = cnt > 0;
       if (grid.blevel >= 0) ++cnt;      // the centre entry (kept for every Gaussian)
       gcount[g] = cnt;
+      entries = cnt;
       if (!live) cls = 2;
       small = live && cls == 0;
       huge = live && cls == 1 && size_rank <= 1;
     }
-    okey[g] = mkey | (size_rank << size_shift) | (cls << cls_shift);
+    order_key = mkey | (size_rank << size_shift) | (cls << cls_shift);
+    okey[g] = order_key;
     glive[g] = (brute || live) ? 1 : 0;
     float4* r4 = reinterpret_cast<float4*>(rec + g * rs);
 #pragma unroll
@@ -285,13 +371,25 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
     }
     bad = nf != 0u;
   }
+  count_digits(order_key, g < n, passes, s_digits);
+  v[0] += live;
+  v[1] += small;
+  v[2] += huge;
+  v[3] |= bad;
+  if (gpart) {
+    const uint32_t ent = __reduce_add_sync(kFullMask, entries);
+    if ((threadIdx.x & 31) == 0 && ent) {
+      atomicAdd(&gpart[group], ent);
+      atomicAdd(&gpart[n_groups + group / kSuper], ent);
+    }
+  }
+  }  // groups
   __shared__ uint32_t s_cnt[kBlockWarps][4];
   __shared__ uint32_t s_mask;
   if (threadIdx.x == 0) s_mask = 0;
   __syncthreads();
-  const uint32_t m = __reduce_or_sync(kFullMask, level_bit);
+  const uint32_t m = __reduce_or_sync(kFullMask, level_bits);
   if ((threadIdx.x & 31) == 0 && m) atomicOr(&s_mask, m);
-  uint32_t v[4] = {live ? 1u : 0u, small ? 1u : 0u, huge ? 1u : 0u, bad ? 1u : 0u};
   block_counts(v, s_cnt);      // its __syncthreads also orders s_mask
   if (threadIdx.x == 0) {
     // the level bits: only when this block adds one (the mask fills up early)
@@ -301,6 +399,7 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
     if (v[2]) atomicAdd(&header->n_huge, v[2]);
     if (v[3]) atomicExch(&header->nonfinite, 1u);
   }
+  flush_digits(s_digits, passes, digit_counts);
 }
 
 __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
@@ -308,11 +407,17 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
                                   const uint8_t* __restrict__ valid, int64_t m,
                                   uint32_t* __restrict__ key, uint32_t* __restrict__ val,
                                   uint32_t* __restrict__ occ, int mark,
-                                  uint32_t* __restrict__ qcount, DeviceHeader* header) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                                  uint32_t* __restrict__ qbits, int passes,
+                                  uint32_t* __restrict__ digit_counts, DeviceHeader* header) {
+  __shared__ uint32_t s_digits[kSortMaxPasses * kSortBins];   // of the sort keys
+  for (int d = threadIdx.x; d < passes * kSortBins; d += blockDim.x) s_digits[d] = 0;
+  __syncthreads();
+  uint32_t v[4] = {0u, 0u, 0u, 0u};      // active, bad hit points of this thread
+  const int64_t chunks = (m + kThreads - 1) / kThreads;
+  for (int64_t chunk = blockIdx.x; chunk < chunks; chunk += gridDim.x) {
+  const int64_t i = chunk * kThreads + threadIdx.x;
   bool active = false, bad = false;
   uint32_t k = grid.key_inactive;  // sort key
-  uint32_t kc = 0u;                 // query-level cell key
   uint32_t c0[3] = {0u, 0u, 0u};   // level-0 cell of an active hit point
   if (i < m) {
     // hemisphere gate n . w_o > 0: the float32 sum when it is far enough
@@ -339,8 +444,7 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
       const uint32_t cy = coord0(x[m + i], grid.oy, grid.inv_cell0, grid.max0y);
       const uint32_t cz = coord0(x[2 * m + i], grid.oz, grid.inv_cell0, grid.max0z);
       const int K = grid.qlevel;
-      kc = qkey_of(grid, cx >> K, cy >> K, cz >> K);
-      k = kc;
+      k = qkey_of(grid, cx >> K, cy >> K, cz >> K);
       if (grid.qsub > 0) {
         // then the Morton code of the sub-cell on level K - qsub (x in the
         // lowest bit of each triple), so that a run of 32 hit points covers
@@ -350,7 +454,7 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
         for (int b = grid.qsub - 1; b >= 0; --b)
           mort = (mort << 3) | (((cz >> (s + b)) & 1u) << 2) | (((cy >> (s + b)) & 1u) << 1) |
                  ((cx >> (s + b)) & 1u);
-        k = (kc << (3 * grid.qsub)) | mort;
+        k = (k << (3 * grid.qsub)) | mort;
       }
       c0[0] = cx; c0[1] = cy; c0[2] = cz;
     }
@@ -358,68 +462,119 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
     val[i] = (uint32_t)i;
   }
   if (mark) {
-    // occupancy bits of every level: all levels' words are read at once,
-    // then on each level the first lane of every run of lanes in the same
-    // cell (all of a warp's on the coarse ones) sets its bit where it is not
-    // set yet
+    // occupancy bits of every level, by the first lane of every run of lanes
+    // in the same cell (differ: the bits in which a lane's cell differs from
+    // its left neighbour's, so level L differs when differ >> L is not zero).
+    // The levels from the query level up are marked once per query-level cell:
+    // by the lane that finds the cell's own bit unset.
+    const bool lactive = __shfl_up_sync(kFullMask, active ? 1 : 0, 1) != 0;
+    uint32_t differ = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) differ |= c0[a] ^ __shfl_up_sync(kFullMask, c0[a], 1);
+    if ((threadIdx.x & 31) == 0 || !lactive) differ = 0xffffffffu;
+    if (!active) differ = 0;
+    const int K = grid.qlevel;
+    bool first = false;
+    if ((differ >> K) != 0 && K < grid.levels) {
+      const uint32_t kc = qkey_of(grid, c0[0] >> K, c0[1] >> K, c0[2] >> K);
+      const uint32_t bit = 1u << (kc & 31u);
+      first = !(qbits[kc >> 5] & bit) && !(atomicOr(&qbits[kc >> 5], bit) & bit);
+    }
+    // all the levels' words are read before the first bit is set
     uint32_t bkt[kMaxLevels], word[kMaxLevels];
 #pragma unroll
     for (int L = 0; L < kMaxLevels; ++L) {
-      bkt[L] = active && L < grid.levels
-                   ? bucket_of(grid, L, c0[0] >> L, c0[1] >> L, c0[2] >> L)
-                   : 0xffffffffu;
-      word[L] = bkt[L] != 0xffffffffu ? occ[bkt[L] >> 5] : 0xffffffffu;
+      word[L] = 0xffffffffu;
+      if (L < grid.levels && (L < K ? (differ >> L) != 0 : first)) {
+        bkt[L] = bucket_of(grid, L, c0[0] >> L, c0[1] >> L, c0[2] >> L);
+        word[L] = occ[bkt[L] >> 5];
+      }
     }
 #pragma unroll
-    for (int L = 0; L < kMaxLevels; ++L) {
-      if (L >= grid.levels) break;
-      const uint32_t b = bkt[L];
-      // setting a bit twice is harmless: skipping a lane whose left
-      // neighbour has the same cell removes nearly all repeats cheaply
-      const uint32_t left = __shfl_up_sync(kFullMask, b, 1);
-      const uint32_t bit = 1u << (b & 31u);
-      if (b != 0xffffffffu && ((threadIdx.x & 31) == 0 || left != b) && !(word[L] & bit))
-        atomicOr(&occ[b >> 5], bit);
-    }
+    for (int L = 0; L < kMaxLevels; ++L)
+      if (word[L] != 0xffffffffu) {
+        const uint32_t bit = 1u << (bkt[L] & 31u);
+        if (!(word[L] & bit)) atomicOr(&occ[bkt[L] >> 5], bit);
+      }
   }
-  // per-cell counts: one atomic per distinct cell of the warp (neighbouring
-  // pixels share query cells)
-  const uint32_t peers = __match_any_sync(kFullMask, active ? kc : 0xffffffffu);
-  if (active && (peers & lanemask_lt()) == 0) atomicAdd(&qcount[kc], (uint32_t)__popc(peers));
+  count_digits(k, i < m, passes, s_digits);
+  v[0] += active;
+  v[1] |= bad;
+  }  // chunks
   __shared__ uint32_t s_cnt[kBlockWarps][4];
-  uint32_t v[4] = {active ? 1u : 0u, bad ? 1u : 0u, 0u, 0u};
-  block_counts(v, s_cnt);
+  block_counts(v, s_cnt);     // its __syncthreads also orders s_digits
+  flush_digits(s_digits, passes, digit_counts);
   if (threadIdx.x == 0 && v[0]) atomicAdd(&header->n_active, v[0]);
   if (threadIdx.x == 0 && v[1]) atomicExch(&header->nonfinite, 1u);
 }
 
 // One (bucket, Gaussian) entry per occupied cell of every Gaussian's level
-// box, in the box's cell order, at the Gaussian's offset (the exclusive scan
-// of the counts). A Gaussian whose cells share a bucket appears there on
-// consecutive entries; the pair loops take only the first.
-__global__ void emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec,
-                            int rs, const uint4* __restrict__ box,
-                            const uint32_t* __restrict__ occ, const uint32_t* __restrict__ gmask,
-                            const uint32_t* __restrict__ goffset,
-                            uint32_t* __restrict__ gkey, uint32_t* __restrict__ gval,
-                            int passes, uint32_t* __restrict__ digit_counts,
-                            uint32_t* __restrict__ cocc, uint32_t* __restrict__ focc,
-                            DeviceHeader* header) {
+// box, in the box's cell order, at the Gaussian's offset (the entries of the
+// Gaussians before it). A Gaussian whose cells share a bucket appears there on
+// consecutive entries; the pair loops take only the first. A block takes one
+// group of preprocess and adds up the counts before it; a warp lays the
+// entries of its 32 Gaussians end to end and writes 32 at a time, so that the
+// stores are coalesced and no lane waits for the Gaussian with the most cells
+// (a thread per Gaussian: 53 us and scattered 4-byte stores at 3.8 M entries).
+__global__ void __launch_bounds__(kThreads)
+emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec, int rs,
+            const uint4* __restrict__ box, const uint32_t* __restrict__ occ,
+            const unsigned long long* __restrict__ gmask, const uint32_t* __restrict__ gcount,
+            const uint32_t* __restrict__ gpart, uint32_t* __restrict__ gkey,
+            uint32_t* __restrict__ gval, int passes, uint32_t* __restrict__ digit_counts,
+            uint32_t* __restrict__ cocc, uint32_t* __restrict__ focc, DeviceHeader* header) {
   // the digit counts of the entry sort, added here as the keys are written
   __shared__ uint32_t cnt[kSortMaxPasses * kSortBins];
+  __shared__ uint32_t s_warp[2][kBlockWarps], s_before[2][kBlockWarps];
   for (int i = threadIdx.x; i < passes * kSortBins; i += blockDim.x) cnt[i] = 0;
   __syncthreads();
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g == 0 && (int64_t)header->n_pairs > p_max) atomicExch(&header->overflow, 1u);
-  auto put = [&](int64_t pos, uint32_t bucket, uint32_t v) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t n_groups = group_count(n, (int)blockDim.x);
+  int odd = 0;           // the shared sums alternate: one barrier per group
+  for (int64_t group = blockIdx.x; group < n_groups; group += gridDim.x, odd ^= 1) {
+  const int64_t g = group * blockDim.x + threadIdx.x;
+  // the entries of the groups before this one
+  {
+    const uint32_t sup = (uint32_t)(group / kSuper);
+    uint32_t before = 0;
+    for (uint32_t i = threadIdx.x; i < sup; i += blockDim.x) before += gpart[n_groups + i];
+    for (uint32_t i = sup * kSuper + threadIdx.x; i < (uint32_t)group; i += blockDim.x)
+      before += gpart[i];
+    before = __reduce_add_sync(kFullMask, before);
+    if (lane == 0) s_before[odd][warp] = before;
+  }
+  const uint32_t c = g < n ? gcount[g] : 0u;
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < kWarp; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == kWarp - 1) s_warp[odd][warp] = incl;
+  __syncthreads();
+  uint32_t warp_base = 0, total_here = 0;
+  for (int w = 0; w < (int)blockDim.x / kWarp; ++w) {
+    total_here += s_before[odd][w] + s_warp[odd][w];
+    warp_base += s_before[odd][w] + (w < warp ? s_warp[odd][w] : 0u);
+  }
+  const uint32_t off = warp_base + incl - c;             // this Gaussian's offset
+  if (group == n_groups - 1 && threadIdx.x == 0) {
+    const uint32_t total = total_here;
+    header->n_pairs = total;
+    if ((int64_t)total > p_max) atomicExch(&header->overflow, 1u);
+  }
+  auto put = [&](int64_t pos, const CellHash& h, uint32_t id) {
     if (pos >= p_max) return;
-    gkey[pos] = bucket;
-    gval[pos] = v;
-    for (int p = 0; p < passes; ++p) atomicAdd(&cnt[p * kSortBins + ((bucket >> (8 * p)) & 255u)], 1u);
+    gkey[pos] = h.bucket;
+    gval[pos] = id | h.tag;
+    for (int p = 0; p < passes; ++p)
+      atomicAdd(&cnt[p * kSortBins + ((h.bucket >> (8 * p)) & 255u)], 1u);
   };
+  uint4 bw = make_uint4(kNoBox, 0u, 0u, 0u);
+  unsigned long long mask = 0;
+  uint32_t centre = 0;
   if (g < n) {
-    const uint4 bw = box[g];
-    int64_t pos = goffset[g];
+    bw = box[g];
     if (grid.blevel >= 0) {
       // the centre entry: the cell of the mean on the centre level
       const float* r = rec + g * rs;
@@ -427,68 +582,210 @@ __global__ void emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __
       const uint32_t cx = coord0(r[0], grid.ox, grid.inv_cell0, grid.max0x) >> Lb;
       const uint32_t cy = coord0(r[1], grid.oy, grid.inv_cell0, grid.max0y) >> Lb;
       const uint32_t cz = coord0(r[2], grid.oz, grid.inv_cell0, grid.max0z) >> Lb;
-      const CellHash h = cell_hash(grid, Lb, cx, cy, cz, kCentreSalt);
-      put(pos, h.bucket, (uint32_t)g | h.tag);
+      put(off, cell_hash(grid, Lb, cx, cy, cz, kCentreSalt), (uint32_t)g);
       const uint32_t bit = cocc_bit(grid, cx, cy, cz);
       atomicOr(cocc + (bit >> 5), 1u << (bit & 31u));
       if (grid.fwords) atomicOr(focc + focc_word(grid, cx, cy, cz), 1u << (cx & 31u));
-      ++pos;
+      centre = 1;
     }
-    if (bw.x != kNoBox) {
-      const LevelBox b = unpack_box(bw);
-      uint32_t mask = gmask[g];
-      if (mask != kMaskAll) {
-        // the set bits only, in increasing cell order (x fastest): cell c of
-        // the box is (c mod nx, (c / nx) mod ny, c / (nx ny)); c < 31, so the
-        // quotients computed as floor((c + 0.5) / d) in float32 are exact
-        const uint32_t nx = b.hx - b.lx + 1, nxy = nx * (b.hy - b.ly + 1);
-        const float inx = 1.0f / (float)nx, inxy = 1.0f / (float)nxy;
-        while (mask) {
-          const uint32_t c = (uint32_t)__ffs(mask) - 1u;
-          mask &= mask - 1u;
-          const uint32_t dz = (uint32_t)(((float)c + 0.5f) * inxy);
-          const uint32_t r = c - dz * nxy;
-          const uint32_t dy = (uint32_t)(((float)r + 0.5f) * inx);
-          const uint32_t dx = r - dy * nx;
-          const CellHash h = cell_hash(grid, b.level, b.lx + dx, b.ly + dy, b.lz + dz);
-          put(pos, h.bucket, (uint32_t)g | h.tag);
-          ++pos;
-        }
-      } else {
-        for (uint32_t iz = b.lz; iz <= b.hz; ++iz)
-          for (uint32_t iy = b.ly; iy <= b.hy; ++iy)
-            for (uint32_t ix = b.lx; ix <= b.hx; ++ix) {
-              const CellHash h = cell_hash(grid, b.level, ix, iy, iz);
-              if (!occupied(occ, h.bucket)) continue;
-              put(pos, h.bucket, (uint32_t)g | h.tag);
-              ++pos;
-            }
+  }
+  const bool boxed = bw.x != kNoBox;
+  const uint32_t nx = (bw.w & 0xffu) + 1, ny = ((bw.w >> 8) & 0xffu) + 1,
+                 nz = ((bw.w >> 16) & 0xffu) + 1;
+  const bool masked = boxed && nx * ny * nz <= (uint32_t)kMaskCells;
+  if (masked) mask = gmask[g];
+  // the masked boxes of the warp, their set cells end to end: item f belongs
+  // to the first lane whose inclusive count exceeds f; cell i of a box is
+  // (i mod nx, (i / nx) mod ny, i / (nx ny)); i < 64, so the quotients
+  // computed as floor((i + 0.5) / d) in float32 are exact
+  const uint32_t my = masked ? c - centre : 0u;
+  uint32_t mi = my;
+#pragma unroll
+  for (int o = 1; o < kWarp; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(kFullMask, mi, o);
+    if (lane >= o) mi += t;
+  }
+  const uint32_t total = __shfl_sync(kFullMask, mi, kWarp - 1);
+  for (uint32_t f0 = 0; f0 < total; f0 += kWarp) {
+    const uint32_t f = f0 + lane;
+    int o = 0;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1)
+      if (__shfl_sync(kFullMask, mi, o + st - 1) <= f) o += st;
+    const uint32_t j = f - __shfl_sync(kFullMask, mi - my, o);
+    const unsigned long long om = __shfl_sync(kFullMask, mask, o);
+    const uint32_t x = __shfl_sync(kFullMask, bw.x, o), ly = __shfl_sync(kFullMask, bw.y, o),
+                   lz = __shfl_sync(kFullMask, bw.z, o), w = __shfl_sync(kFullMask, bw.w, o);
+    const uint32_t pos = __shfl_sync(kFullMask, off + centre, o) + j;
+    if (f < total) {
+      const uint32_t i = nth_bit(om, j);
+      const uint32_t onx = (w & 0xffu) + 1, onxy = onx * (((w >> 8) & 0xffu) + 1);
+      const uint32_t dz = (uint32_t)(((float)i + 0.5f) * (1.0f / (float)onxy));
+      const uint32_t r = i - dz * onxy;
+      const uint32_t dy = (uint32_t)(((float)r + 0.5f) * (1.0f / (float)onx));
+      put(pos, cell_hash(grid, (int)(x >> 20), (x & kCoordMax) + r - dy * onx, ly + dy, lz + dz),
+          (uint32_t)(g - lane) + (uint32_t)o);
+    }
+  }
+  // the larger boxes one at a time, 32 cells at a time
+  for (uint32_t todo = __ballot_sync(kFullMask, boxed && !masked); todo; todo &= todo - 1u) {
+    const int o = __ffs(todo) - 1;
+    const uint32_t x = __shfl_sync(kFullMask, bw.x, o), ly = __shfl_sync(kFullMask, bw.y, o),
+                   lz = __shfl_sync(kFullMask, bw.z, o);
+    const uint32_t bx = __shfl_sync(kFullMask, nx, o), by = __shfl_sync(kFullMask, ny, o),
+                   bz = __shfl_sync(kFullMask, nz, o);
+    const uint32_t cells = bx * by * bz;                 // at most kMaxBoxCells
+    uint32_t pos = __shfl_sync(kFullMask, off + centre, o);
+    for (uint32_t i0 = 0; i0 < cells; i0 += kWarp) {
+      const uint32_t i = i0 + lane;
+      CellHash h{};
+      bool set = false;
+      if (i < cells) {
+        h = cell_hash(grid, (int)(x >> 20), (x & kCoordMax) + i % bx, ly + i / bx % by,
+                      lz + i / (bx * by));
+        set = occupied(occ, h.bucket);
+      }
+      const uint32_t sm = __ballot_sync(kFullMask, set);
+      if (set)
+        put((int64_t)pos + __popc(sm & lanemask_lt()), h, (uint32_t)(g - lane) + (uint32_t)o);
+      pos += (uint32_t)__popc(sm);
+    }
+  }
+  }  // groups
+  __syncthreads();
+  flush_digits(cnt, passes, digit_counts);
+}
+
+// qstart[c] for every query-level cell c < n_out: the number of active hit
+// points in cells before c, found in their sorted keys. A warp takes
+// kStartCells consecutive cells: it finds the first point of its first cell
+// and of the cell after its last by a 32-way search (4-5 probes of 10^6
+// points), fills them with one value when no point lies between - nearly every
+// run: hit points lie on surfaces, 10^5 of the 2 * 10^7 cells of a 1M-Gaussian
+// scene hold one - and else searches that interval once per cell, 16 cells per
+// lane at a time. Bound by the 4 B per cell it writes. Counting the points per
+// cell with atomics and scanning the counts read and wrote every cell three
+// times and cleared it once (22 M cells: 160 us and a 89 MB memset).
+constexpr uint32_t kStartCells = 512;
+__device__ __forceinline__ void cell_starts(uint32_t block, const uint32_t* __restrict__ skey,
+                                            int shift, const DeviceHeader* header,
+                                            uint32_t n_out, uint32_t* __restrict__ qstart) {
+  constexpr int kPer = kStartCells / kWarp;
+  const int lane = threadIdx.x & 31;
+  const uint32_t w = (block * (uint32_t)kThreads + threadIdx.x) / kWarp;
+  if (w > (n_out - 1) / kStartCells) return;
+  const uint32_t c0 = w * kStartCells;
+  const uint32_t n = header->n_active;
+  // first positions of cells c0 and c0 + kStartCells (both searches at once)
+  const uint32_t target[2] = {c0, c0 + kStartCells};
+  uint32_t a[2] = {0u, 0u}, b[2] = {n, n};       // the answer lies in [a, b]
+  while (a[0] < b[0] || a[1] < b[1]) {
+    bool below[2];
+    uint32_t step[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      step[k] = (b[k] - a[k] + kWarp - 1) / kWarp;
+      const uint32_t p = a[k] + (lane + 1) * step[k] - 1;
+      below[k] = a[k] < b[k] && p < b[k] && (__ldg(skey + p) >> shift) < target[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t cnt = (uint32_t)__popc(__ballot_sync(kFullMask, below[k]));
+      if (a[k] < b[k]) {
+        const uint32_t na = min(a[k] + cnt * step[k], b[k]);
+        b[k] = min(b[k], a[k] + (cnt + 1) * step[k] - 1);
+        a[k] = na;
       }
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < passes * kSortBins; i += blockDim.x)
-    if (cnt[i]) atomicAdd(&digit_counts[i], cnt[i]);
+  uint32_t at[kPer];
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) at[j] = a[0];
+  // (keys of a sort that gave up may be out of order: every read stays below n)
+  if (a[1] > a[0]) {
+    uint32_t len = a[1] - a[0];
+    while (len > 0) {
+      const uint32_t half = (len + 1) >> 1;
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        const uint32_t c = c0 + (uint32_t)(j / 4) * (4 * kWarp) + 4 * lane + (j & 3);
+        if ((__ldg(skey + at[j] + half - 1) >> shift) < c) at[j] += half;
+      }
+      len -= half;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kPer; j += 4) {
+    const uint32_t c = c0 + (uint32_t)(j / 4) * (4 * kWarp) + 4 * lane;
+    if (c + 3 < n_out) {
+      *reinterpret_cast<uint4*>(qstart + c) = make_uint4(at[j], at[j + 1], at[j + 2], at[j + 3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (c + i < n_out) qstart[c + i] = at[j + i];
+    }
+  }
 }
 
 // [start, end) of every non-empty bucket from the boundaries of the sorted
-// keys (the other buckets keep the [0, 0) of the memset).
-__global__ void bucket_range_kernel(const uint32_t* __restrict__ keys, const DeviceHeader* header,
-                                    int64_t n_cap, uint2* __restrict__ range) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// keys, and its bit in listed: a lookup reads the table only where the bit is
+// set, so the table (134 MB at 2^24 buckets) is never cleared and the many
+// empty lookups stay in the 2 MB of bits.
+__device__ __forceinline__ void bucket_ranges(uint32_t block, const uint32_t* __restrict__ keys,
+                                              const DeviceHeader* header, int64_t n_cap,
+                                              uint2* __restrict__ range,
+                                              uint32_t* __restrict__ listed) {
+  const int64_t i = (int64_t)block * kThreads + threadIdx.x;
   if (header->stalled) return;
   int64_t n = header->n_pairs;
   if (n > n_cap) n = n_cap;
   if (i >= n) return;
   const uint32_t k = keys[i];
-  if (i == 0 || keys[i - 1] != k) range[k].x = (uint32_t)i;
+  if (i == 0 || keys[i - 1] != k) {
+    range[k].x = (uint32_t)i;
+    atomicOr(&listed[k >> 5], 1u << (k & 31u));
+  }
   if (i == n - 1 || keys[i + 1] != k) range[k].y = (uint32_t)(i + 1);
+}
+
+// The active hit points' positions and ids in sorted order: the pair loops, the
+// tile costs and the backward's packing read them in turn instead of gathering
+// three floats per point by id each time.
+__device__ __forceinline__ void sorted_positions(uint32_t block, const float* __restrict__ x,
+                                                 const uint32_t* __restrict__ qval, int64_t m,
+                                                 const DeviceHeader* header,
+                                                 float4* __restrict__ qpos) {
+  const int64_t k = (int64_t)block * kThreads + threadIdx.x;
+  if (k >= (int64_t)header->n_active || header->stalled) return;
+  const uint32_t q = qval[k];
+  qpos[k] = make_float4(x[q], x[m + q], x[2 * m + q], __uint_as_float(q));
+}
+
+// After the sorts, in one launch: the query-level cells' starts (the first
+// start_blocks blocks), the hit points' positions (the next pos_blocks) and the
+// buckets' ranges (the others).
+__global__ void __launch_bounds__(kThreads)
+ranges_kernel(uint32_t start_blocks, const uint32_t* __restrict__ skey, int shift,
+              uint32_t n_out, uint32_t* __restrict__ qstart, uint32_t pos_blocks,
+              const float* __restrict__ x, const uint32_t* __restrict__ qval, int64_t m,
+              float4* __restrict__ qpos, const uint32_t* __restrict__ keys, int64_t n_cap,
+              uint2* __restrict__ range, uint32_t* __restrict__ listed,
+              const DeviceHeader* header) {
+  const uint32_t b = blockIdx.x;
+  if (b < start_blocks) cell_starts(b, skey, shift, header, n_out, qstart);
+  else if (b < start_blocks + pos_blocks)
+    sorted_positions(b - start_blocks, x, qval, m, header, qpos);
+  else bucket_ranges(b - start_blocks - pos_blocks, keys, header, n_cap, range, listed);
 }
 
 __global__ void index_flags_kernel(const DeviceHeader* header, uint32_t* flags) {
   *flags = index_flags(header);
 }
 
+// Blocks of the kernels that add digit counts: at the end each block adds up to
+// 256 counts per sort pass to the same words, which serialise, so a few blocks
+// per SM take several groups each rather than every group its own block.
+inline unsigned shared_blocks(unsigned groups) { return std::min(groups, 152u * 8u); }
 inline unsigned blocks_for(int64_t n, int t = kThreads) {
   return (unsigned)((n + t - 1) / t);
 }
@@ -509,10 +806,19 @@ gpf_field float32_view(const IndexDims& d, const IndexBuffers& b, const gpf_fiel
   return v;
 }
 
+size_t gpart_words(int64_t n) {
+  // (a group size for every n up to the capacity: the small one gives the most)
+  const int64_t groups = std::max(group_count(std::min(n, kSmallField), 64),
+                                  group_count(n, kThreads)) + 1;
+  return (size_t)(groups + groups / kSuper + 1);
+}
+
 cudaError_t launch_build(const IndexDims& d, const IndexBuffers& b, const gpf_field& f_in,
                          const gpf_queries& q, cudaStream_t stream) {
   const Grid& grid = d.grid;
-  cudaError_t e = cudaMemsetAsync(b.header, 0, sizeof(DeviceHeader), stream);
+  // everything that starts from zero lies in one range: the header, the
+  // occupancy bits, the sorts' counts and status words, the entry sums
+  cudaError_t e = cudaMemsetAsync(b.header, 0, b.clear_bytes, stream);
   if (e != cudaSuccess) return e;
   // 0. 16-bit storage: decode every parameter to float32 once
   if (f_in.storage != GPF_F32 && f_in.n > 0) {
@@ -520,69 +826,56 @@ cudaError_t launch_build(const IndexDims& d, const IndexBuffers& b, const gpf_fi
     note_launches(1);
   }
   const gpf_field f = float32_view(d, b, f_in);
-  if (!d.brute) {
-    e = cudaMemsetAsync(b.occ, 0, sizeof(uint32_t) * ((grid.n_buckets + 31) / 32), stream);
-    if (e != cudaSuccess) return e;
-  }
-  // hit points per query-level cell, counted by the key pass
-  e = cudaMemsetAsync(b.qstart, 0, sizeof(uint32_t) * ((size_t)grid.n_keys + 2), stream);
-  if (e != cudaSuccess) return e;
+  const SortTask sort_q{b.qkey[0], b.qval[0], b.qkey[1], b.qval[1], q.m, nullptr, grid.key_bits,
+                        b.qsort_ws};
+  const SortTask sort_o{b.okey[0], b.oval[0], b.okey[1], b.oval[1], f.n, nullptr, grid.obits,
+                        b.osort_ws};
+  const SortTask sort_g{b.gkey[0], b.gval[0], b.gkey[1], b.gval[1], d.p_max, &b.header->n_pairs,
+                        grid.hash_bits, b.gsort_ws};
+  const bool lists = !d.brute && f.n > 0;
   // 1. hit point keys and occupancy bits of every level
   if (q.m > 0) {
-    query_keys_kernel<<<blocks_for(q.m), kThreads, 0, stream>>>(
+    query_keys_kernel<<<shared_blocks(blocks_for(q.m)), kThreads, 0, stream>>>(
         grid, q.x, q.normal, q.wo, q.valid, q.m, b.qkey[0], b.qval[0], b.occ, d.brute ? 0 : 1,
-        b.qstart, b.header);
+        b.qbits, radix_sort_passes(grid.key_bits), radix_sort_counts(b.qsort_ws), b.header);
     note_launches(1);
   }
-  // 2. Gaussian records, level boxes, entry counts, order keys, level mask
+  // 2. Gaussian records, level boxes, entry counts, order keys, level mask;
+  // 3. (bucket, Gaussian) entries
   if (f.n > 0) {
-    preprocess_kernel<<<blocks_for(f.n), kThreads, 0, stream>>>(
+    const int group = group_size(f.n);
+    const unsigned blocks = shared_blocks(blocks_for(f.n, group));
+    preprocess_kernel<<<blocks, group, 0, stream>>>(
         f, grid, d.cutoff, d.brute ? 1 : 0, b.rec, rec_stride(d.channels), b.box, b.occ,
-        b.gcount, b.glive, b.gmask, b.qbox, b.okey[0], b.oval[0], b.header);
+        b.gcount, b.glive, b.gmask, b.qbox, b.okey[0], b.oval[0], radix_sort_passes(grid.obits),
+        radix_sort_counts(b.osort_ws), lists ? b.gpart : nullptr, b.header);
+    note_launches(1);
+    if (lists) {
+      emit_kernel<<<blocks, group, 0, stream>>>(
+          grid, f.n, d.p_max, b.rec, rec_stride(d.channels), b.box, b.occ, b.gmask, b.gcount,
+          b.gpart, b.gkey[0], b.gval[0], radix_sort_passes(grid.hash_bits),
+          radix_sort_counts(b.gsort_ws), b.cocc, b.focc, b.header);
+      note_launches(1);
+    }
+  }
+  // 4. side by side: hit points by query-level cell (inactive ones last),
+  // Gaussians in the backward's order, entries by bucket
+  const SortTask sorts[3] = {sort_q, sort_o, sort_g};
+  e = radix_sort_counted(sorts, lists ? 3 : 2, &b.header->stalled, stream);
+  if (e != cudaSuccess) return e;
+  // 5. the cells' starts, the hit points' positions and the bucket ranges
+  {
+    const uint32_t n_out = grid.n_keys + 2;
+    const unsigned starts =
+        blocks_for(((int64_t)n_out + kStartCells - 1) / kStartCells * kWarp);
+    const unsigned ranges = lists ? blocks_for(d.p_max) : 0u;
+    const unsigned pos = blocks_for(q.m);
+    ranges_kernel<<<starts + pos + ranges, kThreads, 0, stream>>>(
+        starts, b.qkey[b.qsorted], 3 * grid.qsub, n_out, b.qstart, pos, q.x, b.qval[b.qsorted],
+        q.m, b.qpos, b.gkey[b.gsorted], d.p_max, b.brange, b.listed, b.header);
     note_launches(1);
   }
-  // 3. hit points sorted by query-level cell (inactive ones last), cell starts
-  e = radix_sort_pairs(b.qkey[0], b.qval[0], b.qkey[1], b.qval[1], q.m, nullptr, grid.key_bits,
-                       b.qsort_ws, &b.header->stalled, stream);
-  if (e != cudaSuccess) return e;
-  e = exclusive_scan_u32(b.qstart, b.qstart, (int64_t)grid.n_keys + 2, nullptr, b.scan_ws,
-                         stream);
-  if (e != cudaSuccess) return e;
-  // 4. Gaussians in the backward's order
-  e = radix_sort_pairs(b.okey[0], b.oval[0], b.okey[1], b.oval[1], f.n, nullptr, grid.obits,
-                       b.osort_ws, &b.header->stalled, stream);
-  if (e != cudaSuccess) return e;
-  if (d.brute || f.n == 0) return cudaGetLastError();
-  // 5. (bucket, Gaussian) entries: scan, emit, sort, bucket starts
-  e = exclusive_scan_u32(b.gcount, b.goffset, f.n, &b.header->n_pairs, b.scan_ws, stream);
-  if (e != cudaSuccess) return e;
-  e = radix_sort_clear_counts(b.gsort_ws, stream);
-  if (e != cudaSuccess) return e;
-  if (grid.blevel >= 0) {
-    e = cudaMemsetAsync(
-        b.cocc, 0, sizeof(uint32_t) * (((size_t)grid.cdx * grid.cdy * grid.cdz + 31) / 32), stream);
-    if (e != cudaSuccess) return e;
-    if (grid.fwords && (e = cudaMemsetAsync(b.focc, 0, sizeof(uint32_t) * focc_words(grid),
-                                            stream)) != cudaSuccess)
-      return e;
-  }
-  emit_kernel<<<blocks_for(f.n), kThreads, 0, stream>>>(
-      grid, f.n, d.p_max, b.rec, rec_stride(d.channels), b.box, b.occ, b.gmask, b.goffset,
-      b.gkey[0], b.gval[0], radix_sort_passes(grid.hash_bits), radix_sort_counts(b.gsort_ws),
-      b.cocc, b.focc, b.header);
-  note_launches(1);
-  e = radix_sort_pairs(b.gkey[0], b.gval[0], b.gkey[1], b.gval[1], d.p_max, &b.header->n_pairs,
-                       grid.hash_bits, b.gsort_ws, &b.header->stalled, stream, true);
-  if (e != cudaSuccess) return e;
-  // bucket ranges from the boundaries of the sorted keys
-  e = cudaMemsetAsync(b.brange, 0, sizeof(uint2) * (size_t)grid.n_buckets, stream);
-  if (e != cudaSuccess) return e;
-  if (d.p_max > 0) {
-    bucket_range_kernel<<<blocks_for(d.p_max), kThreads, 0, stream>>>(
-        b.gkey[b.gsorted], b.header, d.p_max, b.brange);
-    note_launches(1);
-  }
-  if (d.split_items > 0 && q.m > 0) {
+  if (lists && d.split_items > 0 && q.m > 0) {
     e = launch_tile_split(d, b, q, stream);
     if (e != cudaSuccess) return e;
   }

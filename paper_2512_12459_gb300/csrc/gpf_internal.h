@@ -31,23 +31,30 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uin
                                void* ws, cudaStream_t stream);
 // The sort's element count limit: status words hold 30-bit counts.
 constexpr int64_t kMaxSortN = int64_t(1) << 30;
-int64_t radix_tiles(int64_t n_max);
-size_t radix_sort_workspace_bytes(int64_t n_max);
-int radix_sort_passes(int bits);
-// Stable sort of min(*d_n, n_max) pairs (n_max pairs when d_n is null) by
-// key bits [0, bits). The result is in (k0, v0) after an even number of
-// passes, in (k1, v1) after an odd one. *stalled (device) is set to 1 if a
-// bounded wait of the single-pass sort gave up (the output is then invalid).
-// counted: the kernel that wrote the keys has already added their digit
-// counts, digit d of pass p at radix_sort_counts(ws)[p * kSortBins + d],
-// into counts that radix_sort_clear_counts zeroed before it ran.
 constexpr int kSortBins = 256;
 constexpr int kSortMaxPasses = 4;
-cudaError_t radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                             int64_t n_max, const uint32_t* d_n, int bits, void* ws,
-                             uint32_t* stalled, cudaStream_t stream, bool counted = false);
+constexpr int kSortMaxJobs = 3;
+// A stable sort of min(*d_n, n_max) pairs (n_max pairs when d_n is null) by
+// key bits [0, bits). The result is in (k0, v0) after an even number of
+// passes, in (k1, v1) after an odd one. ws: radix_sort_workspace_bytes.
+struct SortTask {
+  uint32_t *k0, *v0, *k1, *v1;
+  int64_t n_max;
+  const uint32_t* d_n;
+  int bits;
+  void* ws;
+};
+size_t radix_sort_workspace_bytes(int64_t n_max, int bits);
+int radix_sort_passes(int bits);
+// *stalled (device) is set to 1 if a bounded wait of the single-pass sort
+// gave up (the output is then invalid).
+cudaError_t radix_sort_pairs(const SortTask& t, uint32_t* stalled, cudaStream_t stream);
+// Up to kSortMaxJobs sorts side by side, a pass of each per launch. Their
+// workspaces were zeroed, and the kernels that wrote the keys have added the
+// digit counts: digit d of pass p at radix_sort_counts(ws)[p * kSortBins + d].
+cudaError_t radix_sort_counted(const SortTask* tasks, int count, uint32_t* stalled,
+                               cudaStream_t stream);
 uint32_t* radix_sort_counts(void* ws);
-cudaError_t radix_sort_clear_counts(void* ws, cudaStream_t stream);
 // The failure-detection probe of the single-pass sort's bounded wait (a
 // look-back whose predecessor tile is never processed): buffer size, launch.
 size_t sort_wait_probe_bytes();
@@ -60,10 +67,10 @@ struct IndexBuffers {
   float* rec;           // [N_max * rec_stride] Gaussian records
   uint4* box;           // [N_max] level boxes
   uint32_t* gcount;     // [N_max] entries per Gaussian
+  uint32_t* gpart;      // entries per group of Gaussians, then per kSuper groups
   uint8_t* glive;       // [N_max] 1 if the backward visits the Gaussian (a hit point in reach)
-  uint32_t* gmask;      // [N_max] occupied cells of the level box (boxes of <= 31 cells)
+  unsigned long long* gmask;  // [N_max] occupied cells of the level box (boxes of <= 64 cells)
   uint2* qbox;          // [N_max] query-level cell bounds of each Gaussian (pack_qbox)
-  uint32_t* goffset;    // [N_max] exclusive scan of gcount
   uint32_t* okey[2];    // [N_max] query-level key of each mean (sort ping-pong)
   uint32_t* oval[2];    // [N_max] Gaussian ids in that order
   uint32_t* qkey[2];    // [M_max] sort ping-pong of hit points
@@ -77,7 +84,10 @@ struct IndexBuffers {
   uint32_t* occ;        // [n_buckets / 32] occupancy bits of (level, cell) buckets
   uint32_t* gkey[2];    // [P_max] (bucket, Gaussian) entries, sort ping-pong
   uint32_t* gval[2];
-  uint2* brange;        // [n_buckets] [start, end) of every bucket's list
+  uint2* brange;        // [n_buckets] [start, end) of every bucket's list (listed ones)
+  uint32_t* listed;     // [n_buckets / 32] set: the bucket has a list
+  uint32_t* qbits;      // [n_keys / 32] set: the query-level cell holds a hit point
+  float4* qpos;         // [M_max] position and id of the active hit points, sorted
   // the GPF_NB_BALL_KNN backward (nb_max > 0): selected pairs, per-point
   // counts / offsets, per-Gaussian ranges of the sorted pairs
   uint32_t* nbkey[2];   // [nb_max] Gaussian ids (sort ping-pong)
@@ -89,16 +99,16 @@ struct IndexBuffers {
   void* nbsort_ws;
   int nbsorted;
   // forward tile splitting (split_items > 0)
-  uint32_t* tparts;     // [tiles_max + 1] parts of each tile (1 = not split), then scanned
-  uint32_t* xoff;       // [tiles_max + 1] parts of each split tile (0 otherwise), then scanned
+  uint32_t* tparts;     // [tiles_max] parts of each tile (1 = not split)
+  uint32_t* xpart;      // [tiles_max / 256 + 1] parts of the split tiles of 256 tiles
   uint4* xunit;         // [GPF_MAX_SPLIT_UNITS] (tile, part, parts, valid) of every split unit
   float* xsum;          // [GPF_MAX_SPLIT_UNITS * (C + 1) * 32] partial sums of split units
   // a centre level (ball_radius > 0): occupancy bits of the centre cells'
   // coarse cells (Grid::cshift), and the hybrid forward's tile splitting
   uint32_t* cocc;       // [cdx * cdy * cdz / 32] set: some mean lies in the cell
   uint32_t* focc;       // [focc_words] the same per centre cell (Grid::fwords > 0)
-  uint32_t* hparts;     // [tiles_max + 1] parts of each tile (1 = not split)
-  uint32_t* hoff;       // [tiles_max + 1] parts of each split tile (0 otherwise), then scanned
+  uint32_t* hparts;     // [tiles_max] parts of each tile (1 = not split)
+  uint32_t* hpart;      // [tiles_max / 256 + 1] parts of the split tiles of 256 tiles
   uint32_t* hitems;     // [tiles_max] listed entries of the centre cells of each tile's box
   uint4* hunit;         // [GPF_MAX_SPLIT_UNITS] (tile, part, parts, valid) of every split unit
   float* hsum;          // [GPF_MAX_SPLIT_UNITS * (C + 2) * 32] partial L, Z and count
@@ -109,6 +119,7 @@ struct IndexBuffers {
   void* gsort_ws;
   void* osort_ws;
   int qsorted, gsorted, osorted;  // which ping-pong buffer holds the result
+  size_t clear_bytes;   // from the header on: everything a build starts from zero
 };
 
 struct IndexDims {
@@ -129,12 +140,17 @@ cudaError_t launch_build(const IndexDims& dims, const IndexBuffers& b, const gpf
 // Forward tile splitting (split_items > 0), after the bucket ranges exist:
 // each tile's estimated work, its parts, and the table of split units
 // (gpf_fwd.cu).
-// The unit list of split tiles: xoff (each tile's parts if split, else 0)
-// is scanned in place, tile t's units are written at xunit[xoff[t] ...], and
-// *n_units (device memory) receives their number; a tile whose units would
-// not all fit under GPF_MAX_SPLIT_UNITS gets tparts = 1 and runs unsplit.
-cudaError_t launch_split_units(int64_t n_tiles, uint32_t* tparts, uint32_t* xoff, uint4* xunit,
-                               uint32_t* n_units, void* scan_ws, cudaStream_t stream);
+// The unit list of split tiles: with xpart[b] the parts of the split tiles
+// among tiles [256 b, 256 b + 256), tile t's units follow those of the split
+// tiles before it in xunit, and *n_units (device memory) receives their
+// number; a tile whose units would not all fit under GPF_MAX_SPLIT_UNITS gets
+// tparts = 1 and runs unsplit.
+constexpr int kTileGroup = 256;
+inline int64_t tile_groups(int64_t tiles) { return (tiles + kTileGroup - 1) / kTileGroup; }
+cudaError_t launch_split_units(int64_t n_tiles, uint32_t* tparts, const uint32_t* xpart,
+                               uint4* xunit, uint32_t* n_units, cudaStream_t stream);
+// Words of IndexBuffers::gpart for n Gaussians.
+size_t gpart_words(int64_t n);
 cudaError_t launch_tile_split(const IndexDims& dims, const IndexBuffers& b, const gpf_queries& q,
                               cudaStream_t stream);
 // The float32 field the pair loops read: f itself, or the decoded arrays of

@@ -8,7 +8,7 @@
 //      digit counts do not depend on the order the earlier passes leave);
 //   1. per pass, one kernel: a block claims the next tile of 3072 keys from
 //      an atomic counter (so every earlier tile is held by a block that is
-//      already running); each warp ranks its own 384 keys, 32 at a time
+//      already running; small sorts take tiles of 1024); each warp ranks its own 384 keys, 32 at a time
 //      (groups of equal digits from bit ballots, per-warp digit counters in
 //      shared memory);
 //      the block publishes its digit counts, orders its keys by digit in
@@ -42,6 +42,12 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / kWarp;
 constexpr int kSortPerThread = 12;
 constexpr int kSortTile = kSortThreads * kSortPerThread;  // 3072
+constexpr int kSortSmallPer = 4;
+constexpr int kSortSmall = kSortThreads * kSortSmallPer;  // 1024
+// Sorts of at most this many elements take tiles of kSortSmall keys, so that
+// they spread over the chip.
+constexpr int64_t kSmallMax = int64_t(1) << 17;
+constexpr int kLookBack = 8;     // status words read per step of the look-back
 constexpr int kBins = 256;
 
 // Exclusive scan across a block of kScanThreads threads; returns the prefix
@@ -169,42 +175,70 @@ __global__ void onesweep_hist_kernel(const uint32_t* __restrict__ keys, const ui
     if (cnt[i]) atomicAdd(&ghist[i], cnt[i]);
 }
 
-__global__ void __launch_bounds__(kSortThreads)
-onesweep_pass_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
-                     uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
-                     const uint32_t* d_n, int64_t n_max, int shift,
-                     const uint32_t* __restrict__ ghist, uint32_t* status,
-                     uint32_t* tile_counter, uint32_t tile_base, uint32_t spin_limit,
-                     uint32_t* stalled) {
-  constexpr int kWarpKeys = kSortPerThread * kWarp;   // each warp ranks its own 384 keys
-  __shared__ uint32_t s_keys[kSortTile];
-  __shared__ uint32_t s_vals[kSortTile];
-  __shared__ uint32_t wcnt[kSortWarps][kBins];   // digit counts of each warp, then its bases
-  __shared__ uint32_t tile_start[kBins];
-  __shared__ uint32_t out_base[kBins];
-  __shared__ uint32_t total;
-  __shared__ uint32_t s_tile;
+// One pass of one sort: the job's blocks claim its tiles from its own counter.
+struct PassJob {
+  const uint32_t* keys_in;
+  const uint32_t* vals_in;
+  uint32_t* keys_out;
+  uint32_t* vals_out;
+  const uint32_t* d_n;      // element count on the device, or null (n_max)
+  int64_t n_max;
+  const uint32_t* ghist;    // [kBins] digit counts of this pass
+  uint32_t* status;         // [tiles][kBins]
+  uint32_t* counter;        // tiles claimed so far
+  uint32_t blocks;          // blocks of the launch that work on this job
+  int shift;
+  int small;                // tiles of kSortSmall keys instead of kSortTile
+};
+struct PassArgs {
+  PassJob job[kSortMaxJobs];
+  uint32_t tile_base;
+  uint32_t spin_limit;
+  uint32_t* stalled;
+};
 
+struct PassShared {
+  uint32_t keys[kSortTile];
+  uint32_t vals[kSortTile];
+  uint32_t wcnt[kSortWarps][kBins];   // digit counts of each warp, then its bases
+  uint32_t tile_start[kBins];
+  uint32_t out_base[kBins];
+  uint32_t total;
+  uint32_t tile;
+};
+
+template <int PER>
+__device__ __forceinline__ void onesweep_tile(const PassJob& a, PassShared& s, uint32_t tile_base,
+                                              uint32_t spin_limit, uint32_t* stalled) {
+  constexpr int kTile = kSortThreads * PER;
+  constexpr int kWarpKeys = PER * kWarp;   // each warp ranks its own keys
   const int t = threadIdx.x;        // kSortThreads == kBins: thread t owns digit t
   const int lane = t & 31, warp = t >> 5;
-  if (t == 0) s_tile = tile_base + atomicAdd(tile_counter, 1u);
+  if (t == 0) s.tile = tile_base + atomicAdd(a.counter, 1u);
 #pragma unroll
-  for (int w = 0; w < kSortWarps; ++w) wcnt[w][t] = 0;
+  for (int w = 0; w < kSortWarps; ++w) s.wcnt[w][t] = 0;
+  const uint32_t n = load_count(a.d_n, a.n_max);
+  const uint32_t my_ghist = a.ghist[t];
   __syncthreads();
-  const uint32_t n = load_count(d_n, n_max);
-  const uint32_t tile = s_tile;
-  const int64_t base = (int64_t)tile * kSortTile;
+  const uint32_t tile = s.tile;
+  const int64_t base = (int64_t)tile * kTile;
   if (base >= (int64_t)n) return;                    // the whole block
-  const int tile_n = (int)min((int64_t)kSortTile, (int64_t)n - base);
+  const int tile_n = (int)min((int64_t)kTile, (int64_t)n - base);
+  const int shift = a.shift;
 
-  // 1. ranks inside the warp's 384 keys (taken 32 at a time in order):
-  //    (rank << 9) | digit, digit kBins for the positions past the tile
-  uint32_t rd[kSortPerThread];
+  // 1. ranks inside the warp's keys (taken 32 at a time in order); the keys stay
+  //    in registers, all loaded before the first is ranked
+  uint32_t rd[PER], key[PER];
 #pragma unroll
-  for (int it = 0; it < kSortPerThread; ++it) {
+  for (int it = 0; it < PER; ++it) {
+    const int li = warp * kWarpKeys + it * kWarp + lane;
+    key[it] = li < tile_n ? __ldg(a.keys_in + base + li) : 0u;
+  }
+#pragma unroll
+  for (int it = 0; it < PER; ++it) {
     const int li = warp * kWarpKeys + it * kWarp + lane;
     const bool ok = li < tile_n;
-    const uint32_t d = ok ? (keys_in[base + li] >> shift) & (kBins - 1) : kBins;
+    const uint32_t d = (key[it] >> shift) & (kBins - 1);
     // the lanes with the same digit: nine ballots (validity, then each digit
     // bit), cheaper here than __match_any_sync
     uint32_t peers = __ballot_sync(kFullMask, ok);
@@ -215,69 +249,110 @@ onesweep_pass_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
       peers &= ((d >> b) & 1u) ? m : ~m;
     }
     uint32_t r0 = 0;
-    if (ok) r0 = wcnt[warp][d];
+    if (ok) r0 = s.wcnt[warp][d];
     __syncwarp();
-    if (ok && (peers & lanemask_lt()) == 0) wcnt[warp][d] = r0 + (uint32_t)__popc(peers);
+    if (ok && (peers & lanemask_lt()) == 0) s.wcnt[warp][d] = r0 + (uint32_t)__popc(peers);
     __syncwarp();
-    rd[it] = ((r0 + (uint32_t)__popc(peers & lanemask_lt())) << 9) | d;
+    rd[it] = r0 + (uint32_t)__popc(peers & lanemask_lt());
   }
   __syncthreads();
   // 2. digit t: the warps' bases and the tile's count; publish the count
-  //    (tile 0: its inclusive prefix)
+  //    (tile 0: its inclusive prefix). The values are fetched meanwhile.
+  uint32_t val[PER];
+#pragma unroll
+  for (int it = 0; it < PER; ++it) {
+    const int li = warp * kWarpKeys + it * kWarp + lane;
+    val[it] = li < tile_n ? __ldg(a.vals_in + base + li) : 0u;
+  }
   uint32_t c = 0;
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) {
-    const uint32_t x = wcnt[w][t];
-    wcnt[w][t] = c;
+    const uint32_t x = s.wcnt[w][t];
+    s.wcnt[w][t] = c;
     c += x;
   }
-  st_status(status + (int64_t)tile * kBins + t, (tile == 0 ? kFlagPre : kFlagAgg) | c);
-  tile_start[t] = block_exclusive_scan(c, &total);
-  const uint32_t digit_start = block_exclusive_scan(ghist[t], &total);
-  // 3. keys in digit order in shared memory (reloaded: the tile is in L1/L2)
+  st_status(a.status + (int64_t)tile * kBins + t, (tile == 0 ? kFlagPre : kFlagAgg) | c);
+  s.tile_start[t] = block_exclusive_scan(c, &s.total);
+  const uint32_t digit_start = block_exclusive_scan(my_ghist, &s.total);
+  // 3. keys in digit order in shared memory
 #pragma unroll
-  for (int it = 0; it < kSortPerThread; ++it) {
-    const uint32_t d = rd[it] & 511u;
-    if (d < (uint32_t)kBins) {
-      const int li = warp * kWarpKeys + it * kWarp + lane;
-      const uint32_t pos = tile_start[d] + wcnt[warp][d] + (rd[it] >> 9);
-      s_keys[pos] = keys_in[base + li];
-      s_vals[pos] = vals_in[base + li];
+  for (int it = 0; it < PER; ++it) {
+    const int li = warp * kWarpKeys + it * kWarp + lane;
+    if (li < tile_n) {
+      const uint32_t d = (key[it] >> shift) & (kBins - 1);
+      const uint32_t pos = s.tile_start[d] + s.wcnt[warp][d] + rd[it];
+      s.keys[pos] = key[it];
+      s.vals[pos] = val[it];
     }
   }
-  // 4. digit t in the earlier tiles: walk back to the nearest inclusive prefix
+  // 4. digit t in the earlier tiles: walk back to the nearest inclusive
+  //    prefix, kLookBack tiles a step (their status words are read together:
+  //    one after the other, the chain of L2 latencies was most of a pass)
   uint32_t excl = 0;
   if (tile > 0) {
     int64_t j = (int64_t)tile - 1;
     uint32_t spins = 0;
-    while (j >= 0) {
-      const uint32_t sv = ld_status(status + j * kBins + t);
-      const uint32_t flag = sv & ~kValMask;
-      if (flag == 0u) {
-        if (++spins >= spin_limit) {
-          atomicExch(stalled, 1u);
-          break;
-        }
+    bool found = false;
+    while (j >= 0 && !found) {
+      uint32_t sv[kLookBack];
+#pragma unroll
+      for (int i = 0; i < kLookBack; ++i)
+        sv[i] = j - i >= 0 ? ld_status(a.status + (j - i) * kBins + t) : kFlagPre;
+      // not there yet: poll this one word (eight at a time from every waiting
+      // block kept the tiles that are being ranked from the L2)
+      while ((sv[0] & ~kValMask) == 0u && ++spins < spin_limit) {
         __nanosleep(64);
-        continue;
+        sv[0] = ld_status(a.status + j * kBins + t);
       }
-      excl += sv & kValMask;
-      if (flag == kFlagPre) break;
-      --j;
+      if ((sv[0] & ~kValMask) == 0u) {
+        atomicExch(stalled, 1u);
+        break;
+      }
+      int used = 0;
+#pragma unroll
+      for (int i = 0; i < kLookBack; ++i) {
+        const uint32_t flag = sv[i] & ~kValMask;
+        if (!found && used == i && flag != 0u) {
+          excl += sv[i] & kValMask;
+          used = i + 1;
+          found = flag == kFlagPre;
+        }
+      }
+      j -= used;
     }
-    st_status(status + (int64_t)tile * kBins + t, kFlagPre | ((excl + c) & kValMask));
+    st_status(a.status + (int64_t)tile * kBins + t, kFlagPre | ((excl + c) & kValMask));
   }
-  out_base[t] = digit_start + excl - tile_start[t];
+  s.out_base[t] = digit_start + excl - s.tile_start[t];
   __syncthreads();
   // 5. out in digit order: runs of one digit go to consecutive addresses
   for (int p = t; p < tile_n; p += kSortThreads) {
-    const uint32_t k = s_keys[p];
-    const uint32_t dst = out_base[(k >> shift) & (kBins - 1)] + (uint32_t)p;
+    const uint32_t k = s.keys[p];
+    const uint32_t dst = s.out_base[(k >> shift) & (kBins - 1)] + (uint32_t)p;
     if (dst < n) {
-      keys_out[dst] = k;
-      vals_out[dst] = s_vals[p];
+      a.keys_out[dst] = k;
+      a.vals_out[dst] = s.vals[p];
     }
   }
+}
+
+// One pass of up to kSortMaxJobs independent sorts: the blocks are shared out
+// over the jobs in order. A pass of one sort leaves most of the chip waiting
+// on its look-back and its tail; the index build's three sorts in one launch
+// fill it, and launch once per pass instead of three times.
+__global__ void __launch_bounds__(kSortThreads, 4)
+onesweep_pass_kernel(const __grid_constant__ PassArgs a) {
+  __shared__ PassShared s;
+  uint32_t blk = blockIdx.x;
+  int j = 0;
+#pragma unroll
+  for (int k = 0; k < kSortMaxJobs - 1; ++k)
+    if (j == k && blk >= a.job[k].blocks) {
+      blk -= a.job[k].blocks;
+      j = k + 1;
+    }
+  const PassJob& job = a.job[j];
+  if (job.small) onesweep_tile<kSortSmallPer>(job, s, a.tile_base, a.spin_limit, a.stalled);
+  else onesweep_tile<kSortPerThread>(job, s, a.tile_base, a.spin_limit, a.stalled);
 }
 
 }  // namespace
@@ -303,14 +378,24 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n,
   return cudaGetLastError();
 }
 
-int64_t radix_tiles(int64_t n_max) { return (n_max + kSortTile - 1) / kSortTile; }
+bool radix_small(int64_t n_max) { return n_max <= kSmallMax; }
+
+int64_t radix_tiles(int64_t n_max) {
+  const int64_t tile = radix_small(n_max) ? kSortSmall : kSortTile;
+  return (n_max + tile - 1) / tile;
+}
+
+namespace {
+constexpr size_t kCountBytes = sizeof(uint32_t) * (kMaxPasses * kBins + kMaxPasses);
+}
 
 // The digit counts and tile counters of every pass, then the per-pass tile
-// status words.
-size_t radix_sort_workspace_bytes(int64_t n_max) {
-  const int64_t hist_n = radix_tiles(n_max) * kBins;
-  return align_up(sizeof(uint32_t) * (kMaxPasses * kBins + kMaxPasses)) +
-         align_up((size_t)kMaxPasses * hist_n * sizeof(uint32_t));
+// status words: all of it is zero before a sort.
+size_t radix_sort_workspace_bytes(int64_t n_max, int bits) {
+  // (for every count up to n_max: the most small tiles may exceed n_max's own)
+  const int64_t tiles = std::max(radix_tiles(n_max), radix_tiles(std::min(n_max, kSmallMax)));
+  return align_up(kCountBytes) +
+         align_up((size_t)radix_sort_passes(bits) * tiles * kBins * sizeof(uint32_t));
 }
 
 int radix_sort_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
@@ -326,61 +411,68 @@ cudaError_t launch_sort_wait_probe(void* buf, uint32_t spin_limit, uint32_t* sta
   cudaError_t e = cudaMemsetAsync(buf, 0, sort_wait_probe_bytes(), stream);
   if (e != cudaSuccess) return e;
   uint32_t* w = static_cast<uint32_t*>(buf);
-  uint32_t* keys_in = w;
-  uint32_t* vals_in = w + 2 * kSortTile;
-  uint32_t* keys_out = w + 4 * kSortTile;
-  uint32_t* vals_out = w + 6 * kSortTile;
   uint32_t* ghist = w + 8 * kSortTile;
-  uint32_t* counter = ghist + kBins;
-  uint32_t* status = counter + 1;
+  PassArgs a{};
+  a.job[0] = PassJob{w, w + 2 * kSortTile, w + 4 * kSortTile, w + 6 * kSortTile, nullptr,
+                     2 * kSortTile, ghist, ghist + kBins + 1, ghist + kBins, 1u, 0, 0};
   // one block, claiming tile 1 (tile_base 1): tile 0 is never processed, so
   // its status words stay 0 and the walk back from tile 1 waits on them
-  onesweep_pass_kernel<<<1, kSortThreads, 0, stream>>>(
-      keys_in, vals_in, keys_out, vals_out, nullptr, 2 * kSortTile, 0, ghist, status, counter,
-      1u, spin_limit, stalled);
+  a.tile_base = 1u;
+  a.spin_limit = spin_limit;
+  a.stalled = stalled;
+  onesweep_pass_kernel<<<1, kSortThreads, 0, stream>>>(a);
   note_launches(1);
   return cudaGetLastError();
 }
 
 uint32_t* radix_sort_counts(void* ws) { return static_cast<uint32_t*>(ws); }
 
-cudaError_t radix_sort_clear_counts(void* ws, cudaStream_t stream) {
-  return cudaMemsetAsync(ws, 0, sizeof(uint32_t) * (kMaxPasses * kBins + kMaxPasses), stream);
-}
-
-cudaError_t radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                             int64_t n_max, const uint32_t* d_n, int bits, void* ws,
-                             uint32_t* stalled, cudaStream_t stream, bool counted) {
-  if (n_max <= 0) return cudaSuccess;
-  if (n_max >= kMaxSortN) return cudaErrorInvalidValue;
-  const int64_t tiles = radix_tiles(n_max);
-  const int passes = radix_sort_passes(bits);
-  if (passes == 0) return cudaSuccess;
-  char* p = static_cast<char*>(ws);
-  uint32_t* ghist = reinterpret_cast<uint32_t*>(p);        // [kMaxPasses][kBins]
-  uint32_t* counters = ghist + kMaxPasses * kBins;          // [kMaxPasses]
-  p += align_up(sizeof(uint32_t) * (kMaxPasses * kBins + kMaxPasses));
-  uint32_t* status = reinterpret_cast<uint32_t*>(p);        // [passes][tiles][kBins]
-  cudaError_t e;
-  if (!counted && (e = radix_sort_clear_counts(ws, stream)) != cudaSuccess) return e;
-  e = cudaMemsetAsync(status, 0, sizeof(uint32_t) * (size_t)passes * tiles * kBins, stream);
-  if (e != cudaSuccess) return e;
-  if (!counted) {
-    const unsigned hblocks = (unsigned)std::min<int64_t>(tiles, 1024);
-    onesweep_hist_kernel<<<hblocks, kSortThreads, 0, stream>>>(k0, d_n, n_max, passes, ghist);
+cudaError_t radix_sort_counted(const SortTask* tasks, int count, uint32_t* stalled,
+                               cudaStream_t stream) {
+  if (count > kSortMaxJobs) return cudaErrorInvalidValue;
+  int passes = 0;
+  for (int k = 0; k < count; ++k) {
+    if (tasks[k].n_max >= kMaxSortN) return cudaErrorInvalidValue;
+    if (tasks[k].n_max > 0) passes = std::max(passes, radix_sort_passes(tasks[k].bits));
+  }
+  for (int pass = 0; pass < passes; ++pass) {
+    PassArgs a{};
+    a.spin_limit = kSpinLimit;
+    a.stalled = stalled;
+    unsigned blocks = 0;
+    for (int k = 0; k < count; ++k) {
+      const SortTask& t = tasks[k];
+      if (t.n_max <= 0 || pass >= radix_sort_passes(t.bits)) continue;
+      const int64_t tiles = radix_tiles(t.n_max);
+      uint32_t* counts = static_cast<uint32_t*>(t.ws);       // [kMaxPasses][kBins], counters
+      uint32_t* status = reinterpret_cast<uint32_t*>(static_cast<char*>(t.ws) +
+                                                     align_up(kCountBytes));
+      const bool odd = pass & 1;
+      a.job[k] = PassJob{odd ? t.k1 : t.k0, odd ? t.v1 : t.v0, odd ? t.k0 : t.k1,
+                         odd ? t.v0 : t.v1, t.d_n, t.n_max, counts + pass * kBins,
+                         status + (size_t)pass * tiles * kBins, counts + kMaxPasses * kBins + pass,
+                         (uint32_t)tiles, pass * 8, radix_small(t.n_max) ? 1 : 0};
+      blocks += (unsigned)tiles;
+    }
+    onesweep_pass_kernel<<<blocks, kSortThreads, 0, stream>>>(a);
     note_launches(1);
   }
-  uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
-  for (int pass = 0; pass < passes; ++pass) {
-    onesweep_pass_kernel<<<(unsigned)tiles, kSortThreads, 0, stream>>>(
-        ki, vi, ko, vo, d_n, n_max, pass * 8, ghist + pass * kBins,
-        status + (size_t)pass * tiles * kBins, counters + pass, 0u, kSpinLimit, stalled);
-    uint32_t* tmp;
-    tmp = ki; ki = ko; ko = tmp;
-    tmp = vi; vi = vo; vo = tmp;
-  }
-  note_launches(passes);
   return cudaGetLastError();
+}
+
+cudaError_t radix_sort_pairs(const SortTask& t, uint32_t* stalled, cudaStream_t stream) {
+  if (t.n_max <= 0) return cudaSuccess;
+  if (t.n_max >= kMaxSortN) return cudaErrorInvalidValue;
+  const int passes = radix_sort_passes(t.bits);
+  if (passes == 0) return cudaSuccess;
+  const cudaError_t e =
+      cudaMemsetAsync(t.ws, 0, radix_sort_workspace_bytes(t.n_max, t.bits), stream);
+  if (e != cudaSuccess) return e;
+  const unsigned hblocks = (unsigned)std::min<int64_t>(radix_tiles(t.n_max), 1024);
+  onesweep_hist_kernel<<<hblocks, kSortThreads, 0, stream>>>(t.k0, t.d_n, t.n_max, passes,
+                                                             radix_sort_counts(t.ws));
+  note_launches(1);
+  return radix_sort_counted(&t, 1, stalled, stream);
 }
 
 }  // namespace gpf
