@@ -225,8 +225,9 @@ typedef struct gpf_grid_config {
                             points is one work unit; > 0 = the build
                             estimates each tile's work (the list entries its
                             points walk) and splits a tile above this many
-                            into up to GPF_MAX_TILE_PARTS units over disjoint
-                            chunks of its lists, whose partial sums a final
+                            (and above its share of all tiles' work) into up
+                            to GPF_MAX_TILE_PARTS units over disjoint chunks
+                            of its lists, whose partial sums a final
                             kernel adds in part order (results still
                             deterministic; they differ from the unsplit sums
                             by summation order only)                         */

@@ -108,8 +108,6 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   t.qsort_ws = take(radix_sort_workspace_bytes(M, d.grid.key_bits));
   t.osort_ws = take(radix_sort_workspace_bytes(N, d.grid.obits));
   t.gsort_ws = take(radix_sort_workspace_bytes(P, d.grid.hash_bits));
-  if (d.split_items > 0)
-    t.xpart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tile_groups(tiles) + 1)));
   if (d.grid.blevel >= 0) {
     t.cocc = reinterpret_cast<uint32_t*>(
         take(sizeof(uint32_t) * (((size_t)d.grid.cdx * d.grid.cdy * d.grid.cdz + 31) / 32)));
@@ -118,7 +116,7 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   }
   t.clear_bytes = off;
   t.rec = reinterpret_cast<float*>(take(sizeof(float) * N * rec_stride(d.channels)));
-  t.box = reinterpret_cast<uint4*>(take(sizeof(uint4) * N));
+  t.vet = reinterpret_cast<VetRec*>(take(sizeof(VetRec) * N));
   t.gcount = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * N));
   t.glive = reinterpret_cast<uint8_t*>(take(sizeof(uint8_t) * N));
   t.gmask = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * N));
@@ -254,11 +252,13 @@ gpf_status check_same(const gpf_index* ix, const gpf_field* f, const gpf_queries
 }  // namespace
 
 namespace gpf {
-int64_t persistent_blocks(const void* kernel, int threads, int64_t max_blocks) {
+int64_t persistent_blocks(const void* kernel, int threads, int64_t max_blocks,
+                          size_t dynamic_smem) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads,
+                                                    dynamic_smem) != cudaSuccess ||
       sms <= 0 || per_sm <= 0) {
     cudaGetLastError();  // clear; fall back to one block per work unit
     return max_blocks > 0 ? max_blocks : 1;

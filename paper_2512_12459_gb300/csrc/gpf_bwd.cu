@@ -55,7 +55,6 @@ struct BwdArgs {
   const uint2* qbox;      // [N] query-level cell bounds (pack_qbox), from the build
   void* bpart;            // [kSplitMax * kSplitWays * NS] split Gaussians' partials (T)
   const float* rec;
-  const uint4* box;
   const uint32_t* order;  // Gaussian ids in mean-cell order
   const uint2* nbrange;   // hybrid neighbourhood: [start, end) of each Gaussian's pairs
   const uint32_t* nbval;  // hybrid neighbourhood: the pairs' hit point positions
@@ -831,7 +830,6 @@ cudaError_t launch_backward(const IndexDims& d, const IndexBuffers& b, const gpf
   a.qbox = b.qbox;
   a.bpart = b.bpart;
   a.rec = b.rec;
-  a.box = b.box;
   a.order = b.oval[b.osorted];
   a.nbrange = nullptr;
   a.nbval = nullptr;

@@ -37,7 +37,8 @@ struct DeviceHeader {
   uint32_t nb_pairs;     // (hit point, Gaussian) pairs of the last hybrid backward
   uint32_t n_xunits;     // work units of the split forward tiles (<= GPF_MAX_SPLIT_UNITS)
   uint32_t n_hunits;     // work units of the split hybrid forward tiles (same limit)
-  uint32_t pad[48];
+  unsigned long long split_cost;  // estimated work of all forward tiles
+  uint32_t pad[46];
 };
 static_assert(sizeof(DeviceHeader) == 256, "header is one 256-byte block");
 
@@ -220,26 +221,41 @@ __host__ __device__ __forceinline__ uint32_t bucket_of(const Grid& g, int L, uin
   return cell_hash(g, L, ix, iy, iz).bucket;
 }
 
-// Level box of a Gaussian, packed in a uint4:
-//   x = lo.x | level << 20, y = lo.y, z = lo.z (cell coordinates on that level),
-//   w = span.x | span.y << 8 | span.z << 16 (hi = lo + span, each span <= 255).
-struct LevelBox {
-  int level;
-  uint32_t lx, ly, lz, hx, hy, hz;
+// What the pair loops vet an entry by, one 32-byte load: the mean, the radius
+// of the k-sigma bounding sphere (with the level in its low mantissa bits, as
+// the record's) and the level box. Cells of a level are packed 21 bits per
+// axis, 20 of coordinate below a guard bit: nlo = guard - lo and hig = hi +
+// guard per axis, so that a cell c lies in the box exactly when c + nlo and
+// hig - c both have all three guard bits set (neither crosses into the next
+// axis). nlo = 0: no box.
+struct __align__(32) VetRec {
+  float x, y, z, radius;
+  unsigned long long nlo, hig;
 };
-__device__ __forceinline__ LevelBox unpack_box(const uint4 b) {
-  LevelBox r;
-  r.level = (int)(b.x >> 20);
-  r.lx = b.x & kCoordMax;
-  r.ly = b.y;
-  r.lz = b.z;
-  r.hx = r.lx + (b.w & 0xffu);
-  r.hy = r.ly + ((b.w >> 8) & 0xffu);
-  r.hz = r.lz + ((b.w >> 16) & 0xffu);
-  return r;
+constexpr unsigned long long kCellGuard = (1ull << 20) | (1ull << 41) | (1ull << 62);
+__host__ __device__ __forceinline__ unsigned long long pack_cell(uint32_t x, uint32_t y,
+                                                                 uint32_t z) {
+  return (unsigned long long)x | ((unsigned long long)y << 21) | ((unsigned long long)z << 42);
 }
-__device__ __forceinline__ bool box_holds(const LevelBox& b, uint32_t x, uint32_t y, uint32_t z) {
-  return x >= b.lx && x <= b.hx && y >= b.ly && y <= b.hy && z >= b.lz && z <= b.hz;
+__host__ __device__ __forceinline__ bool cell_in(const VetRec& r, unsigned long long c) {
+  return ((c + r.nlo) & (r.hig - c) & kCellGuard) == kCellGuard;
+}
+__device__ __forceinline__ void ld_global_v8(const float* p, float* r) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]),
+        "=f"(r[7])
+      : "l"(p));
+}
+__device__ __forceinline__ VetRec load_vet(const VetRec* p) {
+  float f[8];
+  ld_global_v8(reinterpret_cast<const float*>(p), f);
+  VetRec r;
+  r.x = f[0]; r.y = f[1]; r.z = f[2]; r.radius = f[3];
+  r.nlo = (unsigned long long)__float_as_uint(f[4]) |
+          ((unsigned long long)__float_as_uint(f[5]) << 32);
+  r.hig = (unsigned long long)__float_as_uint(f[6]) |
+          ((unsigned long long)__float_as_uint(f[7]) << 32);
+  return r;
 }
 
 // Rotation and scale of a Gaussian from its raw parameters: R(q/|q|) with
@@ -314,6 +330,43 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 constexpr float kLog2e = 1.4426950408889634f;
 
+// 1 / sqrt(v) on the special-function unit (2 ulp) for v >= 0; below the
+// smallest normal float as for that float, so that a distance made from it,
+// v / sqrt(v), is finite and below 1e-18.
+__device__ __forceinline__ float rsqrt_approx(float v) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(v, 1.17549435e-38f)));
+  return y;
+}
+// Two float32 values in one 64-bit register, and the packed arithmetic of
+// sm_100 on them: one instruction for two IEEE operations, each rounded as the
+// scalar one.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+
 // Lower bound of sqrt(Q) = |M (x - mu)| over an axis-aligned box with centre
 // c and half-extent h: |M(c - mu)| - |(|M| h)|, lowered by 4e-6 (|M(c-mu)| +
 // |(|M| h)|) to cover float32 rounding. A pair inside the box with Q <= k^2
@@ -331,6 +384,27 @@ __device__ __forceinline__ float mahalanobis_lower_bound(const float* Mrow, floa
   float vn = sqrtf(fmaf(v0, v0, fmaf(v1, v1, v2 * v2)));
   float sn = sqrtf(fmaf(s0, s0, fmaf(s1, s1, s2 * s2)));
   return (vn - sn) - 4e-6f * (vn + sn);
+}
+
+// Position of the j-th (from 0) set bit of m, which has more than j.
+__device__ __forceinline__ uint32_t nth_bit(unsigned long long m, uint32_t j) {
+  uint32_t w = (uint32_t)m, pos = 0;
+  const uint32_t lo = (uint32_t)__popc(w);
+  if (j >= lo) {
+    j -= lo;
+    w = (uint32_t)(m >> 32);
+    pos = 32;
+  }
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    const uint32_t c = (uint32_t)__popc(w & ((1u << h) - 1u));
+    if (j >= c) {
+      j -= c;
+      w >>= h;
+      pos += h;
+    }
+  }
+  return pos;
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {

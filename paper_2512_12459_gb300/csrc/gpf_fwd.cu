@@ -1,20 +1,22 @@
 // gpf_radiance_fwd: radiance at hit points (Sec. 4.2, aggregation equation;
 // the soft falloff and soft normalisation of the query listing of Algorithm S3).
 //
-// One warp per tile of 32 consecutive hit points in cell-sorted order. For
-// every grid level that holds Gaussians, the lanes find their cell on that
-// level and group equal cells (__match_any_sync):
-//   * few distinct cells (the Gaussians of this level are large next to the
-//     tile): warp-cooperative mode. The lanes walk the lists of those cells
-//     together, 32 entries at a time; each lane vets one candidate (it belongs
+// A tile is 32 consecutive hit points in cell-sorted order; a warp takes it, or
+// a team of warps where there are few tiles. The lanes look up their cell's
+// list on every grid level that holds Gaussians and group equal cells:
+//   * levels with few distinct cells (the Gaussians there are large next to the
+//     tile) are walked together. The lists of all their cells are laid end to
+//     end and vetted 32 entries at a time, an entry per lane: the entry belongs
 //     to this level and cell, it was not already taken from an earlier cell of
-//     the tile, and neither its bounding sphere nor a lower bound of its
-//     Mahalanobis distance rules out the tile's box of hit points). Survivors
-//     are staged in shared memory and every lane evaluates all of them.
-//   * many distinct cells (the Gaussians are small next to the spacing of the
-//     hit points): pooled mode. The lanes' own cell lists are concatenated and
-//     taken 32 (hit point, entry) items at a time, one per lane; a segmented
-//     sum over the lanes returns each hit point's share to its lane.
+//     the tile, and its bounding sphere reaches the tile's box. The ids that
+//     pass are queued and their records loaded 32 at a time, tested against a
+//     lower bound of their Mahalanobis distance to the box, staged in shared
+//     memory, and every lane evaluates all of them at its own hit point.
+//   * levels with many distinct cells (the Gaussians are small next to the
+//     spacing of the hit points) are pooled: the lanes' own lists, of all these
+//     levels, are laid end to end and taken 32 (hit point, entry) items at a
+//     time, one per lane; a segmented sum over the lanes returns each hit
+//     point's share to its lane.
 // Every lane applies the exact predicate Q <= k^2, so the result equals the
 // brute-force sum over {i : Q_i <= k^2}. With no cell lists (k = +INF or
 // brute force) the candidates are all Gaussians, in index order.
@@ -32,20 +34,17 @@ namespace {
 
 constexpr int kFwdWarps = 4;
 constexpr int kFwdThreads = kFwdWarps * kWarp;
-// A tile whose hit points fall in at most Grid::coop cells of a level walks
-// that level cooperatively; kUnionMax bounds that threshold.
-constexpr int kUnionMax = GPF_MAX_COOP_CELLS;
+constexpr int kQueue = 128;   // vetted ids of a warp that wait for their records
 
 struct FwdArgs {
   Grid grid;
-  const uint32_t* qkey;    // sorted query-level keys of hit points
   const uint32_t* qval;    // sorted hit point ids
   const float4* qpos;      // sorted positions and ids of the active ones
   const DeviceHeader* header;
   const float* albedo;     // [C,M] or null
   int64_t m;
   const float* rec;
-  const uint4* box;
+  const VetRec* vet;
   const uint2* brange;     // [n_buckets] [start, end) of each bucket's list
   const uint32_t* listed;  // [n_buckets / 32] set: the bucket has a list
   const uint32_t* gval;    // sorted entries (Gaussian ids)
@@ -81,12 +80,12 @@ __device__ __forceinline__ float warp_max(float v) {
 constexpr int kKernGauss = 0, kKernFalloff = 1, kKernDisk = 2;
 constexpr float kNegHalfLog2e = -0.72134752044448170368f;   // -log2(e) / 2
 
-// |d| from d2 = |d|^2 > 0: one reciprocal square root and one Newton step
-// on the square root (residual d2 - s^2 by a fused multiply-add), which
-// leaves about 1 ulp of relative error, as a correctly rounded square root
-// would within an ulp, without its special-case branch.
+// |d| from d2 = |d|^2: one reciprocal square root and one Newton step on the
+// square root (residual d2 - s^2 by a fused multiply-add), which leaves about
+// 1 ulp of relative error, as a correctly rounded square root would within an
+// ulp, without its special-case branch.
 __device__ __forceinline__ float dist_of(float d2) {
-  const float y = rsqrtf(d2);
+  const float y = rsqrt_approx(d2);
   const float s = d2 * y;
   return fmaf(0.5f * y, fmaf(-s, s, d2), s);
 }
@@ -99,10 +98,8 @@ __device__ __forceinline__ float pair_exp2(float Q, float dx, float dy, float dz
   float e = Q * kNegHalfLog2e;
   if (KERN == kKernFalloff) {
     const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    if (d2 > a.r2) {
-      const float t = (dist_of(d2) - a.r) * a.tscale;   // as staged_weight: same w bit for bit
-      e = fmaf(-t, t, e);
-    }
+    const float t = fmaxf(dist_of(d2) - a.r, 0.0f) * a.tscale;   // as eval_staged: same w
+    e = fmaf(-t, t, e);
   }
   return ex2_approx(e);
 }
@@ -154,54 +151,101 @@ __device__ __forceinline__ void eval_pair(const float* __restrict__ r, float px,
   }
 }
 
-// Weight of a staged record r at (px, py, pz) without branches: 0 unless
-// Q <= k^2, else pair_exp2's weight, bit for bit.
-template <int KERN>
-__device__ __forceinline__ float staged_weight(const float* __restrict__ r, float px, float py,
-                                               float pz, const FwdArgs& a) {
-  const float dx = px - r[0], dy = py - r[1], dz = pz - r[2];
-  const float u0 = fmaf(r[4], dx, fmaf(r[5], dy, r[6] * dz));
-  const float u1 = fmaf(r[7], dx, fmaf(r[8], dy, r[9] * dz));
-  const float u2 = fmaf(r[10], dx, fmaf(r[11], dy, r[12] * dz));
-  const float Q = fmaf(u0, u0, fmaf(u1, u1, u2 * u2));
-  float e = Q * kNegHalfLog2e;
-  if (KERN == kKernFalloff) {
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float t = (dist_of(d2) - a.r) * a.tscale;   // not used when d2 <= r^2
-    e = d2 > a.r2 ? fmaf(-t, t, e) : e;
+// Staged records, a field after the other so that one 16-byte load gives a
+// field of four records as two packed pairs: -mu (3), M (9), Phi (C).
+__host__ __device__ constexpr int stage_fields(int C) { return 12 + C; }
+
+// Every staged record of the walked levels at this lane's hit point, four at a
+// time as straight-line code, two records to an instruction: the evaluation is
+// bound by the instructions it issues, about 23 per record packed and 40 not.
+// Every value is rounded as in pair_weight. nk is a multiple of 4: the slots
+// past the last record hold a NaN mean, which fails Q <= k^2, and finite Phi,
+// so their weight is 0. L and Z keep the even and the odd records' sums apart.
+template <int C, int KERN>
+__device__ __forceinline__ void eval_staged(const float* __restrict__ st, int nk, float px,
+                                            float py, float pz, const FwdArgs& a,
+                                            f32x2 (&L)[C], f32x2& Z) {
+  const f32x2 px2 = pack2(px, px), py2 = pack2(py, py), pz2 = pack2(pz, pz);
+  const f32x2 c_e = pack2(-kNegHalfLog2e, -kNegHalfLog2e);
+  const f32x2 c_neg = pack2(-1.0f, -1.0f), c_half = pack2(0.5f, 0.5f);
+  const f32x2 c_r = pack2(-a.r, -a.r), c_t = pack2(a.tscale, a.tscale);
+  for (int s = 0; s < nk; s += 4) {
+    auto field = [&](int f) {
+      return *reinterpret_cast<const ulonglong2*>(st + f * kWarp + s);
+    };
+    f32x2 w[2];
+    {
+      const ulonglong2 nx = field(0), ny = field(1), nz = field(2);
+      const f32x2 dx[2] = {add2(px2, nx.x), add2(px2, nx.y)};
+      const f32x2 dy[2] = {add2(py2, ny.x), add2(py2, ny.y)};
+      const f32x2 dz[2] = {add2(pz2, nz.x), add2(pz2, nz.y)};
+      f32x2 d2[2];
+      if (KERN != kKernGauss) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          d2[h] = fma2(dx[h], dx[h], fma2(dy[h], dy[h], mul2(dz[h], dz[h])));
+      }
+      if (KERN == kKernDisk) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float d0, d1;
+          unpack2(d2[h], d0, d1);
+          w[h] = pack2(d0 <= a.r2 ? 1.0f : 0.0f, d1 <= a.r2 ? 1.0f : 0.0f);
+        }
+      } else {
+        f32x2 u[3][2];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const ulonglong2 m0 = field(3 + 3 * j), m1 = field(4 + 3 * j), m2 = field(5 + 3 * j);
+          u[j][0] = fma2(m0.x, dx[0], fma2(m1.x, dy[0], mul2(m2.x, dz[0])));
+          u[j][1] = fma2(m0.y, dx[1], fma2(m1.y, dy[1], mul2(m2.y, dz[1])));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const f32x2 Q = fma2(u[0][h], u[0][h], fma2(u[1][h], u[1][h], mul2(u[2][h], u[2][h])));
+          f32x2 e = mul2(Q, c_e);          // minus the exponent
+          if (KERN == kKernFalloff) {
+            float d0, d1;
+            unpack2(d2[h], d0, d1);
+            const f32x2 y = pack2(rsqrt_approx(d0), rsqrt_approx(d1));
+            const f32x2 sq = mul2(d2[h], y);
+            const f32x2 res = fma2(mul2(sq, c_neg), sq, d2[h]);
+            const f32x2 dist = fma2(mul2(y, c_half), res, sq);
+            float t0, t1;
+            unpack2(add2(dist, c_r), t0, t1);
+            const f32x2 t = mul2(pack2(fmaxf(t0, 0.0f), fmaxf(t1, 0.0f)), c_t);
+            e = fma2(t, t, e);
+          }
+          float q0, q1, e0, e1;
+          unpack2(Q, q0, q1);
+          unpack2(e, e0, e1);
+          w[h] = pack2(ex2_approx(-(q0 <= a.cut2 ? e0 : INFINITY)),     // 2^-inf = +0
+                       ex2_approx(-(q1 <= a.cut2 ? e1 : INFINITY)));
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const ulonglong2 phi = field(12 + c);
+      L[c] = fma2(w[1], phi.y, fma2(w[0], phi.x, L[c]));
+    }
+    Z = add2(add2(Z, w[0]), w[1]);
   }
-  return ex2_approx(Q <= a.cut2 ? e : -INFINITY);             // 2^-inf = +0
 }
 
-// Every staged record of the cooperative mode at this lane's hit point, four
-// at a time as straight-line code. A group may reach past nk (never past the
-// 32 staged slots): those slots hold zeros or earlier finite records, and
-// their weight is forced to 0, so the sums are those of the first nk in order.
-template <int C, int KERN, bool COUNT>
-__device__ __forceinline__ void eval_staged(const float* __restrict__ recs, int nk, float px,
-                                            float py, float pz, const FwdArgs& a, float (&L)[C],
-                                            float& Z, uint32_t& n_eval, uint32_t& n_inc) {
-  constexpr int RS = rec_stride(C);
-  if (COUNT || KERN == kKernDisk) {
-    for (int s = 0; s < nk; ++s) eval_pair<C, KERN, COUNT>(recs + s * RS, px, py, pz, a, L, Z,
-                                                           n_eval, n_inc);
-    return;
-  }
-  constexpr int kGroup = 4;
-  for (int s = 0; s < nk; s += kGroup) {
-    float w[kGroup];
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const float wj = staged_weight<KERN>(recs + (s + j) * RS, px, py, pz, a);
-      w[j] = s + j < nk ? wj : 0.0f;
-    }
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const float* r = recs + (s + j) * RS;
-#pragma unroll
-      for (int c = 0; c < C; ++c) L[c] = fmaf(w[j], r[13 + c], L[c]);
-      Z += w[j];
-    }
+// The pairs that eval_staged would evaluate and include (count mode).
+template <int C>
+__device__ __forceinline__ void count_staged(const float* __restrict__ st, int nk, float px,
+                                             float py, float pz, const FwdArgs& a,
+                                             uint32_t& n_eval, uint32_t& n_inc) {
+  for (int s = 0; s < nk; ++s) {
+    auto f = [&](int k) { return st[k * kWarp + s]; };
+    const float dx = px + f(0), dy = py + f(1), dz = pz + f(2);
+    const float u0 = fmaf(f(3), dx, fmaf(f(4), dy, f(5) * dz));
+    const float u1 = fmaf(f(6), dx, fmaf(f(7), dy, f(8) * dz));
+    const float u2 = fmaf(f(9), dx, fmaf(f(10), dy, f(11) * dz));
+    ++n_eval;
+    n_inc += fmaf(u0, u0, fmaf(u1, u1, u2 * u2)) <= a.cut2 ? 1u : 0u;
   }
 }
 
@@ -240,54 +284,171 @@ __device__ __forceinline__ void pooled_flush(float (*acc)[kWarp], int lane, int 
   __syncwarp();
 }
 
+// A record, in 32-byte loads where its stride allows them: a gather is bound
+// by the lines its instructions touch, one per lane whatever the width.
 template <int RS>
 __device__ __forceinline__ void load_rec(const float* __restrict__ rec, uint32_t g, float (&r)[RS]) {
-  const float4* src = reinterpret_cast<const float4*>(rec + (int64_t)g * RS);
+  const float* src = rec + (int64_t)g * RS;
+  if constexpr (RS % 8 == 0) {
 #pragma unroll
-  for (int v = 0; v < RS / 4; ++v) {
-    const float4 t = __ldg(src + v);
-    r[4 * v] = t.x; r[4 * v + 1] = t.y; r[4 * v + 2] = t.z; r[4 * v + 3] = t.w;
+    for (int v = 0; v < RS; v += 8) ld_global_v8(src + v, r + v);
+  } else {
+#pragma unroll
+    for (int v = 0; v < RS / 4; ++v) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src) + v);
+      r[4 * v] = t.x; r[4 * v + 1] = t.y; r[4 * v + 2] = t.z; r[4 * v + 3] = t.w;
+    }
   }
 }
 
-// COUNT: count the evaluated and included pairs instead of summing radiance.
-// SPLIT: the index splits heavy tiles into parts (a separate instantiation,
-// so that an index without splitting runs the plain tile loop).
-template <int C, bool BRUTE, int KERN, bool COUNT, bool SPLIT>
-__global__ void __launch_bounds__(kFwdThreads, C <= 4 ? 6 : 5)
-fwd_kernel(FwdArgs a) {
-  constexpr int RS = rec_stride(C);
-  __shared__ __align__(16) float s_rec[kFwdWarps][kWarp * RS];
-  __shared__ unsigned long long s_cell[kFwdWarps][kUnionMax];
-  __shared__ int s_leader[kFwdWarps][kUnionMax];
-  __shared__ uint2 s_range[kFwdWarps][kMaxLevels][kWarp];
-  __shared__ float s_acc[kFwdWarps][C + 1][kWarp];  // pooled-mode sums per hit point
-  // the warp's work unit: its tile's part and number of parts (kept here, not
-  // in registers, which the pair loops need)
-  __shared__ uint32_t s_part[kFwdWarps], s_parts[kFwdWarps];
+// Its first eight values (mean, radius, the first of M), and the others.
+template <int RS>
+__device__ __forceinline__ void load_rec_head(const float* __restrict__ rec, uint32_t g,
+                                              float (&r)[RS]) {
+  const float* src = rec + (int64_t)g * RS;
+  if constexpr (RS % 8 == 0) {
+    ld_global_v8(src, r);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src) + v);
+      r[4 * v] = t.x; r[4 * v + 1] = t.y; r[4 * v + 2] = t.z; r[4 * v + 3] = t.w;
+    }
+  }
+}
+template <int RS>
+__device__ __forceinline__ void load_rec_tail(const float* __restrict__ rec, uint32_t g,
+                                              float (&r)[RS]) {
+  const float* src = rec + (int64_t)g * RS;
+  if constexpr (RS % 8 == 0) {
+#pragma unroll
+    for (int v = 8; v < RS; v += 8) ld_global_v8(src + v, r + v);
+  } else {
+#pragma unroll
+    for (int v = 2; v < RS / 4; ++v) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src) + v);
+      r[4 * v] = t.x; r[4 * v + 1] = t.y; r[4 * v + 2] = t.z; r[4 * v + 3] = t.w;
+    }
+  }
+}
 
+// The shared memory of a warp. Sizes follow the index: levels * coop segments
+// at most, levels ranges per lane.
+struct WarpShared {
+  float* stage;            // [max(rec stride, stage fields)][32]
+  float (*acc)[kWarp];     // [C + 1][32] pooled-mode sums per hit point
+  float4* box;             // [3] the tile's box: (lo, hi.x), (hi.yz, centre.xy),
+                           // (centre.z, half extents)
+  uint2* range;            // [levels][32]
+  unsigned long long* cell;  // [segments] pack_cell
+  uint32_t* start;         // first entry of a segment's list
+  uint32_t* incl;          // entries of the segments up to and with this one
+  uint32_t* tag;
+  uint32_t* lev;           // level | first segment of that level << 8
+  uint32_t* queue;         // [kQueue]
+};
+__host__ __device__ constexpr int stage_words(int C) {
+  return kWarp * (rec_stride(C) > stage_fields(C) ? rec_stride(C) : stage_fields(C));
+}
+__host__ __device__ constexpr int warp_shared_words(int C, int levels, int coop) {
+  // (the segments' count rounded up to even, for 16-byte pieces)
+  return stage_words(C) + (C + 1) * kWarp + 12 + 2 * levels * kWarp +
+         (levels * coop + 1) / 2 * 2 * 6 + kQueue;
+}
+template <int C>
+__device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int levels, int coop) {
+  const int segs = (levels * coop + 1) / 2 * 2;
+  float* p = base + wib * warp_shared_words(C, levels, coop);
+  WarpShared w;
+  w.stage = p;
+  p += stage_words(C);
+  w.acc = reinterpret_cast<float(*)[kWarp]>(p);
+  p += (C + 1) * kWarp;
+  w.box = reinterpret_cast<float4*>(p);
+  p += 12;
+  w.range = reinterpret_cast<uint2*>(p);
+  p += 2 * levels * kWarp;
+  w.cell = reinterpret_cast<unsigned long long*>(p);
+  p += 2 * segs;
+  w.start = reinterpret_cast<uint32_t*>(p);
+  w.incl = w.start + segs;
+  w.tag = w.incl + segs;
+  w.lev = w.tag + segs;
+  w.queue = w.lev + segs;
+  return w;
+}
+
+// As mahalanobis_lower_bound, with the hardware's approximate square roots
+// (2 ulp, well inside the margin of 4e-6).
+__device__ __forceinline__ float sqrt_approx(float v) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float box_distance(const float* M, float ex, float ey, float ez,
+                                              float hx, float hy, float hz) {
+  const float v0 = fmaf(M[0], ex, fmaf(M[1], ey, M[2] * ez));
+  const float v1 = fmaf(M[3], ex, fmaf(M[4], ey, M[5] * ez));
+  const float v2 = fmaf(M[6], ex, fmaf(M[7], ey, M[8] * ez));
+  const float s0 = fmaf(fabsf(M[0]), hx, fmaf(fabsf(M[1]), hy, fabsf(M[2]) * hz));
+  const float s1 = fmaf(fabsf(M[3]), hx, fmaf(fabsf(M[4]), hy, fabsf(M[5]) * hz));
+  const float s2 = fmaf(fabsf(M[6]), hx, fmaf(fabsf(M[7]), hy, fabsf(M[8]) * hz));
+  const float vn = sqrt_approx(fmaf(v0, v0, fmaf(v1, v1, v2 * v2)));
+  const float sn = sqrt_approx(fmaf(s0, s0, fmaf(s1, s1, s2 * s2)));
+  return (vn - sn) - 4e-6f * (vn + sn);
+}
+
+// What bounds it: issue and the latency of dependent gathers together (1M
+// Gaussians, one 1024 x 1024 view, ncu: 2.1 instructions a cycle and SM, 20
+// resident warps, long and short scoreboard the largest stalls, DRAM 5 %). So
+// the lists of a tile are walked as one stream of full chunks, whatever level
+// and cell they belong to, an entry is rejected on one 32-byte load, and only
+// survivors load their record; the same view took 433 M instructions and 620 us
+// with a chunk loop per cell and level, 327 M and 520 us so. 5 blocks of 4 warps
+// per SM: at 6 (80 registers) the spills cost 5 % more than the warps bring.
+// COUNT: count the evaluated and included pairs instead of summing radiance.
+// TEAM: warps of a block that share a tile, each taking every TEAM-th chunk of
+// its lists; their sums are added in order.
+template <int C, bool BRUTE, int KERN, bool COUNT, int TEAM>
+__global__ void __launch_bounds__(TEAM > 4 ? TEAM * kWarp : kFwdThreads,
+                                  TEAM > 4 ? 1 : C <= 4 ? 5 : 4)
+fwd_kernel(const __grid_constant__ FwdArgs a) {
+  constexpr int RS = rec_stride(C);
+  extern __shared__ __align__(16) float s_mem[];
+  __shared__ unsigned long long s_unit;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (index_unusable(a.header)) return;
+  const Grid& G = a.grid;
+  const WarpShared ws = warp_shared<C>(s_mem, wib, G.levels, G.coop);
   // the staged slots start finite: eval_staged reads whole groups of four
-  for (int i = lane; i < kWarp * RS; i += kWarp) s_rec[wib][i] = 0.0f;
+  for (int i = lane; i < stage_words(C); i += kWarp) ws.stage[i] = 0.0f;
   const int64_t n_act = a.header->n_active;
   const int64_t n_tiles = (a.m + kWarp - 1) / kWarp;
   // split tiles (heavy ones, when the index asks for it) come first as
   // n_x units, one per part; then every tile as one unit (a split tile's is
   // skipped)
-  const int64_t n_x = SPLIT ? (int64_t)a.header->n_xunits : 0;
+  const int64_t n_x = a.tparts ? (int64_t)a.header->n_xunits : 0;
+  const uint32_t lmask = a.header->level_mask;
   uint32_t n_eval = 0, n_inc = 0;
-  // persistent: every warp takes the next unit until none is left, so a
+  // persistent: every warp (team) takes the next unit until none is left, so a
   // warp that drew a light tile goes on with another one
   for (;;) {
-  __syncwarp();
-  unsigned long long unit_u = 0;
-  if (lane == 0) unit_u = atomicAdd(a.next_tile, 1ull);
-  const int64_t unit = (int64_t)__shfl_sync(kFullMask, unit_u, 0);
+  int64_t unit;
+  if (TEAM > 1) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_unit = atomicAdd(a.next_tile, 1ull);
+    __syncthreads();
+    unit = (int64_t)s_unit;
+  } else {
+    __syncwarp();
+    unsigned long long unit_u = 0;
+    if (lane == 0) unit_u = atomicAdd(a.next_tile, 1ull);
+    unit = (int64_t)__shfl_sync(kFullMask, unit_u, 0);
+  }
   if (unit >= n_x + n_tiles) break;
   int64_t tile;
   uint32_t part = 0, parts = 1;
-  if (SPLIT && unit < n_x) {
+  if (unit < n_x) {
     const uint4 xu = a.xunit[unit];
     if (!xu.w) continue;                      // a slot left over at the capacity edge
     tile = xu.x;
@@ -295,45 +456,47 @@ fwd_kernel(FwdArgs a) {
     parts = xu.z;
   } else {
     tile = unit - n_x;
-    if (SPLIT && n_x && a.tparts[tile] > 1) continue;  // done by its parts
+    if (n_x && a.tparts[tile] > 1) continue;  // done by its parts
   }
-  const bool split = SPLIT && parts > 1;
-  if (SPLIT && lane == 0) {
-    s_part[wib] = part;
-    s_parts[wib] = parts;
+  const bool split = parts > 1;
+  if (TEAM > 1) {
+    part = part * TEAM + wib;
+    parts *= TEAM;
   }
-  if (SPLIT) __syncwarp();
   const int64_t base = tile * kWarp;
   const int64_t k = base + lane;
   const bool in_range = k < a.m;
   const bool active = k < n_act;
-  const uint32_t q = in_range ? a.qval[k] : 0u;
-  if (!COUNT && !split && in_range && !active) {
+  if (!COUNT && !split && in_range && !active && (TEAM == 1 || wib == 0)) {
+    const uint32_t q = a.qval[k];
 #pragma unroll
     for (int c = 0; c < C; ++c) a.out[(int64_t)c * a.m + q] = 0.0f;
     if (a.z) a.z[q] = 0.0f;
   }
-  if (base >= n_act) continue;  // warp-uniform (never a split tile)
-  uint32_t gchunk = 0;  // chunks of this tile's lists seen so far, all levels and modes
+  if (base >= n_act) continue;  // the whole warp or team (never a split tile)
 
   float px = 0.f, py = 0.f, pz = 0.f;
+  uint32_t q = 0;
   if (active) {
     const float4 p = __ldg(a.qpos + k);
     px = p.x;
     py = p.y;
     pz = p.z;
+    q = __float_as_uint(p.w);
   }
-  float L[C];
+  f32x2 L2[C], Z2 = 0;
 #pragma unroll
-  for (int c = 0; c < C; ++c) L[c] = 0.0f;
-  float Z = 0.0f;
-  float* my_rec = s_rec[wib];
+  for (int c = 0; c < C; ++c) L2[c] = 0;
 #pragma unroll
-  for (int c = 0; c <= C; ++c) s_acc[wib][c][lane] = 0.0f;
+  for (int c = 0; c <= C; ++c) ws.acc[c][lane] = 0.0f;
   __syncwarp();
 
   if (BRUTE) {
-    for (int64_t g0 = 0; g0 < a.n; g0 += kWarp) {
+    float L[C], Z = 0.0f;
+#pragma unroll
+    for (int c = 0; c < C; ++c) L[c] = 0.0f;
+    float* my_rec = ws.stage;
+    for (int64_t g0 = (int64_t)part * kWarp; g0 < a.n; g0 += (int64_t)parts * kWarp) {
       const int64_t g = g0 + lane;
       const int cnt = (int)min((int64_t)kWarp, a.n - g0);
       if (g < a.n) {
@@ -348,225 +511,344 @@ fwd_kernel(FwdArgs a) {
           eval_pair<C, KERN, COUNT>(my_rec + s * RS, px, py, pz, a, L, Z, n_eval, n_inc);
       __syncwarp();
     }
+#pragma unroll
+    for (int c = 0; c < C; ++c) L2[c] = pack2(L[c], 0.0f);
+    Z2 = pack2(Z, 0.0f);
   } else {
-    const Grid& G = a.grid;
     const uint32_t c0x = coord0(px, G.ox, G.inv_cell0, G.max0x);
     const uint32_t c0y = coord0(py, G.oy, G.inv_cell0, G.max0y);
     const uint32_t c0z = coord0(pz, G.oz, G.inv_cell0, G.max0z);
+    // the lane's list on every used level: first the bits of all levels, then
+    // the ranges of those that have one
+    {
+      uint32_t bkt[kMaxLevels], word[kMaxLevels];
+#pragma unroll
+      for (int lev = 0; lev < kMaxLevels; ++lev) {
+        word[lev] = 0;
+        if (lev < G.levels && ((lmask >> lev) & 1u) && active) {
+          bkt[lev] = bucket_of(G, lev, c0x >> lev, c0y >> lev, c0z >> lev);
+          word[lev] = __ldg(a.listed + (bkt[lev] >> 5));
+        }
+      }
+#pragma unroll
+      for (int lev = 0; lev < kMaxLevels; ++lev) {
+        if (lev < G.levels && ((lmask >> lev) & 1u)) {
+          uint2 rg = make_uint2(0u, 0u);
+          if (active && ((word[lev] >> (bkt[lev] & 31u)) & 1u)) rg = __ldg(a.brange + bkt[lev]);
+          ws.range[lev * kWarp + lane] = rg;
+        }
+      }
+    }
     // tile box of the active hit points
     const float bx0 = warp_min(active ? px : INFINITY), bx1 = warp_max(active ? px : -INFINITY);
     const float by0 = warp_min(active ? py : INFINITY), by1 = warp_max(active ? py : -INFINITY);
     const float bz0 = warp_min(active ? pz : INFINITY), bz1 = warp_max(active ? pz : -INFINITY);
-    const float cx = 0.5f * (bx0 + bx1), cy = 0.5f * (by0 + by1), cz = 0.5f * (bz0 + bz1);
-    const float hx = 0.5f * (bx1 - bx0), hy = 0.5f * (by1 - by0), hz = 0.5f * (bz1 - bz0);
-    const float cut_keep = a.cut * 1.0001f;
-    const uint32_t lmask = a.header->level_mask;
-    // the lane's bucket range on every used level, all looked up at once
-#pragma unroll
-    for (int lev = 0; lev < kMaxLevels; ++lev) {
-      if (lev < G.levels && ((lmask >> lev) & 1u)) {
-        uint2 rg = make_uint2(0u, 0u);
-        if (active)
-          rg = bucket_list(a.listed, a.brange, bucket_of(G, lev, c0x >> lev, c0y >> lev, c0z >> lev));
-        s_range[wib][lev][lane] = rg;
-      }
+    if (lane == 0) {         // in shared memory: the evaluation needs the registers
+      ws.box[0] = make_float4(bx0, by0, bz0, bx1);
+      ws.box[1] = make_float4(by1, bz1, 0.5f * (bx0 + bx1), 0.5f * (by0 + by1));
+      ws.box[2] = make_float4(0.5f * (bz0 + bz1), 0.5f * (bx1 - bx0), 0.5f * (by1 - by0),
+                              0.5f * (bz1 - bz0));
     }
     __syncwarp();
 
+    // ---- walked levels: their distinct cells' lists as segments, end to end;
+    // pooled levels: each lane's lists end to end (range[p] of the p-th pooled
+    // level becomes (first entry - items before, items up to and with it))
+    int n_seg = 0, n_pool = 0;
+    uint32_t total = 0;                     // entries of the segments
+    uint32_t len = 0;                       // this lane's pooled items
+    unsigned long long pool_levels = 0;     // 4 bits per pooled level
     for (int lev = 0; lev < G.levels; ++lev) {
       if (!((lmask >> lev) & 1u)) continue;
       const uint32_t lx = c0x >> lev, ly = c0y >> lev, lz = c0z >> lev;
-      const unsigned long long packed =
-          active ? ((unsigned long long)lx | ((unsigned long long)ly << 20) |
-                    ((unsigned long long)lz << 40))
-                 : ~0ull;
+      const unsigned long long packed = active ? pack_cell(lx, ly, lz) : ~0ull;
       const uint32_t peers = __match_any_sync(kFullMask, packed);
       const bool leader = active && (peers & lanemask_lt()) == 0;
       const uint32_t uniq = __ballot_sync(kFullMask, leader);
       const int nu = __popc(uniq);
+      const uint2 rg = ws.range[lev * kWarp + lane];    // (0, 0) for inactive lanes
       if (nu <= G.coop) {
-        // ---- warp-cooperative mode over the tile's distinct cells
-        if (leader) {
-          const int slot = __popc(uniq & lanemask_lt());
-          s_cell[wib][slot] = packed;
-          s_leader[wib][slot] = lane;
-        }
-        __syncwarp();
-        for (int j = 0; j < nu; ++j) {
-          const unsigned long long cj = s_cell[wib][j];
-          const uint32_t ux = (uint32_t)(cj & kCoordMax), uy = (uint32_t)((cj >> 20) & kCoordMax),
-                         uz = (uint32_t)((cj >> 40) & kCoordMax);
-          const uint32_t tag = cell_hash(G, lev, ux, uy, uz).tag;
-          const uint2 rg = s_range[wib][lev][s_leader[wib][j]];
-          // chunks of 32 entries; a split tile's part takes every parts-th
-          // chunk of the tile's lists. The entry words of the next chunk are
-          // fetched while the current one is being vetted.
-          const uint32_t parts_ = SPLIT ? s_parts[wib] : 1u;
-          uint32_t c_first = 0;
-          if (SPLIT && parts_ > 1) {     // warp-uniform: only for split tiles
-            c_first = (s_part[wib] + parts_ - gchunk % parts_) % parts_;
-            gchunk += (rg.y - rg.x + kWarp - 1) / kWarp;
-          }
-          const uint32_t step = parts_ * kWarp;
-          uint32_t e_first = rg.x + c_first * kWarp;
-          uint32_t v = e_first + lane < rg.y ? __ldg(a.gval + e_first + lane) : 0u;
-          uint32_t carry = 0xffffffffu;
-          for (uint32_t e0 = e_first; e0 < rg.y; e0 += step) {
-            const uint32_t e = e0 + lane;
-            const uint32_t vn = e + step < rg.y ? __ldg(a.gval + e + step) : 0u;
-            // a Gaussian listed twice in a bucket sits on consecutive entries
-            uint32_t vprev = __shfl_up_sync(kFullMask, v, 1);
-            if (lane == 0)
-              vprev = parts_ == 1 ? carry : e0 > rg.x ? __ldg(a.gval + e0 - 1) : 0xffffffffu;
-            carry = __shfl_sync(kFullMask, v, kWarp - 1);
-            bool keep = e < rg.y && (v & ~G.id_mask) == tag && v != vprev;
-            const uint32_t g = v & G.id_mask;
-            float rr[RS];
-            if (keep) {
-              const uint4 bw = __ldg(a.box + g);
-              load_rec<RS>(a.rec, g, rr);
-              const LevelBox b = unpack_box(bw);
-              // it must live on this level and cover this cell, and must not
-              // have been taken from an earlier cell of this tile
-              keep = b.level == lev && box_holds(b, ux, uy, uz);
-              for (int jj = 0; jj < j && keep; ++jj) {
-                const unsigned long long ci = s_cell[wib][jj];
-                keep = !box_holds(b, (uint32_t)(ci & kCoordMax), (uint32_t)((ci >> 20) & kCoordMax),
-                                  (uint32_t)((ci >> 40) & kCoordMax));
-              }
-              if (keep) {
-                // sphere test: distance from mu to the tile box vs k * max s
-                const float ex = fmaxf(fmaxf(bx0 - rr[0], rr[0] - bx1), 0.0f);
-                const float ey = fmaxf(fmaxf(by0 - rr[1], rr[1] - by1), 0.0f);
-                const float ez = fmaxf(fmaxf(bz0 - rr[2], rr[2] - bz1), 0.0f);
-                keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= rr[3] * rr[3];
-              }
-              if (keep)
-                keep = mahalanobis_lower_bound(rr + 4, rr[0], rr[1], rr[2], cx, cy, cz, hx, hy, hz) <=
-                       cut_keep;
-            }
-            const uint32_t kb = __ballot_sync(kFullMask, keep);
-            if (keep) {
-              float4* dst = reinterpret_cast<float4*>(my_rec + __popc(kb & lanemask_lt()) * RS);
-#pragma unroll
-              for (int q4 = 0; q4 < RS / 4; ++q4)
-                dst[q4] = make_float4(rr[4 * q4], rr[4 * q4 + 1], rr[4 * q4 + 2], rr[4 * q4 + 3]);
-            }
-            __syncwarp();
-            const int nk = __popc(kb);
-            if (active) eval_staged<C, KERN, COUNT>(my_rec, nk, px, py, pz, a, L, Z, n_eval, n_inc);
-            __syncwarp();
-            v = vn;
-          }
-        }
-      } else {
-        // ---- pooled mode: the lanes' lists are laid end to end and the warp
-        // takes them 32 (hit point, entry) items at a time, one item per lane.
-        // A lane sums what it evaluates for one owner at a time and hands the
-        // sum over (pooled_flush) when the owner of its item slot changes, so
-        // no lane waits for the longest list and every sum has a fixed order.
-        // The cell-box test is not needed here: an entry that reached this
-        // bucket from another cell on the same level has a box that misses
-        // this hit point, so Q > k^2 rejects it; the level test and the
-        // duplicate test keep any Gaussian from being counted twice.
-        const uint32_t tag = cell_hash(G, lev, lx, ly, lz).tag;
-        const uint2 rg = s_range[wib][lev][lane];  // (0, 0) for inactive lanes
-        const uint32_t len = rg.y - rg.x;
-        uint32_t incl = len;  // inclusive prefix sum of the list lengths
+        // (a cell without a list holds no Gaussian that another cell repeats)
+        const bool has = leader && rg.y > rg.x;
+        const uint32_t hm = __ballot_sync(kFullMask, has);
+        uint32_t incl = has ? rg.y - rg.x : 0u;
 #pragma unroll
         for (int o = 1; o < kWarp; o <<= 1) {
           const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
           if (lane >= o) incl += t;
         }
-        const uint32_t total = __shfl_sync(kFullMask, incl, kWarp - 1);
-        int cur = -1;  // owner of this lane's item slot in the previous chunk
-        float pc[C + 1];
-#pragma unroll
-        for (int c = 0; c <= C; ++c) pc[c] = 0.0f;
-        uint32_t o_first = 0, o_start = 0, o_tag = 0;
-        float qx = 0.0f, qy = 0.0f, qz = 0.0f;
-        uint32_t carry = 0xffffffffu;
-        // owner of item i: the first lane whose inclusive end exceeds i
-        // (kWarp: none); the entry word of the next chunk is fetched while
-        // the current chunk is evaluated
-        auto owner_of = [&](uint32_t i) {
-          int o = 0;
-#pragma unroll
-          for (int st = 16; st > 0; st >>= 1) {
-            const uint32_t pe = __shfl_sync(kFullMask, incl, o + st - 1);
-            if (pe <= i) o += st;
-          }
-          return i < total ? o : kWarp;
-        };
-        auto entry_of = [&](uint32_t i, int o) {
-          const int src = o & (kWarp - 1);
-          const uint32_t first = __shfl_sync(kFullMask, incl - len, src);
-          const uint32_t start = __shfl_sync(kFullMask, rg.x, src);
-          return i < total ? __ldg(a.gval + start + (i - first)) : 0u;
-        };
-        // a split tile's part takes every parts-th chunk of 32 items
-        const uint32_t parts_ = SPLIT ? s_parts[wib] : 1u;
-        uint32_t c_first = 0;
-        if (SPLIT && parts_ > 1) {
-          c_first = (s_part[wib] + parts_ - gchunk % parts_) % parts_;
-          gchunk += (total + kWarp - 1) / kWarp;
+        if (has) {
+          const int slot = n_seg + __popc(hm & lanemask_lt());
+          ws.cell[slot] = packed;
+          ws.start[slot] = rg.x;
+          ws.incl[slot] = total + incl;
+          ws.tag[slot] = cell_hash(G, lev, lx, ly, lz).tag;
+          ws.lev[slot] = (uint32_t)lev | ((uint32_t)n_seg << 8);
         }
-        const uint32_t step = parts_ * kWarp;
-        const uint32_t b_first = c_first * kWarp;
-        int own_n = owner_of(b_first + lane);
-        uint32_t v_n = entry_of(b_first + lane, own_n);
-        for (uint32_t b = b_first; b < total; b += step) {
-          const uint32_t i = b + lane;
-          const bool live = i < total;
-          const int own = own_n;
+        n_seg += __popc(hm);
+        total += __shfl_sync(kFullMask, incl, kWarp - 1);
+      } else {
+        // (slot n_pool <= lev: the ranges of this and later levels are read first)
+        ws.range[n_pool * kWarp + lane] = make_uint2(rg.x - len, len + (rg.y - rg.x));
+        len += rg.y - rg.x;
+        pool_levels |= (unsigned long long)lev << (4 * n_pool);
+        ++n_pool;
+      }
+    }
+    __syncwarp();
+
+    // a split tile's part, and a team's warp, take every parts-th chunk of 32
+    // entries, then of 32 items
+    const uint32_t n_chunks = (total + kWarp - 1) / kWarp;
+    if (n_chunks > 0) {
+      const float cut_keep = a.cut * 1.0001f;
+      int top = 1;                          // the segment search's first step
+      while (2 * top < n_seg) top *= 2;
+      // up to 32 segments (none is empty): lane l keeps where the l-th begins, and
+      // a chunk's segments follow from the beginnings inside it, without a search
+      const bool few = n_seg <= kWarp;
+      const uint32_t seg_at =
+          few && lane < n_seg ? (lane > 0 ? ws.incl[lane - 1] : 0u) : 0xffffffffu;
+      const uint32_t le = lanemask_lt() | (1u << lane);
+      // entry e of the stream: its segment (the first whose inclusive count
+      // exceeds e) and entry word, with the previous word of its list
+      auto fetch = [&](uint32_t chunk, int& seg, uint32_t& v, uint32_t& vprev, bool& first) {
+        const uint32_t e = chunk * kWarp + lane;
+        seg = 0;
+        v = vprev = 0u;
+        first = true;
+        if (few) {
+          const uint32_t c0 = chunk * kWarp;
+          const uint32_t inside = __reduce_or_sync(
+              kFullMask, seg_at > c0 && seg_at - c0 < kWarp ? 1u << (seg_at - c0) : 0u);
+          seg = __popc(__ballot_sync(kFullMask, seg_at <= c0)) - 1 + __popc(inside & le);
+        }
+        if (e < total) {
+          if (!few)
+            for (int st = top; st > 0; st >>= 1)
+              if (seg + st <= n_seg - 1 && ws.incl[seg + st - 1] <= e) seg += st;
+          const uint32_t before = seg ? ws.incl[seg - 1] : 0u;
+          const uint32_t* p = a.gval + ws.start[seg] + (e - before);
+          v = __ldg(p);
+          first = e == before;               // of its list
+          if (!first && lane == 0) vprev = __ldg(p - 1);   // (else the lane to the left has it)
+        }
+      };
+      uint32_t chunk = part;
+      int qn = 0;                            // queued ids
+      for (;;) {
+        // vet entries until the queue may overflow; the entry words of the
+        // next chunk are fetched while one is vetted
+        int seg_n;
+        uint32_t v_n, vp_n;
+        bool first_n;
+        fetch(chunk, seg_n, v_n, vp_n, first_n);
+        while (chunk < n_chunks && qn <= kQueue - kWarp) {
+          const int seg = seg_n;
           const uint32_t v = v_n;
-          own_n = owner_of(i + step);
-          v_n = entry_of(i + step, own_n);
-          const bool chg = own != cur;
-          if (__any_sync(kFullMask, chg)) {
-            pooled_flush<C>(s_acc[wib], lane, cur, chg && cur >= 0 && cur < kWarp, pc);
-            const int src = own & (kWarp - 1);
-            o_first = __shfl_sync(kFullMask, incl - len, src);
-            o_start = __shfl_sync(kFullMask, rg.x, src);
-            o_tag = __shfl_sync(kFullMask, tag, src);
-            qx = __shfl_sync(kFullMask, px, src);
-            qy = __shfl_sync(kFullMask, py, src);
-            qz = __shfl_sync(kFullMask, pz, src);
-            cur = own;
+          const bool live = chunk * kWarp + lane < total;
+          const uint32_t left = __shfl_up_sync(kFullMask, v, 1);
+          // a Gaussian listed twice in a bucket sits on consecutive entries
+          const bool again = !first_n && v == (lane == 0 ? vp_n : left);
+          bool keep = live && (v & ~G.id_mask) == ws.tag[seg] && !again;
+          const uint32_t g = v & G.id_mask;
+          VetRec r;
+          if (keep) r = load_vet(a.vet + g);
+          chunk += parts;
+          fetch(chunk, seg_n, v_n, vp_n, first_n);
+          if (keep) {
+            // sphere test: distance from mu to the tile box vs k * max s
+            const float4 b0 = ws.box[0], b1 = ws.box[1];
+            const float ex = fmaxf(fmaxf(b0.x - r.x, r.x - b0.w), 0.0f);
+            const float ey = fmaxf(fmaxf(b0.y - r.y, r.y - b1.x), 0.0f);
+            const float ez = fmaxf(fmaxf(b0.z - r.z, r.z - b1.y), 0.0f);
+            const uint32_t sl = ws.lev[seg];
+            // it must live on this level and cover this cell, and must not
+            // have been taken from an earlier cell of this tile
+            keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= r.radius * r.radius &&
+                   rec_level(r.radius) == (sl & 0xffu) && cell_in(r, ws.cell[seg]);
+            for (int j = (int)(sl >> 8); j < seg && keep; ++j) keep = !cell_in(r, ws.cell[j]);
           }
-          const uint32_t kk = i - o_first;  // position in the owner's list
-          // the owner's previous entry is the previous item
-          uint32_t vprev = __shfl_up_sync(kFullMask, v, 1);
-          if (lane == 0)
-            vprev = parts_ == 1 ? carry
-                                : live && kk > 0 ? __ldg(a.gval + o_start + kk - 1) : 0xffffffffu;
-          carry = __shfl_sync(kFullMask, v, kWarp - 1);
-          if (live && (v & ~G.id_mask) == o_tag && !(kk > 0 && v == vprev)) {
-            float rr[RS];
-            load_rec<RS>(a.rec, v & G.id_mask, rr);
-            if (rec_level(rr[3]) == (uint32_t)lev) {
-              bool hit;
-              const float w = pair_weight<KERN, COUNT>(rr, qx, qy, qz, a, hit, n_eval, n_inc);
-              if (hit) {
-#pragma unroll
-                for (int c = 0; c < C; ++c) pc[c] = fmaf(w, rr[13 + c], pc[c]);
-                pc[C] += w;
-              }
+          const uint32_t kb = __ballot_sync(kFullMask, keep);
+          if (keep) ws.queue[qn + __popc(kb & lanemask_lt())] = g;
+          qn += __popc(kb);
+        }
+        __syncwarp();
+        const bool done = chunk >= n_chunks;
+        const int take = done ? qn : qn & ~(kWarp - 1);
+        for (int i = 0; i < take; i += kWarp) {
+          bool keep = i + lane < take;
+          float rr[RS];
+          if (keep) {
+            load_rec<RS>(a.rec, ws.queue[i + lane], rr);
+            if (KERN != kKernDisk) {
+              const float4 b1 = ws.box[1], b2 = ws.box[2];
+              keep = box_distance(rr + 4, b1.z - rr[0], b1.w - rr[1], b2.x - rr[2], b2.y, b2.z,
+                                  b2.w) <= cut_keep;
             }
           }
+          const uint32_t kb = __ballot_sync(kFullMask, keep);
+          const int nk = __popc(kb);
+          if (keep) {
+            float* d = ws.stage + __popc(kb & lanemask_lt());
+#pragma unroll
+            for (int f = 0; f < 3; ++f) d[f * kWarp] = -rr[f];
+#pragma unroll
+            for (int f = 0; f < 9 + C; ++f) d[(3 + f) * kWarp] = rr[4 + f];
+          } else if (nk + __popc(~kb & lanemask_lt()) < ((nk + 3) & ~3)) {
+            ws.stage[nk + __popc(~kb & lanemask_lt())] = NAN;    // fills the last group of four
+          }
+          __syncwarp();
+          if (COUNT) {
+            if (active) count_staged<C>(ws.stage, nk, px, py, pz, a, n_eval, n_inc);
+          } else {
+            eval_staged<C, KERN>(ws.stage, nk, px, py, pz, a, L2, Z2);
+          }
+          __syncwarp();
         }
-        pooled_flush<C>(s_acc[wib], lane, cur, cur >= 0 && cur < kWarp, pc);
+        if (done) break;
+        // the rest of the queue moves to its front
+        const uint32_t rest = take + lane < qn ? ws.queue[take + lane] : 0u;
+        __syncwarp();
+        qn -= take;
+        if (lane < qn) ws.queue[lane] = rest;
+        __syncwarp();
       }
+    }
+
+    // ---- pooled levels: 32 (hit point, entry) items at a time, one per lane.
+    // A lane sums what it evaluates for one owner at a time and hands the
+    // sum over (pooled_flush) when the owner of its item slot changes, so
+    // no lane waits for the longest list and every sum has a fixed order.
+    // The cell-box test is not needed here: an entry that reached this
+    // bucket from another cell on the same level has a box that misses
+    // this hit point, so Q > k^2 rejects it; the level test and the
+    // duplicate test keep any Gaussian from being counted twice.
+    if (n_pool > 0) {
+      uint32_t incl = len;  // inclusive prefix sum of the lanes' items
+#pragma unroll
+      for (int o = 1; o < kWarp; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const uint32_t items = __shfl_sync(kFullMask, incl, kWarp - 1);
+      // the lanes that have items, in order: (lane, first item); the owners of a
+      // chunk follow from the first items inside it
+      const uint32_t has = __ballot_sync(kFullMask, len > 0u);
+      const uint32_t own_at = len > 0u ? incl - len : 0xffffffffu;
+      uint2* owners = reinterpret_cast<uint2*>(ws.queue);
+      if (len > 0u)
+        owners[__popc(has & lanemask_lt())] = make_uint2((uint32_t)lane, incl - len);
+      __syncwarp();
+      const uint32_t le = lanemask_lt() | (1u << lane);
+      // item i: its owner (the first lane whose inclusive end exceeds i; kWarp:
+      // none), level, entry word and the previous word of its list
+      auto fetch = [&](uint32_t i, int& own, int& lev, uint32_t& v, uint32_t& vprev, bool& first) {
+        const uint32_t i0 = i - lane;
+        const uint32_t inside = __reduce_or_sync(
+            kFullMask, own_at > i0 && own_at - i0 < kWarp ? 1u << (own_at - i0) : 0u);
+        const uint32_t begun = __ballot_sync(kFullMask, own_at <= i0);
+        own = kWarp;
+        lev = 0;
+        v = vprev = 0u;
+        first = true;
+        if (i < items) {
+          const uint2 ow = owners[__popc(begun) - 1 + __popc(inside & le)];
+          const uint32_t o = ow.x, kk = i - ow.y;
+          own = (int)o;
+          uint32_t before = 0;
+          int p = 0;
+          uint2 rg = ws.range[o];
+          while (rg.y <= kk) {
+            before = rg.y;
+            ++p;
+            rg = ws.range[p * kWarp + o];
+          }
+          lev = (int)((pool_levels >> (4 * p)) & 15u);
+          const uint32_t at = rg.x + kk;               // modulo 2^32
+          v = __ldg(a.gval + at);
+          first = kk == before;
+          if (!first && lane == 0) vprev = __ldg(a.gval + (at - 1u));
+        }
+      };
+      int cur = -1;  // owner of this lane's item slot in the previous chunk
+      float pc[C + 1];
+#pragma unroll
+      for (int c = 0; c <= C; ++c) pc[c] = 0.0f;
+      float qx = 0.0f, qy = 0.0f, qz = 0.0f;
+      const uint32_t step = parts * kWarp;
+      uint32_t b = (part + parts - n_chunks % parts) % parts * kWarp;
+      int own_n, lev_n;
+      uint32_t v_n, vp_n;
+      bool first_n;
+      fetch(b + lane, own_n, lev_n, v_n, vp_n, first_n);
+      for (; b < items; b += step) {
+        const int own = own_n, lev = lev_n;
+        const uint32_t v = v_n;
+        const uint32_t left = __shfl_up_sync(kFullMask, v, 1);
+        // (by id: entries of two cells in one bucket may differ in their tags)
+        const bool again = !first_n && ((v ^ (lane == 0 ? vp_n : left)) & G.id_mask) == 0u;
+        const bool take = own < kWarp && !again;
+        float rr[RS];
+        if (take) load_rec_head<RS>(a.rec, v & G.id_mask, rr);
+        fetch(b + step + lane, own_n, lev_n, v_n, vp_n, first_n);
+        const bool chg = own != cur;
+        if (__any_sync(kFullMask, chg)) {
+          pooled_flush<C>(ws.acc, lane, cur, chg && cur >= 0 && cur < kWarp, pc);
+          const int src = own & (kWarp - 1);
+          qx = __shfl_sync(kFullMask, px, src);
+          qy = __shfl_sync(kFullMask, py, src);
+          qz = __shfl_sync(kFullMask, pz, src);
+          cur = own;
+        }
+        // the rest of the record only where its bounding sphere holds the point
+        bool near = take && rec_level(rr[3]) == (uint32_t)lev;
+        if (near) {
+          const float dx = qx - rr[0], dy = qy - rr[1], dz = qz - rr[2];
+          near = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= rr[3] * rr[3];
+        }
+        if (near) {
+          load_rec_tail<RS>(a.rec, v & G.id_mask, rr);
+          bool hit;
+          const float w = pair_weight<KERN, COUNT>(rr, qx, qy, qz, a, hit, n_eval, n_inc);
+          if (hit) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) pc[c] = fmaf(w, rr[13 + c], pc[c]);
+            pc[C] += w;
+          }
+        }
+      }
+      pooled_flush<C>(ws.acc, lane, cur, cur >= 0 && cur < kWarp, pc);
     }
   }
 
   if (!COUNT) {
-    // the pooled-mode sums of this lane's hit point
+    // the staged sums and the pooled sums of this lane's hit point
     __syncwarp();
+    float L[C], Z;
 #pragma unroll
-    for (int c = 0; c < C; ++c) L[c] += s_acc[wib][c][lane];
-    Z += s_acc[wib][C][lane];
-    if (SPLIT && s_parts[wib] > 1) {
+    for (int c = 0; c <= C; ++c) {
+      float lo, hi;
+      unpack2(c < C ? L2[c < C ? c : 0] : Z2, lo, hi);
+      const float s = (lo + hi) + ws.acc[c][lane];
+      if (c < C) L[c < C ? c : 0] = s;
+      else Z = s;
+    }
+    if (TEAM > 1) {
+      // the team's sums, added in warp order by warp 0
+#pragma unroll
+      for (int c = 0; c < C; ++c) ws.acc[c][lane] = L[c];
+      ws.acc[C][lane] = Z;
+      __syncthreads();
+      if (wib > 0) continue;
+      for (int w = 1; w < TEAM; ++w) {
+        const WarpShared o = warp_shared<C>(s_mem, w, G.levels, G.coop);
+#pragma unroll
+        for (int c = 0; c < C; ++c) L[c] += o.acc[c][lane];
+        Z += o.acc[C][lane];
+      }
+    }
+    if (split) {
       // this part's sums; fwd_split_combine_kernel adds the parts in order
       float* xs = a.xsum + (size_t)unit * (C + 1) * kWarp;
 #pragma unroll
@@ -612,6 +894,7 @@ __global__ void fwd_split_combine_kernel(FwdArgs a) {
   float L[C], Z = 0.0f;
 #pragma unroll
   for (int c = 0; c < C; ++c) L[c] = 0.0f;
+#pragma unroll 4
   for (uint32_t p = 0; p < xu.z; ++p) {
     const float* xs = a.xsum + (size_t)(u + p) * (C + 1) * kWarp;
 #pragma unroll
@@ -634,16 +917,20 @@ __global__ void fwd_split_combine_kernel(FwdArgs a) {
 
 // Estimated work of every tile of 32 hit points, from a sample of eight of its
 // points (every fourth: neighbouring points of the cell order see similar
-// lists), on every used level: where the sample falls in at most
-// Grid::coop cells, the distinct cells' lists, counted 8 times for the
-// staged evaluation of their survivors by the whole warp; else the points'
-// own lists, counted 4 times for the points not sampled. Then the tile's
-// number of parts. Four tiles per warp, eight lanes each.
+// lists), on every used level: where the sample falls in at most Grid::coop
+// cells, the distinct cells' lists, walked by the whole warp; else the points'
+// own lists, and four times as many for the points not sampled. 32 entries of
+// either kind cost a warp about the same (a least-squares fit over the units of
+// a 1M-Gaussian view: 1.5 us per 32 walked, 1.6 us per 32 pooled entries, and
+// 17 us a unit; weighting the pooled ones an eighth left single units of up to
+// 690 us at the end of a 1.8 ms forward). And the sum over all tiles. Four tiles
+// per warp, eight lanes each.
+constexpr uint32_t kCostPerEntry = 8, kCostPerTile = 8 * 32 * 10;
 __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
                                  const float4* __restrict__ qpos, int64_t m,
                                  const uint2* __restrict__ brange,
-                                 const uint32_t* __restrict__ listed, int split_items,
-                                 uint32_t* __restrict__ tparts, uint32_t* __restrict__ xpart) {
+                                 const uint32_t* __restrict__ listed,
+                                 uint32_t* __restrict__ tcost, unsigned long long* total) {
   const int lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t tile = gt >> 3;
@@ -680,20 +967,67 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
     const int nu = __popc(__ballot_sync(kFullMask, leader) & group);
     const uint32_t len = rg[lev].y - rg[lev].x;
     // (eight samples see at most 8 cells: all 8 distinct reads as more than 8)
-    cost += nu <= min(grid.coop, 7) ? (leader ? 8u * len : 0u) : 4u * len;
+    cost += kCostPerEntry * (nu <= min(grid.coop, 7) ? (leader ? len : 0u) : 4u * len);
   }
   // the eight lanes of a tile are consecutive: sum them
   cost += __shfl_xor_sync(kFullMask, cost, 1);
   cost += __shfl_xor_sync(kFullMask, cost, 2);
   cost += __shfl_xor_sync(kFullMask, cost, 4);
-  if ((lane & 7) == 0 && tile < n_tiles) {
-    uint32_t parts = 1;
-    if (cost > (uint32_t)split_items)
-      parts = min((cost + (uint32_t)split_items - 1) / (uint32_t)split_items,
-                  (uint32_t)GPF_MAX_TILE_PARTS);
-    tparts[tile] = parts;
-    if (parts > 1) atomicAdd(&xpart[tile / kTileGroup], parts);
+  if (tile < n_tiles && tile * kWarp < n_act) cost += kCostPerTile;
+  if ((lane & 7) == 0 && tile < n_tiles) tcost[tile] = cost;
+  __shared__ uint32_t s_sum;
+  if (threadIdx.x == 0) s_sum = 0;
+  __syncthreads();
+  const uint32_t sum = __reduce_add_sync(kFullMask, (lane & 7) == 0 ? min(cost, 1u << 26) : 0u);
+  if (lane == 0 && sum) atomicAdd(&s_sum, sum);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_sum) atomicAdd(total, (unsigned long long)s_sum);
+}
+
+// Parts of every tile from its cost, and the split units. A tile is split when
+// its cost exceeds both split_items and 1 / kSplitShare of all tiles' (a
+// quarter of what a resident warp has to do anyway: splitting the ordinary
+// tiles of a large batch only repeats their lookups; 22 K tiles of a 1M field
+// were 35 K units). The second bound also keeps the units below
+// GPF_MAX_SPLIT_UNITS: a split tile has at most 2 cost / bound parts. Which
+// slots a tile's units get depends on the order of the blocks; its sums do not.
+constexpr uint32_t kSplitShare = 152 * 24 * 4;
+static_assert(2 * kSplitShare <= GPF_MAX_SPLIT_UNITS, "room for every split unit");
+__global__ void __launch_bounds__(kTileGroup)
+tile_parts_kernel(int64_t n_tiles, int split_items, uint32_t* __restrict__ tparts,
+                  const unsigned long long* total, uint4* __restrict__ xunit,
+                  uint32_t* n_units) {
+  __shared__ uint32_t s_warp[kTileGroup / kWarp], s_first;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * kTileGroup + threadIdx.x;
+  const unsigned long long bound =
+      max((unsigned long long)split_items, *total / kSplitShare + 1ull);
+  uint32_t parts = 1;
+  if (t < n_tiles) {
+    const unsigned long long cost = min(tparts[t], 1u << 26);     // as summed
+    if (cost > bound)
+      parts = (uint32_t)min((cost + bound - 1) / bound, (unsigned long long)GPF_MAX_TILE_PARTS);
+    tparts[t] = parts;
   }
+  uint32_t incl = parts > 1 ? parts : 0u;
+#pragma unroll
+  for (int o = 1; o < kWarp; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(kFullMask, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == kWarp - 1) s_warp[warp] = incl;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t sum = 0;
+    for (int w = 0; w < kTileGroup / kWarp; ++w) sum += s_warp[w];
+    s_first = sum ? atomicAdd(n_units, sum) : 0u;
+  }
+  __syncthreads();
+  if (parts <= 1) return;
+  uint32_t o = s_first + incl - parts;
+  for (int w = 0; w < warp; ++w) o += s_warp[w];
+  for (uint32_t p = 0; p < parts && o + p < (uint32_t)GPF_MAX_SPLIT_UNITS; ++p)
+    xunit[o + p] = make_uint4((uint32_t)t, p, parts, 1u);
 }
 
 // The split units: a split tile's parts follow those of the split tiles before
@@ -750,9 +1084,18 @@ cudaError_t launch_tile_split(const IndexDims& d, const IndexBuffers& b, const g
                               cudaStream_t stream) {
   const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
   tile_cost_kernel<<<(unsigned)((n_tiles * 8 + 255) / 256), 256, 0, stream>>>(
-      d.grid, b.header, b.qpos, q.m, b.brange, b.listed, d.split_items, b.tparts, b.xpart);
-  note_launches(1);
-  return launch_split_units(n_tiles, b.tparts, b.xpart, b.xunit, &b.header->n_xunits, stream);
+      d.grid, b.header, b.qpos, q.m, b.brange, b.listed, b.tparts, &b.header->split_cost);
+  tile_parts_kernel<<<(unsigned)tile_groups(n_tiles), kTileGroup, 0, stream>>>(
+      n_tiles, d.split_items, b.tparts, &b.header->split_cost, b.xunit, &b.header->n_xunits);
+  note_launches(2);
+  return cudaGetLastError();
+}
+
+// Warps per tile: the chip holds 152 SMs x 20 warps of the forward at once, so
+// fewer tiles than that leave it waiting for the longest list of one warp (the
+// 512 tiles of a 4,096-Gaussian cube: 377 us with a warp each, 62 with 16).
+static int forward_team(int64_t n_tiles) {
+  return n_tiles <= 152 * 8 ? 16 : n_tiles <= 152 * 32 ? 4 : 1;
 }
 
 cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_queries& q,
@@ -766,14 +1109,13 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
   if (q.m == 0) return cudaSuccess;
   FwdArgs a;
   a.grid = d.grid;
-  a.qkey = b.qkey[b.qsorted];
   a.qval = b.qval[b.qsorted];
   a.qpos = b.qpos;
   a.header = b.header;
   a.albedo = q.albedo;
   a.m = q.m;
   a.rec = b.rec;
-  a.box = b.box;
+  a.vet = b.vet;
   a.brange = b.brange;
   a.listed = b.listed;
   a.gval = b.gval[b.gsorted];
@@ -800,30 +1142,43 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
     const cudaError_t e = cudaMemsetAsync(a.next_tile, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
   }
-  const int64_t tiles = (q.m + kWarp - 1) / kWarp + (split ? GPF_MAX_SPLIT_UNITS : 0);
-  const int64_t want = (tiles + kFwdWarps - 1) / kFwdWarps;
-#define GPF_FWD_LAUNCH2(CC, BR, PS, CN, SP)                                                \
-  do {                                                                                    \
-    const unsigned blocks = (unsigned)persistent_blocks(                                  \
-        reinterpret_cast<const void*>(&fwd_kernel<CC, BR, PS, CN, SP>), kFwdThreads, want); \
-    fwd_kernel<CC, BR, PS, CN, SP><<<blocks, kFwdThreads, 0, stream>>>(a);                \
+  const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
+  const int64_t units = n_tiles + (split ? GPF_MAX_SPLIT_UNITS : 0);
+  const int team = forward_team(n_tiles);
+  const int64_t want = team > 1 ? units : (units + kFwdWarps - 1) / kFwdWarps;
+#define GPF_FWD_LAUNCH(CC, BR, PS, CN, TM)                                                   \
+  do {                                                                                       \
+    constexpr int warps = TM > 4 ? TM : kFwdWarps;                                           \
+    const int smem =                                                                         \
+        (int)sizeof(float) * warps * warp_shared_words(CC, d.grid.levels, d.grid.coop);      \
+    const auto kernel = fwd_kernel<CC, BR, PS, CN, TM>;                                      \
+    cudaError_t e = cudaSuccess;                                                             \
+    if (smem > 48 * 1024)                                                                    \
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);   \
+    if (e != cudaSuccess) return e;                                                          \
+    const unsigned blocks = (unsigned)persistent_blocks(                                     \
+        reinterpret_cast<const void*>(kernel), warps * kWarp, want, smem);                   \
+    kernel<<<blocks, warps * kWarp, smem, stream>>>(a);                                      \
   } while (0)
-#define GPF_FWD_LAUNCH(CC, BR, PS, CN)                \
-  do {                                                \
-    if (!BR && split) GPF_FWD_LAUNCH2(CC, false, PS, CN, true); \
-    else GPF_FWD_LAUNCH2(CC, BR, PS, CN, false);      \
-  } while (0)
-#define GPF_FWD_MODES(CC, BR)                                          \
+#define GPF_FWD_TEAMS(CC, PS)                                          \
   do {                                                                 \
-    if (counts) GPF_FWD_LAUNCH(CC, BR, kKernGauss, true);              \
-    else if (kern == kKernDisk) GPF_FWD_LAUNCH(CC, BR, kKernDisk, false); \
-    else if (kern == kKernFalloff) GPF_FWD_LAUNCH(CC, BR, kKernFalloff, false); \
-    else GPF_FWD_LAUNCH(CC, BR, kKernGauss, false);                    \
+    if (team == 16) GPF_FWD_LAUNCH(CC, false, PS, false, 16);          \
+    else if (team == 4) GPF_FWD_LAUNCH(CC, false, PS, false, 4);       \
+    else GPF_FWD_LAUNCH(CC, false, PS, false, 1);                      \
   } while (0)
 #define GPF_FWD_CASE(CC)                                                              \
   case CC:                                                                            \
-    if (d.brute) GPF_FWD_MODES(CC, true);                                             \
-    else GPF_FWD_MODES(CC, false);                                                    \
+    if (d.brute) {                                                                    \
+      if (counts) GPF_FWD_LAUNCH(CC, true, kKernGauss, true, 1);                      \
+      else if (kern == kKernDisk) GPF_FWD_LAUNCH(CC, true, kKernDisk, false, 1);      \
+      else if (kern == kKernFalloff) GPF_FWD_LAUNCH(CC, true, kKernFalloff, false, 1); \
+      else GPF_FWD_LAUNCH(CC, true, kKernGauss, false, 1);                            \
+    } else {                                                                          \
+      if (counts) GPF_FWD_LAUNCH(CC, false, kKernGauss, true, 1);                     \
+      else if (kern == kKernDisk) GPF_FWD_TEAMS(CC, kKernDisk);                       \
+      else if (kern == kKernFalloff) GPF_FWD_TEAMS(CC, kKernFalloff);                 \
+      else GPF_FWD_TEAMS(CC, kKernGauss);                                             \
+    }                                                                                 \
     note_launches(1);                                                                 \
     if (split && !counts) {                                                           \
       fwd_split_combine_kernel<CC><<<GPF_MAX_SPLIT_UNITS / 4, 128, 0, stream>>>(a);   \
@@ -848,9 +1203,8 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
       return cudaErrorInvalidValue;
   }
 #undef GPF_FWD_CASE
-#undef GPF_FWD_MODES
+#undef GPF_FWD_TEAMS
 #undef GPF_FWD_LAUNCH
-#undef GPF_FWD_LAUNCH2
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return ev.stop ? cudaEventRecord(ev.stop, stream) : cudaSuccess;

@@ -56,7 +56,6 @@ __device__ __forceinline__ void block_counts(uint32_t (&v)[4], uint32_t (*s)[4])
 }
 // Boxes with more cells than this on their level are refused (overflow flag).
 constexpr int64_t kMaxBoxCells = int64_t(1) << 16;
-constexpr uint32_t kNoBox = 0xffffffffu;
 // Boxes of up to this many cells keep a bit mask of the occupied ones; emit
 // tests the cells of the others again.
 constexpr int64_t kMaskCells = 64;
@@ -96,27 +95,6 @@ __device__ __forceinline__ void flush_digits(const uint32_t* cnt, int passes,
                                              uint32_t* __restrict__ out) {
   for (int i = threadIdx.x; i < passes * kSortBins; i += blockDim.x)
     if (cnt[i]) atomicAdd(&out[i], cnt[i]);
-}
-
-// Position of the j-th (from 0) set bit of m, which has more than j.
-__device__ __forceinline__ uint32_t nth_bit(unsigned long long m, uint32_t j) {
-  uint32_t w = (uint32_t)m, pos = 0;
-  const uint32_t lo = (uint32_t)__popc(w);
-  if (j >= lo) {
-    j -= lo;
-    w = (uint32_t)(m >> 32);
-    pos = 32;
-  }
-#pragma unroll
-  for (int h = 16; h > 0; h >>= 1) {
-    const uint32_t c = (uint32_t)__popc(w & ((1u << h) - 1u));
-    if (j >= c) {
-      j -= c;
-      w >>= h;
-      pos += h;
-    }
-  }
-  return pos;
 }
 
 __device__ __forceinline__ bool occupied(const uint32_t* occ, uint32_t b) {
@@ -213,7 +191,7 @@ __global__ void quantize_bf16_kernel(gpf_field src, gpf_field dst) {
 // hit point (its list entries) and its key in the backward's order.
 __global__ void __launch_bounds__(kThreads, 4)
 preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
-                                  float* __restrict__ rec, int rs, uint4* __restrict__ box,
+                                  float* __restrict__ rec, int rs, VetRec* __restrict__ vet,
                                   const uint32_t* __restrict__ occ,
                                   uint32_t* __restrict__ gcount, uint8_t* __restrict__ glive,
                                   unsigned long long* __restrict__ gmask,
@@ -295,11 +273,12 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
       const int64_t vol = (int64_t)(sx + 1) * (sy + 1) * (sz + 1);
       uint32_t cnt = 0;
       if (sx > 255 || sy > 255 || sz > 255 || vol > kMaxBoxCells) {
-        box[g] = make_uint4(kNoBox, kNoBox, kNoBox, 0);
+        vet[g] = VetRec{mu[0], mu[1], mu[2], rv[3], 0ull, 0ull};
         atomicExch(&header->overflow, 1u);
       } else {
-        box[g] = make_uint4(lx | ((uint32_t)L << 20), ly, lz, sx | (sy << 8) | (sz << 16));
         rv[3] = rec_radius_with_level(rv[3], (uint32_t)L);
+        vet[g] = VetRec{mu[0], mu[1], mu[2], rv[3], kCellGuard - pack_cell(lx, ly, lz),
+                        kCellGuard + pack_cell(lx + sx, ly + sy, lz + sz)};
         level_bits |= 1u << L;
         // bit c of the mask: the c-th cell of the box (x fastest) holds a
         // hit point; emit walks the set bits only
@@ -517,8 +496,8 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
 // stores are coalesced and no lane waits for the Gaussian with the most cells
 // (a thread per Gaussian: 53 us and scattered 4-byte stores at 3.8 M entries).
 __global__ void __launch_bounds__(kThreads)
-emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec, int rs,
-            const uint4* __restrict__ box, const uint32_t* __restrict__ occ,
+emit_kernel(Grid grid, int64_t n, int64_t p_max, const VetRec* __restrict__ vet,
+            const uint32_t* __restrict__ occ,
             const unsigned long long* __restrict__ gmask, const uint32_t* __restrict__ gcount,
             const uint32_t* __restrict__ gpart, uint32_t* __restrict__ gkey,
             uint32_t* __restrict__ gval, int passes, uint32_t* __restrict__ digit_counts,
@@ -570,18 +549,28 @@ emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec, 
     for (int p = 0; p < passes; ++p)
       atomicAdd(&cnt[p * kSortBins + ((h.bucket >> (8 * p)) & 255u)], 1u);
   };
-  uint4 bw = make_uint4(kNoBox, 0u, 0u, 0u);
+  uint32_t bx = 0, by = 0, bz = 0;        // lowest cell of the box, the level above bx
+  uint32_t nx = 0, ny = 0, nz = 0;        // cells per axis (0: no box)
   unsigned long long mask = 0;
   uint32_t centre = 0;
   if (g < n) {
-    bw = box[g];
+    const VetRec r = load_vet(vet + g);
+    if (r.nlo != 0ull) {
+      const unsigned long long lo = kCellGuard - r.nlo, hi = r.hig - kCellGuard;
+      bx = (uint32_t)lo & kCoordMax;
+      by = (uint32_t)(lo >> 21) & kCoordMax;
+      bz = (uint32_t)(lo >> 42) & kCoordMax;
+      nx = ((uint32_t)hi & kCoordMax) - bx + 1;
+      ny = ((uint32_t)(hi >> 21) & kCoordMax) - by + 1;
+      nz = ((uint32_t)(hi >> 42) & kCoordMax) - bz + 1;
+      bx |= rec_level(r.radius) << kCoordBits;
+    }
     if (grid.blevel >= 0) {
       // the centre entry: the cell of the mean on the centre level
-      const float* r = rec + g * rs;
       const int Lb = grid.blevel;
-      const uint32_t cx = coord0(r[0], grid.ox, grid.inv_cell0, grid.max0x) >> Lb;
-      const uint32_t cy = coord0(r[1], grid.oy, grid.inv_cell0, grid.max0y) >> Lb;
-      const uint32_t cz = coord0(r[2], grid.oz, grid.inv_cell0, grid.max0z) >> Lb;
+      const uint32_t cx = coord0(r.x, grid.ox, grid.inv_cell0, grid.max0x) >> Lb;
+      const uint32_t cy = coord0(r.y, grid.oy, grid.inv_cell0, grid.max0y) >> Lb;
+      const uint32_t cz = coord0(r.z, grid.oz, grid.inv_cell0, grid.max0z) >> Lb;
       put(off, cell_hash(grid, Lb, cx, cy, cz, kCentreSalt), (uint32_t)g);
       const uint32_t bit = cocc_bit(grid, cx, cy, cz);
       atomicOr(cocc + (bit >> 5), 1u << (bit & 31u));
@@ -589,16 +578,14 @@ emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec, 
       centre = 1;
     }
   }
-  const bool boxed = bw.x != kNoBox;
-  const uint32_t nx = (bw.w & 0xffu) + 1, ny = ((bw.w >> 8) & 0xffu) + 1,
-                 nz = ((bw.w >> 16) & 0xffu) + 1;
-  const bool masked = boxed && nx * ny * nz <= (uint32_t)kMaskCells;
-  if (masked) mask = gmask[g];
+  const bool masked = nx * ny * nz <= (uint32_t)kMaskCells;
+  if (masked && nx) mask = gmask[g];
+  const uint32_t size = nx | (ny << 8) | (nz << 16);     // masked boxes: at most 64 each
   // the masked boxes of the warp, their set cells end to end: item f belongs
   // to the first lane whose inclusive count exceeds f; cell i of a box is
   // (i mod nx, (i / nx) mod ny, i / (nx ny)); i < 64, so the quotients
   // computed as floor((i + 0.5) / d) in float32 are exact
-  const uint32_t my = masked ? c - centre : 0u;
+  const uint32_t my = masked && nx ? c - centre : 0u;
   uint32_t mi = my;
 #pragma unroll
   for (int o = 1; o < kWarp; o <<= 1) {
@@ -614,35 +601,36 @@ emit_kernel(Grid grid, int64_t n, int64_t p_max, const float* __restrict__ rec, 
       if (__shfl_sync(kFullMask, mi, o + st - 1) <= f) o += st;
     const uint32_t j = f - __shfl_sync(kFullMask, mi - my, o);
     const unsigned long long om = __shfl_sync(kFullMask, mask, o);
-    const uint32_t x = __shfl_sync(kFullMask, bw.x, o), ly = __shfl_sync(kFullMask, bw.y, o),
-                   lz = __shfl_sync(kFullMask, bw.z, o), w = __shfl_sync(kFullMask, bw.w, o);
+    const uint32_t x = __shfl_sync(kFullMask, bx, o), y = __shfl_sync(kFullMask, by, o),
+                   z = __shfl_sync(kFullMask, bz, o), w = __shfl_sync(kFullMask, size, o);
     const uint32_t pos = __shfl_sync(kFullMask, off + centre, o) + j;
     if (f < total) {
       const uint32_t i = nth_bit(om, j);
-      const uint32_t onx = (w & 0xffu) + 1, onxy = onx * (((w >> 8) & 0xffu) + 1);
+      const uint32_t onx = w & 0xffu, onxy = onx * ((w >> 8) & 0xffu);
       const uint32_t dz = (uint32_t)(((float)i + 0.5f) * (1.0f / (float)onxy));
       const uint32_t r = i - dz * onxy;
       const uint32_t dy = (uint32_t)(((float)r + 0.5f) * (1.0f / (float)onx));
-      put(pos, cell_hash(grid, (int)(x >> 20), (x & kCoordMax) + r - dy * onx, ly + dy, lz + dz),
+      put(pos, cell_hash(grid, (int)(x >> kCoordBits), (x & kCoordMax) + r - dy * onx, y + dy,
+                         z + dz),
           (uint32_t)(g - lane) + (uint32_t)o);
     }
   }
   // the larger boxes one at a time, 32 cells at a time
-  for (uint32_t todo = __ballot_sync(kFullMask, boxed && !masked); todo; todo &= todo - 1u) {
+  for (uint32_t todo = __ballot_sync(kFullMask, !masked); todo; todo &= todo - 1u) {
     const int o = __ffs(todo) - 1;
-    const uint32_t x = __shfl_sync(kFullMask, bw.x, o), ly = __shfl_sync(kFullMask, bw.y, o),
-                   lz = __shfl_sync(kFullMask, bw.z, o);
-    const uint32_t bx = __shfl_sync(kFullMask, nx, o), by = __shfl_sync(kFullMask, ny, o),
-                   bz = __shfl_sync(kFullMask, nz, o);
-    const uint32_t cells = bx * by * bz;                 // at most kMaxBoxCells
+    const uint32_t x = __shfl_sync(kFullMask, bx, o), y = __shfl_sync(kFullMask, by, o),
+                   z = __shfl_sync(kFullMask, bz, o);
+    const uint32_t ox = __shfl_sync(kFullMask, nx, o), oy = __shfl_sync(kFullMask, ny, o),
+                   oz = __shfl_sync(kFullMask, nz, o);
+    const uint32_t cells = ox * oy * oz;                 // at most kMaxBoxCells
     uint32_t pos = __shfl_sync(kFullMask, off + centre, o);
     for (uint32_t i0 = 0; i0 < cells; i0 += kWarp) {
       const uint32_t i = i0 + lane;
       CellHash h{};
       bool set = false;
       if (i < cells) {
-        h = cell_hash(grid, (int)(x >> 20), (x & kCoordMax) + i % bx, ly + i / bx % by,
-                      lz + i / (bx * by));
+        h = cell_hash(grid, (int)(x >> kCoordBits), (x & kCoordMax) + i % ox, y + i / ox % oy,
+                      z + i / (ox * oy));
         set = occupied(occ, h.bucket);
       }
       const uint32_t sm = __ballot_sync(kFullMask, set);
@@ -846,13 +834,13 @@ cudaError_t launch_build(const IndexDims& d, const IndexBuffers& b, const gpf_fi
     const int group = group_size(f.n);
     const unsigned blocks = shared_blocks(blocks_for(f.n, group));
     preprocess_kernel<<<blocks, group, 0, stream>>>(
-        f, grid, d.cutoff, d.brute ? 1 : 0, b.rec, rec_stride(d.channels), b.box, b.occ,
+        f, grid, d.cutoff, d.brute ? 1 : 0, b.rec, rec_stride(d.channels), b.vet, b.occ,
         b.gcount, b.glive, b.gmask, b.qbox, b.okey[0], b.oval[0], radix_sort_passes(grid.obits),
         radix_sort_counts(b.osort_ws), lists ? b.gpart : nullptr, b.header);
     note_launches(1);
     if (lists) {
       emit_kernel<<<blocks, group, 0, stream>>>(
-          grid, f.n, d.p_max, b.rec, rec_stride(d.channels), b.box, b.occ, b.gmask, b.gcount,
+          grid, f.n, d.p_max, b.vet, b.occ, b.gmask, b.gcount,
           b.gpart, b.gkey[0], b.gval[0], radix_sort_passes(grid.hash_bits),
           radix_sort_counts(b.gsort_ws), b.cocc, b.focc, b.header);
       note_launches(1);

@@ -18,10 +18,11 @@ inline size_t focc_words(const Grid& g) {
 // Host-side count of the kernels this library has launched (gpf_launch_count).
 void note_launches(uint64_t k);
 
-// Blocks of a persistent launch of `kernel` (static shared memory only):
+// Blocks of a persistent launch of `kernel`:
 // the blocks that can be resident on all SMs of the current device at once,
 // at most max_blocks and at least 1.
-int64_t persistent_blocks(const void* kernel, int threads, int64_t max_blocks);
+int64_t persistent_blocks(const void* kernel, int threads, int64_t max_blocks,
+                          size_t dynamic_smem = 0);
 
 // ---- scan / sort (gpf_sort.cu)
 int64_t scan_partials_count(int64_t n);
@@ -65,7 +66,7 @@ cudaError_t launch_sort_wait_probe(void* buf, uint32_t spin_limit, uint32_t* sta
 struct IndexBuffers {
   DeviceHeader* header;
   float* rec;           // [N_max * rec_stride] Gaussian records
-  uint4* box;           // [N_max] level boxes
+  VetRec* vet;          // [N_max] mean, bounding sphere and level box (list vetting)
   uint32_t* gcount;     // [N_max] entries per Gaussian
   uint32_t* gpart;      // entries per group of Gaussians, then per kSuper groups
   uint8_t* glive;       // [N_max] 1 if the backward visits the Gaussian (a hit point in reach)
@@ -99,8 +100,7 @@ struct IndexBuffers {
   void* nbsort_ws;
   int nbsorted;
   // forward tile splitting (split_items > 0)
-  uint32_t* tparts;     // [tiles_max] parts of each tile (1 = not split)
-  uint32_t* xpart;      // [tiles_max / 256 + 1] parts of the split tiles of 256 tiles
+  uint32_t* tparts;     // [tiles_max] cost, then parts of each tile (1 = not split)
   uint4* xunit;         // [GPF_MAX_SPLIT_UNITS] (tile, part, parts, valid) of every split unit
   float* xsum;          // [GPF_MAX_SPLIT_UNITS * (C + 1) * 32] partial sums of split units
   // a centre level (ball_radius > 0): occupancy bits of the centre cells'
