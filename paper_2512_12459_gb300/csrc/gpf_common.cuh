@@ -33,12 +33,15 @@ struct DeviceHeader {
   // work counters of the persistent pair loops (reset before each launch)
   unsigned long long next_tile;       // forward: next tile of 32 hit points
   unsigned long long next_work;       // backward: next work item
+  uint32_t wild_grad;    // backward: 1 if a packed hit point holds a non-finite value
+  uint32_t wild_field;   // 1 if a coordinate or 1/scale is so large that a pair's
+                         // u = M (x - mu) could overflow
   uint32_t nonfinite;    // 1 if a Gaussian parameter or an active hit point is not finite
   uint32_t nb_pairs;     // (hit point, Gaussian) pairs of the last hybrid backward
   uint32_t n_xunits;     // work units of the split forward tiles (<= GPF_MAX_SPLIT_UNITS)
   uint32_t n_hunits;     // work units of the split hybrid forward tiles (same limit)
   unsigned long long split_cost;  // estimated work of all forward tiles
-  uint32_t pad[46];
+  uint32_t pad[44];
 };
 static_assert(sizeof(DeviceHeader) == 256, "header is one 256-byte block");
 
@@ -111,6 +114,18 @@ __host__ __device__ constexpr int rec_stride(int channels) {
 __host__ __device__ constexpr int qrec_stride(int channels) {
   return 4 * ((5 + channels + 3) / 4);
 }
+// The float32 backward's packed hit points: two neighbours of the sorted order
+// interleaved value by value, so that each value of both is one operand of the
+// packed arithmetic. Their positions and zeta (8 floats) lie in one array, read
+// by every test, kappa and gamma (padded to 8 floats) in a second one, read by
+// the pairs that pass.
+__host__ __device__ constexpr int pair_tail(int channels) {
+  return 8 * ((2 * (1 + channels) + 7) / 8);
+}
+__host__ __device__ constexpr int pair_stride(int channels) { return 8 + pair_tail(channels); }
+// Above these a float32 pair could overflow on the way (kWildInvScale * 2
+// kWildCoord stays below the largest float).
+constexpr float kWildCoord = 1e8f, kWildInvScale = 1e29f;
 // Per-Gaussian sums of the backward (A 6, B 3, D 3, dPhi C), zero padded.
 __host__ __device__ constexpr int gacc_stride(int channels) {
   return 12 + channels <= 16 ? 16 : 32;
@@ -383,6 +398,26 @@ __device__ __forceinline__ float mahalanobis_lower_bound(const float* Mrow, floa
   float s2 = fmaf(fabsf(Mrow[6]), hx, fmaf(fabsf(Mrow[7]), hy, fabsf(Mrow[8]) * hz));
   float vn = sqrtf(fmaf(v0, v0, fmaf(v1, v1, v2 * v2)));
   float sn = sqrtf(fmaf(s0, s0, fmaf(s1, s1, s2 * s2)));
+  return (vn - sn) - 4e-6f * (vn + sn);
+}
+
+// As mahalanobis_lower_bound, with the hardware's approximate square roots
+// (2 ulp, well inside the margin of 4e-6).
+__device__ __forceinline__ float sqrt_approx(float v) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float box_distance(const float* M, float ex, float ey, float ez,
+                                              float hx, float hy, float hz) {
+  const float v0 = fmaf(M[0], ex, fmaf(M[1], ey, M[2] * ez));
+  const float v1 = fmaf(M[3], ex, fmaf(M[4], ey, M[5] * ez));
+  const float v2 = fmaf(M[6], ex, fmaf(M[7], ey, M[8] * ez));
+  const float s0 = fmaf(fabsf(M[0]), hx, fmaf(fabsf(M[1]), hy, fabsf(M[2]) * hz));
+  const float s1 = fmaf(fabsf(M[3]), hx, fmaf(fabsf(M[4]), hy, fabsf(M[5]) * hz));
+  const float s2 = fmaf(fabsf(M[6]), hx, fmaf(fabsf(M[7]), hy, fabsf(M[8]) * hz));
+  const float vn = sqrt_approx(fmaf(v0, v0, fmaf(v1, v1, v2 * v2)));
+  const float sn = sqrt_approx(fmaf(s0, s0, fmaf(s1, s1, s2 * s2)));
   return (vn - sn) - 4e-6f * (vn + sn);
 }
 

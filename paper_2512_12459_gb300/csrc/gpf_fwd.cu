@@ -378,26 +378,6 @@ __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int leve
   return w;
 }
 
-// As mahalanobis_lower_bound, with the hardware's approximate square roots
-// (2 ulp, well inside the margin of 4e-6).
-__device__ __forceinline__ float sqrt_approx(float v) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ float box_distance(const float* M, float ex, float ey, float ez,
-                                              float hx, float hy, float hz) {
-  const float v0 = fmaf(M[0], ex, fmaf(M[1], ey, M[2] * ez));
-  const float v1 = fmaf(M[3], ex, fmaf(M[4], ey, M[5] * ez));
-  const float v2 = fmaf(M[6], ex, fmaf(M[7], ey, M[8] * ez));
-  const float s0 = fmaf(fabsf(M[0]), hx, fmaf(fabsf(M[1]), hy, fabsf(M[2]) * hz));
-  const float s1 = fmaf(fabsf(M[3]), hx, fmaf(fabsf(M[4]), hy, fabsf(M[5]) * hz));
-  const float s2 = fmaf(fabsf(M[6]), hx, fmaf(fabsf(M[7]), hy, fabsf(M[8]) * hz));
-  const float vn = sqrt_approx(fmaf(v0, v0, fmaf(v1, v1, v2 * v2)));
-  const float sn = sqrt_approx(fmaf(s0, s0, fmaf(s1, s1, s2 * s2)));
-  return (vn - sn) - 4e-6f * (vn + sn);
-}
-
 // What bounds it: issue and the latency of dependent gathers together (1M
 // Gaussians, one 1024 x 1024 view, ncu: 2.1 instructions a cycle and SM, 20
 // resident warps, long and short scoreboard the largest stalls, DRAM 5 %). So
