@@ -340,24 +340,21 @@ struct WarpShared {
   float4* box;             // [3] the tile's box: (lo, hi.x), (hi.yz, centre.xy),
                            // (centre.z, half extents)
   uint2* range;            // [levels][32]
-  unsigned long long* cell;  // [segments] pack_cell
-  uint32_t* start;         // first entry of a segment's list
-  uint32_t* incl;          // entries of the segments up to and with this one
-  uint32_t* tag;
-  uint32_t* lev;           // level | first segment of that level << 8
+  unsigned long long* cell;  // [segments + 3] pack_cell
+  uint4* seg;              // [segments] entries before it, first entry of its list - those,
+                           // tag, level | first segment of that level << 8
   uint32_t* queue;         // [kQueue]
 };
 __host__ __device__ constexpr int stage_words(int C) {
   return kWarp * (rec_stride(C) > stage_fields(C) ? rec_stride(C) : stage_fields(C));
 }
 __host__ __device__ constexpr int warp_shared_words(int C, int levels, int coop) {
-  // (the segments' count rounded up to even, for 16-byte pieces)
+  // (the cells' count rounded up to even, for 16-byte pieces)
   return stage_words(C) + (C + 1) * kWarp + 12 + 2 * levels * kWarp +
-         (levels * coop + 1) / 2 * 2 * 6 + kQueue;
+         (levels * coop + 4) / 2 * 2 * 2 + levels * coop * 4 + kQueue;
 }
 template <int C>
 __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int levels, int coop) {
-  const int segs = (levels * coop + 1) / 2 * 2;
   float* p = base + wib * warp_shared_words(C, levels, coop);
   WarpShared w;
   w.stage = p;
@@ -369,12 +366,10 @@ __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int leve
   w.range = reinterpret_cast<uint2*>(p);
   p += 2 * levels * kWarp;
   w.cell = reinterpret_cast<unsigned long long*>(p);
-  p += 2 * segs;
-  w.start = reinterpret_cast<uint32_t*>(p);
-  w.incl = w.start + segs;
-  w.tag = w.incl + segs;
-  w.lev = w.tag + segs;
-  w.queue = w.lev + segs;
+  p += (levels * coop + 4) / 2 * 2 * 2;
+  w.seg = reinterpret_cast<uint4*>(p);
+  p += levels * coop * 4;
+  w.queue = reinterpret_cast<uint32_t*>(p);
   return w;
 }
 
@@ -559,11 +554,10 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
         }
         if (has) {
           const int slot = n_seg + __popc(hm & lanemask_lt());
+          const uint32_t before = total + incl - (rg.y - rg.x);
           ws.cell[slot] = packed;
-          ws.start[slot] = rg.x;
-          ws.incl[slot] = total + incl;
-          ws.tag[slot] = cell_hash(G, lev, lx, ly, lz).tag;
-          ws.lev[slot] = (uint32_t)lev | ((uint32_t)n_seg << 8);
+          ws.seg[slot] = make_uint4(before, rg.x - before, cell_hash(G, lev, lx, ly, lz).tag,
+                                    (uint32_t)lev | ((uint32_t)n_seg << 8));
         }
         n_seg += __popc(hm);
         total += __shfl_sync(kFullMask, incl, kWarp - 1);
@@ -588,7 +582,7 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
       // a chunk's segments follow from the beginnings inside it, without a search
       const bool few = n_seg <= kWarp;
       const uint32_t seg_at =
-          few && lane < n_seg ? (lane > 0 ? ws.incl[lane - 1] : 0u) : 0xffffffffu;
+          few && lane < n_seg ? ws.seg[lane].x : 0xffffffffu;
       const uint32_t le = lanemask_lt() | (1u << lane);
       // entry e of the stream: its segment (the first whose inclusive count
       // exceeds e) and entry word, with the previous word of its list
@@ -606,11 +600,11 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
         if (e < total) {
           if (!few)
             for (int st = top; st > 0; st >>= 1)
-              if (seg + st <= n_seg - 1 && ws.incl[seg + st - 1] <= e) seg += st;
-          const uint32_t before = seg ? ws.incl[seg - 1] : 0u;
-          const uint32_t* p = a.gval + ws.start[seg] + (e - before);
+              if (seg + st <= n_seg - 1 && ws.seg[seg + st].x <= e) seg += st;
+          const uint2 sg = *reinterpret_cast<const uint2*>(ws.seg + seg);
+          const uint32_t* p = a.gval + (sg.y + e);         // modulo 2^32
           v = __ldg(p);
-          first = e == before;               // of its list
+          first = e == sg.x;                 // of its list
           if (!first && lane == 0) vprev = __ldg(p - 1);   // (else the lane to the left has it)
         }
       };
@@ -630,7 +624,8 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
           const uint32_t left = __shfl_up_sync(kFullMask, v, 1);
           // a Gaussian listed twice in a bucket sits on consecutive entries
           const bool again = !first_n && v == (lane == 0 ? vp_n : left);
-          bool keep = live && (v & ~G.id_mask) == ws.tag[seg] && !again;
+          const uint2 sl = reinterpret_cast<const uint2*>(ws.seg + seg)[1];   // tag, level
+          bool keep = live && (v & ~G.id_mask) == sl.x && !again;
           const uint32_t g = v & G.id_mask;
           VetRec r;
           if (keep) r = load_vet(a.vet + g);
@@ -642,12 +637,12 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
             const float ex = fmaxf(fmaxf(b0.x - r.x, r.x - b0.w), 0.0f);
             const float ey = fmaxf(fmaxf(b0.y - r.y, r.y - b1.x), 0.0f);
             const float ez = fmaxf(fmaxf(b0.z - r.z, r.z - b1.y), 0.0f);
-            const uint32_t sl = ws.lev[seg];
             // it must live on this level and cover this cell, and must not
             // have been taken from an earlier cell of this tile
             keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= r.radius * r.radius &&
-                   rec_level(r.radius) == (sl & 0xffu) && cell_in(r, ws.cell[seg]);
-            for (int j = (int)(sl >> 8); j < seg && keep; ++j) keep = !cell_in(r, ws.cell[j]);
+                   rec_level(r.radius) == (sl.y & 0xffu) && cell_in(r, ws.cell[seg]);
+            for (int j = (int)(sl.y >> 8); j < seg && keep; j += 2)      // two loads at a time
+              keep = !(cell_in(r, ws.cell[j]) || (j + 1 < seg && cell_in(r, ws.cell[j + 1])));
           }
           const uint32_t kb = __ballot_sync(kFullMask, keep);
           if (keep) ws.queue[qn + __popc(kb & lanemask_lt())] = g;
