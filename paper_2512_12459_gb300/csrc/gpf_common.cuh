@@ -222,7 +222,9 @@ __host__ __device__ __forceinline__ CellHash cell_hash(const Grid& g, int L, uin
   z ^= z >> 16;
   CellHash h;
   h.bucket = z >> (32 - g.hash_bits);
-  h.tag = z << g.id_bits;
+  // (a centre entry and a box entry of one Gaussian in one bucket never have the
+  // same tag: the highest bit tells them apart)
+  h.tag = ((z << g.id_bits) & 0x7fffffffu) | (salt ? 0x80000000u : 0u);
   return h;
 }
 // [start, end) of a bucket's list ([0, 0): it has none).

@@ -23,10 +23,11 @@
 //   * kNN: the hit points whose ball holds fewer than k_min Gaussians take
 //     the k_min nearest means instead, searched by the whole warp for one
 //     group of such points at a time (those within one cell of each other):
-//     rings of cells around the group's cells, slice by slice (slices and
-//     cells with no mean skipped by the bitmaps), each slice's cells spread
-//     over the lanes and their listed means 32 at a time, every point
-//     keeping its own sorted list in shared memory; a cell beyond every
+//     rings of cells around the group's cells (the slices with a mean from the
+//     coarse bitmap, a slice per lane, then the ring's occupied cells from the
+//     fine one, a word per lane), the occupied cells spread over the lanes and
+//     their listed means 32 at a time, every point keeping its own sorted list
+//     in shared memory; a cell beyond every
 //     point's k-th distance is skipped, and a point is settled once its
 //     k-th distance is within the searched box.
 // The same selection serves the backward (Sec. 4.2, Differentiable
@@ -212,21 +213,6 @@ __device__ __forceinline__ float unord_f(uint32_t u) {
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-// Cell j of the border of the rectangle [x0, x1] x [y0, y1] (both sides at
-// least 3 cells): along y0, up x1, back along y1, down x0.
-__device__ __forceinline__ void slice_border_cell(int j, int x0, int y0, int x1, int y1, int& x,
-                                                  int& y) {
-  const int wx = x1 - x0 + 1, wy = y1 - y0 + 1;
-  if (j < wx - 1) { x = x0 + j; y = y0; return; }
-  j -= wx - 1;
-  if (j < wy - 1) { x = x1; y = y0 + j; return; }
-  j -= wy - 1;
-  if (j < wx - 1) { x = x1 - j; y = y1; return; }
-  j -= wx - 1;
-  x = x0;
-  y = y1 - j;
-}
-
 // Distance along one axis from [lo, hi] (points) to the cell spanning finest
 // cells [c_lo, c_hi) from the origin o, grown by half a finest cell.
 __device__ __forceinline__ float cell_gap(float o, float cell0, int c_lo, int c_hi, float lo,
@@ -308,86 +294,100 @@ __device__ int warp_knn(const HybArgs& a, bool need, float px, float py, float p
     const int rmax = max(max(max(qx0, mx - qx1), max(qy0, my - qy1)), max(qz0, mz - qz1));
     for (int R = 0; R <= min(rmax, kMaxRing); ++R) {
       const int x0 = qx0 - R, x1 = qx1 + R, y0 = qy0 - R, y1 = qy1 + R, z0 = qz0 - R, z1 = qz1 + R;
-      // the ring slice by slice along z: the grown box's rectangle on its
-      // two z faces (every slice for R = 0), the rectangle's border between
-      const int wx = x1 - x0 + 1, wy = y1 - y0 + 1;
-      const int per = 2 * (wx + wy) - 4;
-      const float rwx = 1.0f / (float)wx;
-      // the occupancy cells under the rectangle (clipped to the grid)
+      // the grown box's cells that lie on its faces (all of them for R = 0),
+      // clipped to the grid, as rows along x: whole rows on the y and z faces,
+      // the two end cells of the others
+      const int fx0 = max(x0, 0), fx1 = min(x1, mx), fy0 = max(y0, 0), fy1 = min(y1, my);
+      const int fz1 = min(z1, mz);
+      // the occupancy cells under a slice, and the fine bits' words of its rows
       const int cs = G.cshift - Lb;
-      const int ux0 = max(x0, 0) >> cs, uy0 = max(y0, 0) >> cs;
-      const int unx = (min(x1, mx) >> cs) - ux0 + 1, nu = unx * ((min(y1, my) >> cs) - uy0 + 1);
-      const float runx = 1.0f / (float)unx;
-      // the fine bits' words under the rectangle: rows fy0.., words fw0..
-      const int fx0 = max(x0, 0), fx1 = min(x1, mx), fy0 = max(y0, 0);
+      const int ux0 = fx0 >> cs, uy0 = fy0 >> cs;
+      const int unx = (fx1 >> cs) - ux0 + 1, nu = unx * ((fy1 >> cs) - uy0 + 1);
       const int fw0 = fx0 >> 5, fnw = (fx1 >> 5) - fw0 + 1;
-      const int fn = G.fwords ? fnw * (min(y1, my) - fy0 + 1) : 0;
-      const float rfnw = 1.0f / (float)fnw;
-      for (int sz = max(z0, 0); sz <= min(z1, mz); ++sz) {
-        // a slice with no mean under its rectangle is skipped whole: first by
-        // the coarse bits (a few words in cache), then by the fine ones
+      const int per_slice = fnw * (fy1 - fy0 + 1);
+      for (int zb = max(z0, 0); zb <= fz1; zb += kWarp) {
+        // the slices that hold a mean, by the coarse bits, one slice per lane
         uint32_t any = 0u;
-        for (int u = lane; u < nu; u += kWarp) {
-          const int uy = (int)(((float)u + 0.5f) * runx);   // u / unx, exact at these sizes
-          const uint32_t bit = ((uint32_t)(sz >> cs) * G.cdy + (uint32_t)(uy0 + uy)) * G.cdx +
-                               (uint32_t)(ux0 + u - uy * unx);
-          any |= (__ldg(a.cocc + (bit >> 5)) >> (bit & 31u)) & 1u;
-        }
-        if (!__any_sync(kFullMask, any != 0u)) continue;
-        if (G.fwords) {
-          any = 0u;
-          for (int u = lane; u < fn; u += kWarp) {
-            const int r = (int)(((float)u + 0.5f) * rfnw);  // u / fnw, exact at these sizes
-            const int w = fw0 + u - r * fnw;
-            // the bits of word w inside [fx0, fx1]
-            const int b0 = max(fx0 - 32 * w, 0), b1 = min(fx1 - 32 * w, 31);
-            const uint32_t m = (b1 == 31 ? 0xffffffffu : (2u << b1) - 1u) & ~((1u << b0) - 1u);
-            any |= __ldg(a.focc + ((uint32_t)sz * G.fdy + (uint32_t)(fy0 + r)) * G.fwords +
-                         (uint32_t)w) & m;
+        if (zb + lane <= fz1) {
+          const uint32_t uz = (uint32_t)((zb + lane) >> cs) * G.cdy;
+          for (int u = 0, ux = 0, uy = 0; u < nu; ++u) {
+            const uint32_t bit = (uz + (uint32_t)(uy0 + uy)) * G.cdx + (uint32_t)(ux0 + ux);
+            any |= (__ldg(a.cocc + (bit >> 5)) >> (bit & 31u)) & 1u;
+            if (++ux == unx) {
+              ux = 0;
+              ++uy;
+            }
           }
-          if (!__any_sync(kFullMask, any != 0u)) continue;
         }
-        const bool face = R == 0 || sz == z0 || sz == z1;
-        const int n_slice = face ? wx * wy : per;
-        for (int c0 = 0; c0 < n_slice; c0 += kWarp) {
-          // one cell of the slice per lane: its entries, unless the cell lies
-          // beyond every needing point's k-th distance (box grown by half a
-          // finest cell for the rounding of the cell coordinates)
+        const uint32_t slices = __ballot_sync(kFullMask, any != 0u);
+        // their rows' words, one per lane: the occupied cells of the ring
+        const int words = __popc(slices) * per_slice;
+        for (int wb = 0; wb < words; wb += kWarp) {
+          uint32_t cells = 0u;
+          int rx = 0, ry = 0, rz = 0;       // the word's first cell
+          if (wb + lane < words) {
+            const int q = (wb + lane) / per_slice, r = wb + lane - q * per_slice;
+            rz = zb + (int)nth_bit(slices, (uint32_t)q);
+            ry = fy0 + r / fnw;
+            rx = 32 * (fw0 + r % fnw);
+            const bool face = R == 0 || rz == z0 || rz == z1 || ry == y0 || ry == y1;
+            // bits [lo, hi] of the word, or those of the row's two ends
+            const int lo = max(fx0 - rx, 0), hi = min(fx1 - rx, 31);
+            cells = (hi == 31 ? 0xffffffffu : (2u << hi) - 1u) & ~((1u << lo) - 1u);
+            if (!face) {
+              uint32_t ends = 0u;
+              if (x0 >= rx && x0 < rx + 32) ends |= 1u << (x0 - rx);
+              if (x1 >= rx && x1 < rx + 32) ends |= 1u << (x1 - rx);
+              cells &= ends;
+            }
+            if (G.fwords && cells)
+              cells &= __ldg(a.focc + ((uint32_t)rz * G.fdy + (uint32_t)ry) * G.fwords +
+                             (uint32_t)(rx >> 5));
+          }
+          uint32_t ci = (uint32_t)__popc(cells);
+          if (!__any_sync(kFullMask, ci != 0u)) continue;
+          const uint32_t mine_c = ci;
+#pragma unroll
+          for (int o = 1; o < kWarp; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFullMask, ci, o);
+            if (lane >= o) ci += t;
+          }
+          const uint32_t n_cells = __shfl_sync(kFullMask, ci, kWarp - 1);
+          for (uint32_t c0 = 0; c0 < n_cells; c0 += kWarp) {
+          // one cell per lane: its entries, unless the cell lies beyond every
+          // needing point's k-th distance (box grown by half a finest cell for
+          // the rounding of the cell coordinates)
           const uint32_t tmax = __reduce_max_sync(
               kFullMask, mine ? __float_as_uint(found == k ? thr_d : INFINITY) : 0u);
-          int cx = 0, cy = 0;
-          const int cz = sz;
+          const uint32_t cf = c0 + lane;
+          int co = 0;
+#pragma unroll
+          for (int st = 16; st > 0; st >>= 1)
+            if (__shfl_sync(kFullMask, ci, co + st - 1) <= cf) co += st;
+          const uint32_t word = __shfl_sync(kFullMask, cells, co);
+          const uint32_t before = __shfl_sync(kFullMask, ci - mine_c, co);
+          int cx = __shfl_sync(kFullMask, rx, co);
+          const int cy = __shfl_sync(kFullMask, ry, co);
+          const int cz = __shfl_sync(kFullMask, rz, co);
           uint32_t cnt = 0, eb = 0, tag = 0;
-          const int j = c0 + lane;
-          if (j < n_slice) {
-            if (face) {
-              const int q = (int)(((float)j + 0.5f) * rwx);   // j / wx, exact at these sizes
-              cy = y0 + q;
-              cx = x0 + j - q * wx;
-            } else {
-              slice_border_cell(j, x0, y0, x1, y1, cx, cy);
+          if (cf < n_cells) {
+            cx += (int)nth_bit(word, cf - before);
+            const float dx = cell_gap(G.ox, G.cell0, cx << Lb, (cx + 1) << Lb, bx0, bx1);
+            const float dy = cell_gap(G.oy, G.cell0, cy << Lb, (cy + 1) << Lb, by0, by1);
+            const float dz = cell_gap(G.oz, G.cell0, cz << Lb, (cz + 1) << Lb, bz0, bz1);
+            const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * 0.99999f;
+            bool occupied = true;
+            if (!G.fwords) {
+              const uint32_t bit = cocc_bit(G, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz);
+              occupied = (__ldg(a.cocc + (bit >> 5)) >> (bit & 31u)) & 1u;
             }
-            if (cx >= 0 && cx <= mx && cy >= 0 && cy <= my) {
-              const float dx = cell_gap(G.ox, G.cell0, cx << Lb, (cx + 1) << Lb, bx0, bx1);
-              const float dy = cell_gap(G.oy, G.cell0, cy << Lb, (cy + 1) << Lb, by0, by1);
-              const float dz = cell_gap(G.oz, G.cell0, cz << Lb, (cz + 1) << Lb, bz0, bz1);
-              const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * 0.99999f;
-              bool occupied;
-              if (G.fwords) {
-                occupied = (__ldg(a.focc + focc_word(G, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz)) >>
-                            (cx & 31)) & 1u;
-              } else {
-                const uint32_t bit = cocc_bit(G, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz);
-                occupied = (__ldg(a.cocc + (bit >> 5)) >> (bit & 31u)) & 1u;
-              }
-              if (!(d2 > __uint_as_float(tmax)) && occupied) {
-                const CellHash h =
-                    cell_hash(G, Lb, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz, kCentreSalt);
-                const uint2 rg = bucket_list(a.listed, a.brange, h.bucket);
-                eb = rg.x;
-                cnt = rg.y - rg.x;
-                tag = h.tag;
-              }
+            if (!(d2 > __uint_as_float(tmax)) && occupied) {
+              const CellHash h =
+                  cell_hash(G, Lb, (uint32_t)cx, (uint32_t)cy, (uint32_t)cz, kCentreSalt);
+              const uint2 rg = bucket_list(a.listed, a.brange, h.bucket);
+              eb = rg.x;
+              cnt = rg.y - rg.x;
+              tag = h.tag;
             }
           }
           uint32_t incl = cnt;
@@ -399,31 +399,47 @@ __device__ int warp_knn(const HybArgs& a, bool need, float px, float py, float p
           const uint32_t total = __shfl_sync(kFullMask, incl, kWarp - 1);
           // the cells' entries, 32 at a time: entry f of the chunk belongs to
           // the first lane whose inclusive count exceeds f
-          for (uint32_t f0 = 0; f0 < total; f0 += kWarp) {
-            const uint32_t f = f0 + lane;
-            int o = 0;
+          // (the entry words of the next 32 are fetched meanwhile). A mean
+          // farther from the needing points' box than all their k-th distances
+          // is not offered to them: in a dense cell that is nearly all of them,
+          // and each offer is read by every point (2,300 means beside a caustic:
+          // 170 us for one tile, at the end of the pass)
+          auto fetch = [&](uint32_t f, int& o, uint32_t& v) {
+            o = 0;
 #pragma unroll
             for (int st = 16; st > 0; st >>= 1)
               if (__shfl_sync(kFullMask, incl, o + st - 1) <= f) o += st;
             const uint32_t e = __shfl_sync(kFullMask, eb, o) + f -
                                (__shfl_sync(kFullMask, incl, o) - __shfl_sync(kFullMask, cnt, o));
+            v = f < total ? __ldg(a.gval + e) : 0u;
+          };
+          int o_n;
+          uint32_t v_n;
+          fetch((uint32_t)lane, o_n, v_n);
+          for (uint32_t f0 = 0; f0 < total; f0 += kWarp) {
+            const int o = o_n;
+            const uint32_t v = v_n;
             const uint32_t otag = __shfl_sync(kFullMask, tag, o);
             const int ox = __shfl_sync(kFullMask, cx, o);
             const int oy = __shfl_sync(kFullMask, cy, o);
             const int oz = __shfl_sync(kFullMask, cz, o);
-            bool have = false;
+            const bool match = f0 + lane < total && (v & ~G.id_mask) == otag;
             float4 cand = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (f < total) {
-              const uint32_t v = __ldg(a.gval + e);
-              if ((v & ~G.id_mask) == otag) {
-                const uint32_t g = v & G.id_mask;
-                const float4 t = __ldg(reinterpret_cast<const float4*>(a.rec + (int64_t)g * RS));
-                const float mu[3] = {t.x, t.y, t.z};
-                if (in_centre_cell(G, mu, (uint32_t)ox, (uint32_t)oy, (uint32_t)oz)) {
-                  cand = make_float4(t.x, t.y, t.z, __uint_as_float(g));
-                  have = true;
-                }
-              }
+            if (match)
+              cand = __ldg(reinterpret_cast<const float4*>(
+                  a.rec + (int64_t)(v & G.id_mask) * RS));
+            if (f0 + kWarp < total) fetch(f0 + kWarp + lane, o_n, v_n);
+            const float thr = __uint_as_float(__reduce_max_sync(
+                kFullMask, mine ? __float_as_uint(found == k ? thr_d : INFINITY) : 0u));
+            bool have = false;
+            if (match) {
+              const float mu[3] = {cand.x, cand.y, cand.z};
+              const float ex = fmaxf(fmaxf(bx0 - cand.x, cand.x - bx1), 0.0f);
+              const float ey = fmaxf(fmaxf(by0 - cand.y, cand.y - by1), 0.0f);
+              const float ez = fmaxf(fmaxf(bz0 - cand.z, cand.z - bz1), 0.0f);
+              have = !(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) * 0.99999f > thr) &&
+                     in_centre_cell(G, mu, (uint32_t)ox, (uint32_t)oy, (uint32_t)oz);
+              cand.w = __uint_as_float(v & G.id_mask);
             }
             const uint32_t hm = __ballot_sync(kFullMask, have);
             if (hm == 0u) continue;
@@ -456,6 +472,7 @@ __device__ int warp_knn(const HybArgs& a, bool need, float px, float py, float p
               }
             }
             __syncwarp();
+          }
           }
         }
       }
