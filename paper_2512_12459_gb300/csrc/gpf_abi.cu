@@ -148,6 +148,7 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   if (d.split_items > 0) {
     t.tparts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.xunit = reinterpret_cast<uint4*>(take(sizeof(uint4) * GPF_MAX_SPLIT_UNITS));
+    t.xheavy = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.xsum = reinterpret_cast<float*>(
         take(sizeof(float) * (size_t)GPF_MAX_SPLIT_UNITS * (d.channels + 1) * kWarp));
   }

@@ -31,6 +31,8 @@ struct DeviceHeader {
   uint32_t n_huge;       // live large Gaussians of the two top size ranks (split in the backward)
   uint32_t stalled;      // 1 if a bounded wait of the build's sort gave up
   // work counters of the persistent pair loops (reset before each launch)
+  unsigned long long next_heavy;      // forward, second launch: next unit of a deferred tile
+  unsigned long long n_heavy;         // forward: tiles deferred to the second launch
   unsigned long long next_tile;       // forward: next tile of 32 hit points
   unsigned long long next_work;       // backward: next work item
   uint32_t wild_grad;    // backward: 1 if a packed hit point holds a non-finite value
@@ -41,7 +43,7 @@ struct DeviceHeader {
   uint32_t n_xunits;     // work units of the split forward tiles (<= GPF_MAX_SPLIT_UNITS)
   uint32_t n_hunits;     // work units of the split hybrid forward tiles (same limit)
   unsigned long long split_cost;  // estimated work of all forward tiles
-  uint32_t pad[44];
+  uint32_t pad[40];
 };
 static_assert(sizeof(DeviceHeader) == 256, "header is one 256-byte block");
 

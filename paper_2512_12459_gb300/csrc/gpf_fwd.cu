@@ -34,13 +34,15 @@ namespace {
 
 constexpr int kFwdWarps = 4;
 constexpr int kFwdThreads = kFwdWarps * kWarp;
+// Units of a tile's estimated work (tile_cost_kernel).
+constexpr uint32_t kCostPerEntry = 8, kCostPerTile = 8 * 32 * 10;
 constexpr int kQueue = 128;   // vetted ids of a warp that wait for their records
 
 struct FwdArgs {
   Grid grid;
   const uint32_t* qval;    // sorted hit point ids
   const float4* qpos;      // sorted positions and ids of the active ones
-  const DeviceHeader* header;
+  DeviceHeader* header;
   const float* albedo;     // [C,M] or null
   int64_t m;
   const float* rec;
@@ -58,9 +60,10 @@ struct FwdArgs {
   float* out;              // [C,M]
   float* z;                // [M] or null
   unsigned long long* counts;  // count mode: [candidates, included]
-  unsigned long long* next_tile;  // work counter, zero at launch
   const uint32_t* tparts;  // split forward: parts of each tile (null: no splitting)
-  const uint4* xunit;      // split forward: (tile, part, parts, valid) of each split unit
+  uint4* xunit;            // split forward: (tile, part, parts, valid) of each split unit
+  uint32_t* xheavy;        // split forward: tiles deferred to the second launch
+  int late;                // 1: the second launch, over the deferred tiles
   float* xsum;             // split forward: [unit][C + 1][32] partial sums
 };
 
@@ -381,6 +384,25 @@ __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int leve
 // survivors load their record; the same view took 433 M instructions and 620 us
 // with a chunk loop per cell and level, 327 M and 520 us so. 5 blocks of 4 warps
 // per SM: at 6 (80 registers) the spills cost 5 % more than the warps bring.
+// A tile of a split forward that turns out longer than its estimate (eight
+// sampled points may miss the one in a dense cell) is deferred, before its lists
+// are walked, to a second launch, which splits it kHeavyParts ways: one such tile
+// begun late kept its warp for 290 us after all the others of a 215 us density
+// estimate had ended, and 690 us of a 1,860 us forward over eight views. Longer
+// means an eighth of what every warp has to do; nothing is deferred below
+// kHeavyChunks chunks. If they were too many for the list of units, the second
+// launch takes them whole (all of them, so that the sums do not depend on which
+// warp came first).
+constexpr uint32_t kHeavyParts = 8, kHeavyChunks = 48;
+__device__ __forceinline__ uint32_t heavy_chunks(const DeviceHeader* h) {
+  const unsigned long long share =
+      h->split_cost / ((unsigned long long)kCostPerEntry * kWarp * 152u * 20u);
+  return max(kHeavyChunks, (uint32_t)min(share / 8, 1ull << 20));
+}
+__device__ __forceinline__ bool heavy_fits(const DeviceHeader* h) {
+  return h->n_xunits + kHeavyParts * h->n_heavy <= (unsigned long long)GPF_MAX_SPLIT_UNITS;
+}
+
 // COUNT: count the evaluated and included pairs instead of summing radiance.
 // TEAM: warps of a block that share a tile, each taking every TEAM-th chunk of
 // its lists; their sums are added in order.
@@ -403,6 +425,12 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
   // n_x units, one per part; then every tile as one unit (a split tile's is
   // skipped)
   const int64_t n_x = a.tparts ? (int64_t)a.header->n_xunits : 0;
+  const bool late = !COUNT && a.late;
+  const bool late_split = late && heavy_fits(a.header);
+  const int64_t n_units =
+      late ? (int64_t)a.header->n_heavy * (late_split ? (int64_t)kHeavyParts : 1) : n_x + n_tiles;
+  const uint32_t limit = !COUNT && !late && a.tparts ? heavy_chunks(a.header) : 0xffffffffu;
+  unsigned long long* const next_unit = late ? &a.header->next_heavy : &a.header->next_tile;
   const uint32_t lmask = a.header->level_mask;
   uint32_t n_eval = 0, n_inc = 0;
   // persistent: every warp (team) takes the next unit until none is left, so a
@@ -411,19 +439,29 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
   int64_t unit;
   if (TEAM > 1) {
     __syncthreads();
-    if (threadIdx.x == 0) s_unit = atomicAdd(a.next_tile, 1ull);
+    if (threadIdx.x == 0) s_unit = atomicAdd(next_unit, 1ull);
     __syncthreads();
     unit = (int64_t)s_unit;
   } else {
     __syncwarp();
     unsigned long long unit_u = 0;
-    if (lane == 0) unit_u = atomicAdd(a.next_tile, 1ull);
+    if (lane == 0) unit_u = atomicAdd(next_unit, 1ull);
     unit = (int64_t)__shfl_sync(kFullMask, unit_u, 0);
   }
-  if (unit >= n_x + n_tiles) break;
+  if (unit >= n_units) break;
   int64_t tile;
   uint32_t part = 0, parts = 1;
-  if (unit < n_x) {
+  if (late) {
+    if (late_split) {
+      unit += n_x;
+      const uint4 xu = a.xunit[unit];
+      tile = xu.x;
+      part = xu.y;
+      parts = kHeavyParts;
+    } else {
+      tile = a.xheavy[unit];
+    }
+  } else if (unit < n_x) {
     const uint4 xu = a.xunit[unit];
     if (!xu.w) continue;                      // a slot left over at the capacity edge
     tile = xu.x;
@@ -574,6 +612,20 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
     // a split tile's part, and a team's warp, take every parts-th chunk of 32
     // entries, then of 32 items
     const uint32_t n_chunks = (total + kWarp - 1) / kWarp;
+    if (!split && n_chunks + __reduce_add_sync(kFullMask, len) / kWarp > limit) {
+      if (TEAM == 1 || wib == 0) {
+        uint32_t slot = 0;
+        if (lane == 0) {
+          slot = (uint32_t)atomicAdd(&a.header->n_heavy, 1ull);
+          a.xheavy[slot] = (uint32_t)tile;
+        }
+        const int64_t first =
+            n_x + (int64_t)kHeavyParts * __shfl_sync(kFullMask, slot, 0);
+        if (first + kHeavyParts <= GPF_MAX_SPLIT_UNITS && lane < kHeavyParts)
+          a.xunit[first + lane] = make_uint4((uint32_t)tile, lane, kHeavyParts, 1u);
+      }
+      continue;
+    }
     if (n_chunks > 0) {
       const float cut_keep = a.cut * 1.0001f;
       int top = 1;                          // the segment search's first step
@@ -862,7 +914,10 @@ template <int C>
 __global__ void fwd_split_combine_kernel(FwdArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (index_unusable(a.header) || u >= (int64_t)a.header->n_xunits) return;
+  const int64_t n_heavy = heavy_fits(a.header) ? (int64_t)a.header->n_heavy : 0;
+  if (index_unusable(a.header) ||
+      u >= (int64_t)a.header->n_xunits + (int64_t)kHeavyParts * n_heavy)
+    return;
   const uint4 xu = a.xunit[u];
   if (!xu.w || xu.y != 0u) return;
   const int64_t k = (int64_t)xu.x * kWarp + lane;
@@ -900,7 +955,6 @@ __global__ void fwd_split_combine_kernel(FwdArgs a) {
 // 17 us a unit; weighting the pooled ones an eighth left single units of up to
 // 690 us at the end of a 1.8 ms forward). And the sum over all tiles. Four tiles
 // per warp, eight lanes each.
-constexpr uint32_t kCostPerEntry = 8, kCostPerTile = 8 * 32 * 10;
 __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
                                  const float4* __restrict__ qpos, int64_t m,
                                  const uint2* __restrict__ brange,
@@ -1108,13 +1162,15 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
   a.out = out;
   a.z = z;
   a.counts = counts;
-  a.next_tile = &b.header->next_tile;
+  a.late = 0;
   const bool split = d.split_items > 0 && !d.brute;
   a.tparts = split ? b.tparts : nullptr;
   a.xunit = split ? b.xunit : nullptr;
+  a.xheavy = split ? b.xheavy : nullptr;
   a.xsum = split ? b.xsum : nullptr;
   {
-    const cudaError_t e = cudaMemsetAsync(a.next_tile, 0, sizeof(unsigned long long), stream);
+    const cudaError_t e =
+        cudaMemsetAsync(&b.header->next_heavy, 0, 3 * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
   }
   const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
@@ -1134,6 +1190,12 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
     const unsigned blocks = (unsigned)persistent_blocks(                                     \
         reinterpret_cast<const void*>(kernel), warps * kWarp, want, smem);                   \
     kernel<<<blocks, warps * kWarp, smem, stream>>>(a);                                      \
+    if (split && !CN) {                                                                      \
+      FwdArgs late = a;                                                                      \
+      late.late = 1;                                                                         \
+      kernel<<<blocks, warps * kWarp, smem, stream>>>(late);                                 \
+      note_launches(1);                                                                      \
+    }                                                                                        \
   } while (0)
 #define GPF_FWD_TEAMS(CC, PS)                                          \
   do {                                                                 \

@@ -103,6 +103,7 @@ struct IndexBuffers {
   uint32_t* tparts;     // [tiles_max] cost, then parts of each tile (1 = not split)
   uint4* xunit;         // [GPF_MAX_SPLIT_UNITS] (tile, part, parts, valid) of every split unit
   float* xsum;          // [GPF_MAX_SPLIT_UNITS * (C + 1) * 32] partial sums of split units
+  uint32_t* xheavy;     // [tiles_max] tiles deferred to the forward's second launch
   // a centre level (ball_radius > 0): occupancy bits of the centre cells'
   // coarse cells (Grid::cshift), and the hybrid forward's tile splitting
   uint32_t* cocc;       // [cdx * cdy * cdz / 32] set: some mean lies in the cell

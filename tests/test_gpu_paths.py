@@ -2,8 +2,9 @@
 pair loops, each against the brute-force path or the float64 build of the same
 library: teams of warps per tile, boxes of more cells than the occupancy mask
 holds, fields on either side of the small-group limit, hit points that fill a
-cell with odd counts between empty ones, upstream gradients that are not
-finite, and a centre grid too large for its fine occupancy bits."""
+cell with odd counts between empty ones, tiles longer than their samples say,
+upstream gradients that are not finite, and a centre grid too large for its
+fine occupancy bits."""
 
 import math
 
@@ -67,6 +68,28 @@ def test_group_edges_and_boxes_of_many_cells(gpf, n, span):
                                                     max_span=span)
     assert c == cb and idx.stats()["flags"] == 0
     np.testing.assert_allclose(z, zb, rtol=SUM_RTOL, atol=1e-30)
+
+
+@pytest.mark.parametrize("per", [1535, 1537, 4000])
+def test_tiles_whose_samples_miss_a_dense_cell(gpf, per):
+    """One hit point in a hundred stands in a dense cell of its own, so most of
+    those tiles cost more than their sampled points say; just below and above
+    the length at which such a tile is put off, and far above it."""
+    rng = np.random.default_rng(per)
+    m, dense = 1600, 16
+    x = rng.uniform(0.0, 1.0, (m, 3))
+    n = per * dense
+    fnp, qnp = synth.config1_random(seed=per, n=n, m=m)
+    fnp.mean = np.repeat(x[::m // dense], per, axis=0).T.astype(np.float32).copy()
+    fnp.logscale = np.full_like(fnp.logscale, math.log(3e-3))
+    qnp.x = np.ascontiguousarray(x.T.astype(np.float32))
+    qnp.valid = np.ones_like(qnp.valid)
+    _, _, ((o, z, c, idx), (ob, zb, cb, _)) = _both(gpf, fnp, qnp, gpf.GPF_SUM, 0.02,
+                                                    query_cell=0.02, split_items=64)
+    assert c == cb and idx.stats()["flags"] == 0
+    tol = 4000 * 2.0 ** -24                       # at most 4000 positive terms
+    np.testing.assert_allclose(z, zb, rtol=tol, atol=1e-30)
+    np.testing.assert_allclose(o, ob, rtol=tol, atol=1e-30)
 
 
 def _clusters(seed, per, n_clusters=60):
