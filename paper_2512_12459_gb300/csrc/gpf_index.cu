@@ -187,6 +187,37 @@ __global__ void quantize_bf16_kernel(gpf_field src, gpf_field dst) {
   for (int c = 0; c < src.channels; ++c) dspec[c * n + g] = f32_to_bf16(spec[c * n + g]);
 }
 
+// The bits of a box's occupancy mask per row and per slice: 3 and 9 for boxes of
+// up to 3 cells an axis, 4 and 16 for up to 4 (constants for the code that sets
+// them), else the box's own.
+__device__ __forceinline__ uint2 mask_strides(uint32_t nx, uint32_t ny, uint32_t nz) {
+  const uint32_t most = max(nx, max(ny, nz));
+  return most <= 3 ? make_uint2(3u, 9u) : most <= 4 ? make_uint2(4u, 16u)
+                                                    : make_uint2(nx, nx * ny);
+}
+
+// The occupancy mask of a box of at most N cells an axis: the N x N reads of a z
+// slice go out together, without a branch per cell.
+template <int N>
+__device__ __forceinline__ unsigned long long small_box_mask(
+    const Grid& grid, const uint32_t* __restrict__ occ, int L, uint32_t lx, uint32_t ly,
+    uint32_t lz, uint32_t sx, uint32_t sy, uint32_t sz) {
+  unsigned long long mask = 0;
+  for (uint32_t dz = 0; dz <= sz; ++dz) {
+    uint32_t bkt[N * N], word[N * N];
+#pragma unroll
+    for (int j = 0; j < N * N; ++j) {
+      bkt[j] = bucket_of(grid, L, lx + j % N, ly + j / N, lz + dz);
+      word[j] = (uint32_t)(j % N) <= sx && (uint32_t)(j / N) <= sy ? __ldg(occ + (bkt[j] >> 5)) : 0u;
+    }
+    uint32_t bits = 0;
+#pragma unroll
+    for (int j = 0; j < N * N; ++j) bits |= ((word[j] >> (bkt[j] & 31u)) & 1u) << j;
+    mask |= (unsigned long long)bits << (N * N * dz);
+  }
+  return mask;
+}
+
 // Per Gaussian: record, level box, the number of cells of that box holding a
 // hit point (its list entries) and its key in the backward's order.
 __global__ void __launch_bounds__(kThreads, 4)
@@ -284,36 +315,15 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
         vet[g] = VetRec{mu[0], mu[1], mu[2], rv[3], kCellGuard - pack_cell(lx, ly, lz),
                         kCellGuard + pack_cell(lx + sx, ly + sy, lz + sz)};
         level_bits |= 1u << L;
-        // bit c of the mask: the c-th cell of the box (x fastest) holds a
-        // hit point; emit walks the set bits only
+        // bit c of the mask: the c-th cell of the box (x fastest, rows and
+        // slices mask_strides apart) holds a hit point; emit walks the set bits
         unsigned long long mask = 0;
         if (sx <= 2 && sy <= 2 && sz <= 2) {
-          // at most 3 x 3 x 3 cells: the nine occupancy reads of a z slice
-          // are independent and go out together
-          for (uint32_t dz = 0; dz <= sz; ++dz) {
-#pragma unroll
-            for (uint32_t j = 0; j < 9; ++j) {
-              const uint32_t dy = j / 3, dx = j % 3;
-              if (dy <= sy && dx <= sx &&
-                  occupied(occ, bucket_of(grid, L, lx + dx, ly + dy, lz + dz))) {
-                ++cnt;
-                mask |= 1ull << ((dz * (sy + 1) + dy) * (sx + 1) + dx);
-              }
-            }
-          }
+          mask = small_box_mask<3>(grid, occ, L, lx, ly, lz, sx, sy, sz);
+          cnt = (uint32_t)__popcll(mask);
         } else if (sx <= 3 && sy <= 3 && sz <= 3) {
-          // the same for up to 4 x 4 x 4 cells
-          for (uint32_t dz = 0; dz <= sz; ++dz) {
-#pragma unroll
-            for (uint32_t j = 0; j < 16; ++j) {
-              const uint32_t dy = j / 4, dx = j % 4;
-              if (dy <= sy && dx <= sx &&
-                  occupied(occ, bucket_of(grid, L, lx + dx, ly + dy, lz + dz))) {
-                ++cnt;
-                mask |= 1ull << ((dz * (sy + 1) + dy) * (sx + 1) + dx);
-              }
-            }
-          }
+          mask = small_box_mask<4>(grid, occ, L, lx, ly, lz, sx, sy, sz);
+          cnt = (uint32_t)__popcll(mask);
         } else {
           uint32_t c = 0;
           for (uint32_t iz = lz; iz <= lz + sz; ++iz)
@@ -593,10 +603,11 @@ emit_kernel(Grid grid, int64_t n, int64_t p_max, const VetRec* __restrict__ vet,
   }
   const bool masked = nx * ny * nz <= (uint32_t)kMaskCells;
   if (masked && nx) mask = gmask[g];
-  const uint32_t size = nx | (ny << 8) | (nz << 16);     // masked boxes: at most 64 each
+  const uint2 strides = mask_strides(nx, ny, nz);
+  const uint32_t size = strides.x | (strides.y << 8);    // masked boxes: at most 64 each
   // the masked boxes of the warp, their set cells end to end: item f belongs
-  // to the first lane whose inclusive count exceeds f; cell i of a box is
-  // (i mod nx, (i / nx) mod ny, i / (nx ny)); i < 64, so the quotients
+  // to the first lane whose inclusive count exceeds f; bit i of a box's mask is
+  // cell (i mod row, (i mod slice) / row, i / slice); i < 64, so the quotients
   // computed as floor((i + 0.5) / d) in float32 are exact
   const uint32_t my = masked && nx ? c - centre : 0u;
   uint32_t mi = my;
@@ -619,7 +630,7 @@ emit_kernel(Grid grid, int64_t n, int64_t p_max, const VetRec* __restrict__ vet,
     const uint32_t pos = __shfl_sync(kFullMask, off + centre, o) + j;
     if (f < total) {
       const uint32_t i = nth_bit(om, j);
-      const uint32_t onx = w & 0xffu, onxy = onx * ((w >> 8) & 0xffu);
+      const uint32_t onx = w & 0xffu, onxy = w >> 8;
       const uint32_t dz = (uint32_t)(((float)i + 0.5f) * (1.0f / (float)onxy));
       const uint32_t r = i - dz * onxy;
       const uint32_t dy = (uint32_t)(((float)r + 0.5f) * (1.0f / (float)onx));
