@@ -229,13 +229,14 @@ struct KnnList {
 };
 
 // The k_min nearest means of the tile's points that need them (need: the
-// ball held fewer), searched by the whole warp together, one centre cell of
-// needing points at a time: the points of a cell have the same rings of
-// cells around them, which are now read once for all of them instead of
-// once per point. Ring 0 is the cell itself, ring R the cells at Chebyshev
-// distance R from it; the lanes share a ring's rows (a row of cells along
-// x; away from the ring's outer faces only its two end cells belong to the
-// ring), each lane walking its rows' entries, and every round the warp
+// ball held fewer), searched by the whole warp together, one group of adjacent
+// centre cells (at most 3 x 3 x 3) at a time: its points share the rings of
+// cells around it, which are read once for all of them. Ring 0 is the group's
+// box itself, ring R the cells of its box grown by R that lie on its faces. A
+// slice's coarse occupancy bits say whether it holds a mean at all; of the
+// others the fine bits of a row are taken 32 to a word, a word per lane, and
+// masked to the ring; the set bits are laid end to end, a cell per lane, and
+// the entries of those cells likewise. Every round the warp
 // stages one mean per lane in shared memory, where each needing lane of the
 // cell offers all of them to its own sorted list of the nearest (squared
 // distance, then index). A point is settled once it holds k_min means and

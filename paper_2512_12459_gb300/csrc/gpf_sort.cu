@@ -6,11 +6,13 @@
 // Adinets and Merrill, "Onesweep", 2022):
 //   0. one kernel counts the digits of every pass over all keys (the global
 //      digit counts do not depend on the order the earlier passes leave);
-//   1. per pass, one kernel: a block claims the next tile of 3072 keys from
-//      an atomic counter (so every earlier tile is held by a block that is
-//      already running; small sorts take tiles of 1024); each warp ranks its own 384 keys, 32 at a time
-//      (groups of equal digits from bit ballots, per-warp digit counters in
-//      shared memory);
+//   1. per pass, one kernel for up to three sorts side by side (a sort that
+//      has no such pass takes no blocks): a block claims the next tile of its
+//      sort, 3072 keys (small sorts 1024), from an atomic counter, so every
+//      earlier tile is held by a block that is already running; keys and
+//      values are read into registers, and each warp ranks its own, 32 at a
+//      time (groups of equal digits from bit ballots, per-warp digit counters
+//      in shared memory);
 //      the block publishes its digit counts, orders its keys by digit in
 //      shared memory, adds up the counts the earlier tiles published for each
 //      digit, walking back until a tile whose inclusive prefix is known,
