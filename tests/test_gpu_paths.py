@@ -57,6 +57,17 @@ def test_teams_of_warps_sum_the_same_pairs(gpf, m, split):
     np.testing.assert_allclose(o, ob, rtol=SUM_RTOL, atol=1e-30)
 
 
+@pytest.mark.parametrize("n", [2**17, 2**19 - 1, 2**19, 2**19 + 1])
+def test_sort_on_either_side_of_the_small_tiles(gpf, n):
+    import torch
+    k = np.random.default_rng(n).integers(0, 1 << 20, n, dtype=np.uint64).astype(np.uint32)
+    ok, ov = gpf.gpf_sort_pairs(torch.from_numpy(k.view(np.int32)).cuda(),
+                                torch.arange(n, dtype=torch.int32, device="cuda"), 20)
+    order = np.argsort(k, kind="stable")
+    assert np.array_equal(ok.cpu().numpy().view(np.uint32), k[order])
+    assert np.array_equal(ov.cpu().numpy(), order.astype(np.int32))
+
+
 @pytest.mark.parametrize("n", [63, 64, 65, 65536, 65537])
 @pytest.mark.parametrize("span", [4, 5, 9])
 def test_group_edges_and_boxes_of_many_cells(gpf, n, span):
