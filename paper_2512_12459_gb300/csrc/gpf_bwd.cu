@@ -822,9 +822,35 @@ __device__ __forceinline__ void bwd_pair2(const PairG2<C>& P, uint32_t pair, flo
 // neighbouring hit points at a time. A row's pairs may reach one point past
 // either end, which is left out: over empty cells it may belong to another row
 // of the same Gaussian. A small Gaussian runs on a lane
-// unless its cells hold more than kLanePoints hit points (many views of one
-// place): the warp takes those one by one, as the large ones.
-constexpr uint32_t kLanePoints = 192;
+// unless the warp does better to take it as it takes the large ones, one by one
+// (lane_limit).
+//
+// Hit points up to which a small Gaussian stays on its lane, of this warp's 32.
+// The lanes go as long as the longest of them, a pair each a round, and their
+// loads go to 32 places (kLaneRound); a Gaussian that the whole warp takes costs
+// 1/32 of its rounds, of coalesced loads, and kWholeRounds more for its rows and
+// the reduction. So a few long ones among short ones (many views of one place)
+// leave the lanes, and 32 that are alike stay up to some 130 points: the
+// doubling limit with the least cost is taken. Pair loop over 1M Gaussians with
+// query cells of 0.031 and 0.062: 0.74 and 1.11 ms at a fixed limit of 192
+// points, 0.69 and 1.65 at 768; kLaneRound 1, 2, 3, 5: 0.68, 0.62, 0.58, 0.57
+// and 1.67, 1.09, 1.09, 1.10 ms.
+constexpr uint32_t kLanePoints = 96, kLaneRound = 5, kWholeRounds = 8;
+__device__ __forceinline__ uint32_t lane_limit(uint32_t points) {
+  uint32_t limit = kLanePoints, best = 0xffffffffu, t = kLanePoints;
+  for (;;) {
+    const bool stays = points <= t;
+    const uint32_t rounds =
+        kLaneRound * (__reduce_max_sync(kFullMask, stays ? points : 0u) >> 1) +
+        __reduce_add_sync(kFullMask, stays ? 0u : (points >> 6) + kWholeRounds);
+    if (rounds < best) {
+      best = rounds;
+      limit = t;
+    }
+    if (__all_sync(kFullMask, stays)) return limit;
+    t *= 2;
+  }
+}
 // Resident blocks: the loads of the hit points are what the warps wait for, so
 // more warps win over fewer spills up to four channels (1M Gaussians, 3
 // channels: 5, 6, 7, 8 blocks per SM give a training step of 1.97, 1.90, 1.85,
@@ -899,19 +925,20 @@ bwd_pairs_kernel(const __grid_constant__ BwdArgs a) {
     uint32_t part = 0, parts = 1;              // this unit's share of the row blocks
     if (w < small_warps) {
       const uint32_t idx = w * kWarp + lane;
-      bool heavy = false;
+      uint32_t mine = 0, points = 0;
+      uint2 box = make_uint2(0u, 0u);
+      // at most 2 x 2 rows
+      uint2 row[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) row[r] = make_uint2(0u, 0u);
       if (idx < n_small) {
-        const uint32_t mine = a.order[idx];
-        const uint2 box = a.qbox[mine];
+        mine = a.order[idx];
+        box = a.qbox[mine];
         uint32_t lo[3], hi[3];
         unpack_qbox(box, lo, hi);
         const uint32_t nx = hi[0] - lo[0] + 1;
-        // at most 2 x 2 rows
-        uint2 row[4];
-        uint32_t points = 0;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          row[r] = make_uint2(0u, 0u);
           const uint32_t iy = lo[1] + (r & 1), iz = lo[2] + (r >> 1);
           if (iy <= hi[1] && iz <= hi[2]) {
             const uint32_t key = qkey_of(Gd, lo[0], iy, iz);
@@ -919,7 +946,9 @@ bwd_pairs_kernel(const __grid_constant__ BwdArgs a) {
             points += row[r].y - row[r].x;
           }
         }
-        heavy = points > kLanePoints;
+      }
+      const bool heavy = points > lane_limit(points);
+      if (idx < n_small) {
         if (heavy) {
           s_unit[wib][lane] = make_uint4(mine, box.x, box.y, 0u);
         } else {

@@ -138,6 +138,37 @@ def test_backward_row_ends_and_full_cells(gpf, per, channels):
                 assert float((a - b).norm()) <= GRAD_TOL * float(b.norm()), (k, cell, mode)
 
 
+@pytest.mark.parametrize("most", [95, 97, 500, 3000])
+def test_small_gaussians_over_uneven_cells(gpf, most):
+    """Gaussians of a few cells whose cells hold one hit point or many, side by
+    side in a warp: those with many may leave their lanes for the whole warp."""
+    import torch
+    from paper_2512_12459_gb300.setup_index import make_index
+    rng = np.random.default_rng(most)
+    c = rng.uniform(0.05, 0.95, (40, 3))
+    x = np.repeat(c, np.where(np.arange(40) % 5, 1, most), axis=0)
+    x = x + rng.normal(0, 2e-3, x.shape)
+    m = len(x)
+    up = np.tile(np.array([[0.0], [0.0], [1.0]]), (1, m)).astype(np.float32)
+    queries = gpf.Queries.from_numpy(synth.Queries(
+        x=np.ascontiguousarray(x.T.astype(np.float32)), n=up, wo=up.copy(),
+        valid=np.ones(m, np.uint8)))
+    fnp, _ = synth.config1_random(seed=most, n=960, m=8)
+    fnp.mean = (np.tile(c, (24, 1)) + rng.normal(0, 2e-3, (960, 3))).T.astype(np.float32).copy()
+    fnp.logscale = rng.normal(math.log(4e-3), 0.3, (3, 960)).astype(np.float32)
+    field = gpf.Field.from_numpy(fnp)
+    G = torch.as_tensor(rng.standard_normal((3, m)).astype(np.float32), device="cuda")
+    idx = make_index(field, queries, query_cell=0.05)
+    idx.build(field, queries)
+    assert idx.stats()["n_small"] > 0
+    o, z = gpf.gpf_radiance_fwd(idx, field, queries, gpf.GPF_SUM, r_max=0.2)
+    g, g64 = (gpf.gpf_radiance_bwd(idx, field, queries, G, o, z, gpf.GPF_SUM, r_max=0.2,
+                                   f64_sums=f) for f in (False, True))
+    for k in KEYS:
+        a, b = getattr(g, k).double(), getattr(g64, k).double()
+        assert float((a - b).norm()) <= GRAD_TOL * float(b.norm()), k
+
+
 @pytest.mark.parametrize("value", [math.nan, math.inf])
 def test_a_wild_upstream_value_reaches_its_own_gaussians_only(gpf, value):
     import torch
