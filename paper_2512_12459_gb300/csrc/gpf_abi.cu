@@ -131,10 +131,7 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   }
   t.qpos = reinterpret_cast<float4*>(take(sizeof(float4) * M));
   t.qstart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * ncp));
-  // (either layout: single hit points, or pairs with room for an odd last one)
-  t.qrec = reinterpret_cast<float*>(
-      take(sizeof(float) * std::max<size_t>((size_t)M * qrec_stride(d.channels),
-                                            (size_t)(M + 1) / 2 * pair_stride(d.channels))));
+  t.qrec = reinterpret_cast<float*>(take(sizeof(float) * M * qrec_stride(d.channels)));
   // room for float64 sums (the gradient-check build of the backward)
   t.gacc = reinterpret_cast<float*>(take(sizeof(double) * N * gacc_stride(d.channels)));
   t.bpart = reinterpret_cast<float*>(take(sizeof(double) * std::min<int64_t>(N, kSplitMax) *

@@ -40,18 +40,15 @@ constexpr int kBwdThreads = kBwdWarps * kWarp;
 
 struct BwdArgs {
   Grid grid;
-  DeviceHeader* header;
-  const uint32_t* qval;
+  const DeviceHeader* header;
   const float4* qpos;
   const uint32_t* qstart;
-  const float* x;
   const float* albedo;
   const float* grad_out;
   const float* out;
   const float* z;
   int64_t m;
-  float* qrec;            // packed hit points (float32 grid path: the pairs' heads)
-  float* qtail;           // float32 grid path: the pairs' tails
+  float* qrec;            // packed hit points
   void* gacc;             // [N * NS] per-Gaussian sums (type T), by Gaussian id
   const uint8_t* glive;   // [N] 1 if the pair loop visits the Gaussian
   const uint2* qbox;      // [N] query-level cell bounds (pack_qbox), from the build
@@ -76,7 +73,8 @@ __global__ void pack_qrec_kernel(BwdArgs a) {
   constexpr int QS = qrec_stride(C);
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (index_unusable(a.header) || k >= (int64_t)a.header->n_active) return;
-  const uint32_t q = a.qval[k];
+  const float4 at = __ldg(a.qpos + k);
+  const uint32_t q = __float_as_uint(at.w);
   float gam[C];
   float kappa = 0.0f, zeta = 1.0f;
 #pragma unroll
@@ -105,67 +103,15 @@ __global__ void pack_qrec_kernel(BwdArgs a) {
     }
   }
   float* r = a.qrec + k * QS;
-  r[0] = a.x[q];
-  r[1] = a.x[a.m + q];
-  r[2] = a.x[2 * a.m + q];
+  r[0] = at.x;
+  r[1] = at.y;
+  r[2] = at.z;
   r[3] = zeta;
   r[4] = kappa;
 #pragma unroll
   for (int c = 0; c < C; ++c) r[5 + c] = gam[c];
 #pragma unroll
   for (int c = 5 + C; c < QS; ++c) r[c] = 0.0f;
-}
-
-// The packed hit points of the float32 grid path: one thread per pair of
-// neighbours in the sorted order (an absent second one is zero). Flags non-finite values (wild_grad).
-template <int C>
-__global__ void pack_pairs_kernel(BwdArgs a) {
-  constexpr int PT = pair_tail(C);
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n_act = a.header->n_active;
-  if (index_unusable(a.header) || 2 * p >= n_act) return;
-  float v[8 + PT];
-#pragma unroll
-  for (int i = 0; i < 8 + PT; ++i) v[i] = 0.0f;
-  bool wild = false;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if (2 * p + h >= n_act) continue;
-    const float4 at = __ldg(a.qpos + 2 * p + h);
-    const uint32_t q = __float_as_uint(at.w);
-    float kappa = 0.0f, zeta = 1.0f;
-    float g[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) g[c] = a.grad_out[(int64_t)c * a.m + q];
-    if (a.mode == GPF_NORMALIZED) {
-      const float Z = a.z[q];
-      if (Z > a.eps) {
-        zeta = 1.0f / Z;
-#pragma unroll
-        for (int c = 0; c < C; ++c) kappa = fmaf(g[c], a.out[(int64_t)c * a.m + q], kappa);
-      } else {
-        zeta = 1.0f / a.eps;
-      }
-    }
-    v[h] = at.x;
-    v[2 + h] = at.y;
-    v[4 + h] = at.z;
-    v[6 + h] = zeta;
-    v[8 + h] = kappa;
-    wild = wild || !isfinite(zeta) || !isfinite(kappa);
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const float gam = g[c] * (a.albedo ? a.albedo[(int64_t)c * a.m + q] : 1.0f);
-      v[10 + 2 * c + h] = gam;
-      wild = wild || !isfinite(gam);
-    }
-  }
-  float4* r = reinterpret_cast<float4*>(a.qrec + p * 8);
-  float4* t = reinterpret_cast<float4*>(a.qtail + p * PT);
-#pragma unroll
-  for (int i = 0; i < 2 + PT / 4; ++i)
-    (i < 2 ? r[i] : t[i - 2]) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-  if (wild) a.header->wild_grad = 1u;
 }
 
 // acc += a * b and acc += a for float32 terms a, b into sums of type T:
@@ -266,10 +212,7 @@ template <int C>
 __device__ __forceinline__ void load_qrec(const float* __restrict__ qr,
                                           float (&q)[qrec_stride(C)]) {
 #pragma unroll
-  for (int v = 0; v < qrec_stride(C) / 4; ++v) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(qr) + v);
-    q[4 * v] = t.x; q[4 * v + 1] = t.y; q[4 * v + 2] = t.z; q[4 * v + 3] = t.w;
-  }
+  for (int v = 0; v < qrec_stride(C); v += 8) ld_global_v8(qr + v, q + v);
 }
 
 // One (Gaussian, hit point) pair of the backward in float64 (the
@@ -390,6 +333,101 @@ __device__ __forceinline__ void bwd_pair(const PairG<C, T>& P, const float* __re
   bwd_pair_q<C, PSI, T>(P, q, a, acc);
 }
 
+// Whether the whole-warp loop takes two chunks of hit points at a time, in packed
+// arithmetic. It needs the Gaussian's values twice: at 56 registers that spills 56
+// bytes for 3 channels and 400 for 8 (64 views over 2M Gaussians, 3 channels: 8.53
+// ms with, 8.89 without; 200K Gaussians, 4 channels: 1.20 and 1.30; two views, 8
+// channels: 3.67 and 1.88). Fewer, larger blocks cost more than the spills.
+__host__ __device__ constexpr bool two_points(int channels, size_t sum_bytes) {
+  return sum_bytes == 4 && channels <= 4;
+}
+
+// A Gaussian with every value doubled, as the packed arithmetic takes it.
+template <int C>
+struct PairG2 {
+  f32x2 nmx, nmy, nmz;      // -mu
+  f32x2 M[9], phi[C];
+};
+
+// One Gaussian and two packed hit points, the second after the first: the terms
+// of bwd_pair_q, two to an instruction and each rounded as there, and the sums in
+// turn, a scalar operation each (an excluded point adds nothing). cut0, cut1:
+// cut2, or -1 where there is no such point.
+template <int C, bool PSI>
+__device__ __forceinline__ void bwd_pair2(const PairG2<C>& P, const float* __restrict__ qr0,
+                                          const float* __restrict__ qr1, float cut0, float cut1,
+                                          const BwdArgs& a, Acc<C, float>& acc) {
+  constexpr int QS = qrec_stride(C);
+  float q0[QS], q1[QS];
+  load_qrec<C>(qr0, q0);
+  load_qrec<C>(qr1, q1);
+  auto q = [&](int i) { return pack2(q0[i], q1[i]); };
+  const f32x2 dx = add2(q(0), P.nmx), dy = add2(q(1), P.nmy), dz = add2(q(2), P.nmz);
+  f32x2 u[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    u[j] = fma2(P.M[3 * j], dx, fma2(P.M[3 * j + 1], dy, mul2(P.M[3 * j + 2], dz)));
+  const f32x2 Q = fma2(u[0], u[0], fma2(u[1], u[1], mul2(u[2], u[2])));
+  float Q0, Q1;
+  unpack2(Q, Q0, Q1);
+  const bool in0 = Q0 <= cut0, in1 = Q1 <= cut1;
+  if (!(in0 || in1)) return;
+  f32x2 e = mul2(Q, pack2(-0.5f, -0.5f));
+  f32x2 pcoef = 0;   // 6 t / (r' |d|), the falloff's share of dw/dmu per unit w
+  if (PSI) {
+    const f32x2 d2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    float d0, d1;
+    unpack2(d2, d0, d1);
+    // |d| and 1/|d| from one reciprocal square root; t = 0 within the radius
+    const f32x2 inv_d = pack2(rsqrt_approx(d0), rsqrt_approx(d1));
+    const f32x2 irr = pack2(a.inv_rr, a.inv_rr);
+    float t0, t1;
+    unpack2(mul2(fma2(d2, inv_d, pack2(-a.r, -a.r)), irr), t0, t1);
+    const f32x2 t = pack2(d0 > a.r2 ? t0 : 0.0f, d1 > a.r2 ? t1 : 0.0f);
+    e = fma2(mul2(pack2(-3.0f, -3.0f), t), t, e);
+    pcoef = mul2(mul2(mul2(pack2(6.0f, 6.0f), t), irr), inv_d);
+  }
+  float e0, e1;
+  unpack2(mul2(e, pack2(kLog2e, kLog2e)), e0, e1);
+  const f32x2 w = pack2(ex2_approx(e0), ex2_approx(e1));
+  const f32x2 zeta = q(3);
+  f32x2 gp = mul2(q(5), P.phi[0]);
+#pragma unroll
+  for (int c = 1; c < C; ++c) gp = fma2(q(5 + c), P.phi[c], gp);
+  const f32x2 bw = mul2(mul2(zeta, fma2(q(4), pack2(-1.0f, -1.0f), gp)), w);
+  const f32x2 b[3] = {mul2(bw, u[0]), mul2(bw, u[1]), mul2(bw, u[2])};
+  const f32x2 pc = mul2(bw, pcoef), wz = mul2(w, zeta);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (!(h ? in1 : in0)) continue;
+    auto half = [&](f32x2 v) {
+      float lo, hi;
+      unpack2(v, lo, hi);
+      return h ? hi : lo;
+    };
+    const float b0 = half(b[0]), b1 = half(b[1]), b2 = half(b[2]);
+    const float u0 = half(u[0]), u1 = half(u[1]), u2 = half(u[2]);
+    acc.A00 = fmaf(b0, u0, acc.A00);
+    acc.A01 = fmaf(b0, u1, acc.A01);
+    acc.A02 = fmaf(b0, u2, acc.A02);
+    acc.A11 = fmaf(b1, u1, acc.A11);
+    acc.A12 = fmaf(b1, u2, acc.A12);
+    acc.A22 = fmaf(b2, u2, acc.A22);
+    acc.B0 += b0;
+    acc.B1 += b1;
+    acc.B2 += b2;
+    if (PSI) {
+      const float p = half(pc);
+      acc.D0 = fmaf(p, half(dx), acc.D0);
+      acc.D1 = fmaf(p, half(dy), acc.D1);
+      acc.D2 = fmaf(p, half(dz), acc.D2);
+    }
+    const float wh = half(wz);
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc.P[c] = fmaf(h ? q1[5 + c] : q0[5 + c], wh, acc.P[c]);
+  }
+}
+
 // Gradients of one Gaussian from its reduced sums (runs on one lane), in
 // the sums' type T.
 template <int C, typename T>
@@ -500,6 +538,17 @@ __device__ __forceinline__ void load_pair_gaussian(const BwdArgs& a, int64_t gi,
   }
 }
 
+template <int C>
+__device__ __forceinline__ void double_gaussian(const PairG<C, float>& P, PairG2<C>& R) {
+  R.nmx = pack2(-P.G.mx, -P.G.mx);
+  R.nmy = pack2(-P.G.my, -P.G.my);
+  R.nmz = pack2(-P.G.mz, -P.G.mz);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) R.M[i] = pack2(P.G.M[i], P.G.M[i]);
+#pragma unroll
+  for (int c = 0; c < C; ++c) R.phi[c] = pack2(P.phi[c], P.phi[c]);
+}
+
 // Stores NS sums of type T (16-byte vectors).
 template <int NS, typename T>
 __device__ __forceinline__ void store_sums(T* dst, const T (&v)[NS]) {
@@ -539,6 +588,13 @@ __device__ void bwd_lane_gaussian(const BwdArgs& a, int64_t gi) {
   T v[NS];
   acc.to_array(v);
   store_sums<NS, T>(static_cast<T*>(a.gacc) + gi * NS, v);
+}
+
+// u / d for inv = 1 / d in float32, exact for u below 2^22: the product is within
+// u / d * 2^-23 of (u + 1/2) / d, which is less than 1 / (2 d) from it. An integer
+// division by a run-time value is a call that costs the pair loop's registers.
+__device__ __forceinline__ uint32_t quotient(uint32_t u, float inv) {
+  return (uint32_t)(((float)u + 0.5f) * inv);
 }
 
 // Grid path. The Gaussians come in (class, size, mean-cell) order, the small
@@ -595,7 +651,7 @@ bwd_grid_kernel(BwdArgs a) {
   const bool split = u < n_split * kSplitWays;
   const int64_t j = split ? n_small + u / kSplitWays : n_small + n_split + (u - n_split * kSplitWays);
   const int part = split ? (int)(u % kSplitWays) : 0;       // this unit's share of the rows
-  const int row_step = split ? kSplitWays * kWarp : kWarp;
+  const int step = split ? kSplitWays : 1;
   const Grid& Gd = a.grid;
   const int64_t gi = a.order[j];
   PairG<C, T> P;
@@ -614,13 +670,32 @@ bwd_grid_kernel(BwdArgs a) {
   const int rows = ny * nz;
   const bool xborder = lx == 0 || lx + nx - 1 == Gd.dx - 1;
   const float rcx = Gd.ox + (lx + 0.5f * nx) * cellK, rhx = 0.5f * nx * cellK * 1.001f;
+  const float inv_ny = 1.0f / (float)ny;
+  constexpr bool kTwo = two_points(C, sizeof(T));
+  PairG2<C> P2;
+  if constexpr (kTwo) double_gaussian<C>(P, P2);
   Acc<C, T> acc;
   acc.zero();
-  for (int rb = part * kWarp; rb < rows; rb += row_step) {
-    const int ri = rb + lane;
+  // this unit's blocks of 32 rows, 32 of them looked at side by side: those with
+  // no hit point between their first and their last cell are passed over (hit
+  // points lie on surfaces, and most rows of a large box are empty)
+  const int blocks = (rows + kWarp - 1) / kWarp;
+  bool any = false;
+  for (int b0 = part; b0 < blocks; b0 += kWarp * step) {
+  const int b = b0 + lane * step;
+  bool has = b < blocks;
+  if (has && blocks > 1) {
+    const int r0 = b * kWarp, r1 = min(r0 + kWarp, rows) - 1;
+    const int z0 = (int)quotient((uint32_t)r0, inv_ny), z1 = (int)quotient((uint32_t)r1, inv_ny);
+    has = a.qstart[qkey_of(Gd, lx, ly + r0 - z0 * ny, lz + z0)] <
+          a.qstart[qkey_of(Gd, lx + nx - 1, ly + r1 - z1 * ny, lz + z1) + 1];
+  }
+  for (uint32_t todo = __ballot_sync(kFullMask, has); todo; todo &= todo - 1u) {
+    const int ri = (b0 + (__ffs(todo) - 1) * step) * kWarp + lane;
     uint32_t qs = 0, cnt = 0;
     if (ri < rows) {
-      const int iy = ly + ri % ny, iz = lz + ri / ny;
+      const int sl = (int)quotient((uint32_t)ri, inv_ny);
+      const int iy = ly + ri - sl * ny, iz = lz + sl;
       const uint32_t key = qkey_of(Gd, lx, iy, iz);
       qs = a.qstart[key];
       cnt = a.qstart[key + nx] - qs;
@@ -642,6 +717,8 @@ bwd_grid_kernel(BwdArgs a) {
       if (lane >= o) incl += t;
     }
     const uint32_t tot = __shfl_sync(kFullMask, incl, 31);
+    if (tot == 0u) continue;
+    any = true;
     const uint32_t excl = incl - cnt;
     // item f of the flattened rows belongs to the non-empty row with the
     // largest start excl <= f. The non-empty rows, ranked in lane order, keep
@@ -654,455 +731,45 @@ bwd_grid_kernel(BwdArgs a) {
     if (ne) s_base[wib][__popc(ne_mask & lanemask_lt())] = qs - excl;
     __syncwarp();
     const uint32_t le = lanemask_lt() | (1u << lane);
-    for (uint32_t f0 = 0; f0 < tot; f0 += kWarp) {
-      const uint32_t f = f0 + lane;
+    // the hit point of item f: its position in the sorted order
+    auto item = [&](uint32_t f0) {
       const uint32_t starts =
           __reduce_or_sync(kFullMask, ne && excl > f0 && excl < f0 + kWarp ? 1u << (excl - f0) : 0u);
       const int r0 = __popc(__ballot_sync(kFullMask, ne && excl <= f0)) - 1;
-      if (f < tot) {
-        const int r = r0 + __popc(starts & le);
-        const uint32_t k = s_base[wib][r] + f;     // modulo 2^32: qs - excl may wrap
-        bwd_pair<C, PSI, T>(P, a.qrec + (int64_t)k * QS, a, acc);
+      const uint32_t f = f0 + lane;
+      const int r = r0 + __popc(starts & le);
+      return f < tot ? s_base[wib][r] + f : 0xffffffffu;   // modulo 2^32: qs - excl may wrap
+    };
+    if constexpr (kTwo) {
+      // two chunks at a time
+      for (uint32_t f0 = 0; f0 < tot; f0 += 2 * kWarp) {
+        const uint32_t k0 = item(f0);
+        const uint32_t k1 = f0 + kWarp < tot ? item(f0 + kWarp) : 0xffffffffu;
+        if (k0 != 0xffffffffu)
+          bwd_pair2<C, PSI>(P2, a.qrec + (int64_t)k0 * QS,
+                            a.qrec + (int64_t)(k1 != 0xffffffffu ? k1 : k0) * QS, a.cut2,
+                            k1 != 0xffffffffu ? a.cut2 : -1.0f, a, acc);
+      }
+    } else {
+      for (uint32_t f0 = 0; f0 < tot; f0 += kWarp) {
+        const uint32_t k = item(f0);
+        if (k != 0xffffffffu) bwd_pair<C, PSI, T>(P, a.qrec + (int64_t)k * QS, a, acc);
       }
     }
     __syncwarp();
+  }
+  }
+  T* dst = split ? static_cast<T*>(a.bpart) + ((j - n_small) * kSplitWays + part) * NS
+                 : static_cast<T*>(a.gacc) + gi * NS;
+  if (!any) {                                  // most parts of a huge Gaussian
+    if (lane < NS) dst[lane] = T(0);
+    continue;
   }
   T v[NS];
   acc.to_array(v);
   int slot;
   const T sum = reduce_scatter<NS, T>(v, lane, &slot);
-  T* dst = split ? static_cast<T*>(a.bpart) + ((j - n_small) * kSplitWays + part) * NS
-                 : static_cast<T*>(a.gacc) + gi * NS;
   if (NS == 32 || (lane & 1) == 0) dst[slot] = sum;
-  }
-  }  // work loop
-}
-
-// ---- the float32 grid path, two hit points to an instruction
-
-// A Gaussian with every value doubled, and the sums of the even and of the odd
-// hit points.
-template <int C>
-struct PairG2 {
-  f32x2 nmx, nmy, nmz;      // -mu
-  f32x2 M[9], phi[C];
-};
-template <int C>
-struct Acc2 {
-  f32x2 A[6], B[3], D[3], P[C];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) A[i] = 0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) B[i] = D[i] = 0;
-#pragma unroll
-    for (int c = 0; c < C; ++c) P[c] = 0;
-  }
-  static constexpr int NS = Acc<C, float>::NS;
-  __device__ __forceinline__ void to_array(float (&v)[NS]) const {
-    auto sum = [](f32x2 x) {
-      float lo, hi;
-      unpack2(x, lo, hi);
-      return lo + hi;
-    };
-#pragma unroll
-    for (int i = 0; i < 6; ++i) v[i] = sum(A[i]);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      v[6 + i] = sum(B[i]);
-      v[9 + i] = sum(D[i]);
-    }
-#pragma unroll
-    for (int c = 0; c < C; ++c) v[12 + c] = sum(P[c]);
-#pragma unroll
-    for (int i = 12 + C; i < NS; ++i) v[i] = 0.0f;
-  }
-};
-
-template <int C>
-__device__ __forceinline__ void load_gaussian2(const BwdArgs& a, int64_t gi, PairG2<C>& P) {
-  GaussianRegs G;
-  float phi[C];
-  load_gaussian<C>(a, gi, G, phi);
-  P.nmx = pack2(-G.mx, -G.mx);
-  P.nmy = pack2(-G.my, -G.my);
-  P.nmz = pack2(-G.mz, -G.mz);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) P.M[i] = pack2(G.M[i], G.M[i]);
-#pragma unroll
-  for (int c = 0; c < C; ++c) P.phi[c] = pack2(phi[c], phi[c]);
-}
-
-// One Gaussian and a pair of packed hit points: the terms of bwd_pair_q, each
-// rounded as there, without a branch per point. A point outside Q <= cut
-// (cut0, cut1: cut2, or -1 for a point past the end of the row) has weight 0,
-// which takes it out of every sum while its values are finite; where some may
-// not be (guard: header flags), they are zeroed.
-template <int C, bool PSI>
-__device__ __forceinline__ void bwd_pair2(const PairG2<C>& P, uint32_t pair, float cut0,
-                                          float cut1, const BwdArgs& a, bool guard,
-                                          Acc2<C>& acc) {
-  constexpr int PT = pair_tail(C);
-  float qf[8 + PT];
-  ld_global_v8(a.qrec + (int64_t)pair * 8, qf);
-  auto q = [&](int i) { return pack2(qf[2 * i], qf[2 * i + 1]); };
-  f32x2 dx = add2(q(0), P.nmx), dy = add2(q(1), P.nmy), dz = add2(q(2), P.nmz);
-  f32x2 u[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-    u[j] = fma2(P.M[3 * j], dx, fma2(P.M[3 * j + 1], dy, mul2(P.M[3 * j + 2], dz)));
-  const f32x2 Q = fma2(u[0], u[0], fma2(u[1], u[1], mul2(u[2], u[2])));
-  float q0, q1;
-  unpack2(Q, q0, q1);
-  const bool in0 = q0 <= cut0, in1 = q1 <= cut1;
-  if (!(in0 || in1)) return;
-#pragma unroll
-  for (int v = 0; v < PT; v += 8) ld_global_v8(a.qtail + (int64_t)pair * PT + v, qf + 8 + v);
-  f32x2 zeta = q(3), kappa = q(4), gam[C];
-#pragma unroll
-  for (int c = 0; c < C; ++c) gam[c] = q(5 + c);
-  if (guard) {
-    auto only = [&](f32x2 v) {
-      float lo, hi;
-      unpack2(v, lo, hi);
-      return pack2(in0 ? lo : 0.0f, in1 ? hi : 0.0f);
-    };
-    dx = only(dx); dy = only(dy); dz = only(dz);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) u[j] = only(u[j]);
-    zeta = only(zeta);
-    kappa = only(kappa);
-#pragma unroll
-    for (int c = 0; c < C; ++c) gam[c] = only(gam[c]);
-  }
-  f32x2 e = mul2(Q, pack2(-0.5f, -0.5f));
-  f32x2 pcoef = 0;   // 6 t / (r' |d|), the falloff's share of dw/dmu per unit w
-  if (PSI) {
-    const f32x2 d2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-    float d0, d1;
-    unpack2(d2, d0, d1);
-    // |d| and 1/|d| from one reciprocal square root; t = 0 within the radius
-    const f32x2 inv_d = pack2(rsqrt_approx(d0), rsqrt_approx(d1));
-    float t0, t1;
-    unpack2(fma2(d2, inv_d, pack2(-a.r, -a.r)), t0, t1);
-    const f32x2 irr = pack2(a.inv_rr, a.inv_rr);
-    const f32x2 t = mul2(pack2(fmaxf(t0, 0.0f), fmaxf(t1, 0.0f)), irr);
-    e = fma2(mul2(pack2(-3.0f, -3.0f), t), t, e);
-    pcoef = mul2(mul2(mul2(pack2(6.0f, 6.0f), t), irr), inv_d);
-  }
-  float e0, e1;
-  unpack2(mul2(e, pack2(kLog2e, kLog2e)), e0, e1);
-  const f32x2 w = pack2(ex2_approx(in0 ? e0 : -INFINITY), ex2_approx(in1 ? e1 : -INFINITY));
-  f32x2 gp = mul2(gam[0], P.phi[0]);
-#pragma unroll
-  for (int c = 1; c < C; ++c) gp = fma2(gam[c], P.phi[c], gp);
-  const f32x2 bw = mul2(mul2(zeta, fma2(kappa, pack2(-1.0f, -1.0f), gp)), w);
-  const f32x2 b0 = mul2(bw, u[0]), b1 = mul2(bw, u[1]), b2 = mul2(bw, u[2]);
-  acc.A[0] = fma2(b0, u[0], acc.A[0]);
-  acc.A[1] = fma2(b0, u[1], acc.A[1]);
-  acc.A[2] = fma2(b0, u[2], acc.A[2]);
-  acc.A[3] = fma2(b1, u[1], acc.A[3]);
-  acc.A[4] = fma2(b1, u[2], acc.A[4]);
-  acc.A[5] = fma2(b2, u[2], acc.A[5]);
-  acc.B[0] = add2(acc.B[0], b0);
-  acc.B[1] = add2(acc.B[1], b1);
-  acc.B[2] = add2(acc.B[2], b2);
-  if (PSI) {
-    const f32x2 pc = mul2(bw, pcoef);
-    acc.D[0] = fma2(pc, dx, acc.D[0]);
-    acc.D[1] = fma2(pc, dy, acc.D[1]);
-    acc.D[2] = fma2(pc, dz, acc.D[2]);
-  }
-  const f32x2 wz = mul2(w, zeta);
-#pragma unroll
-  for (int c = 0; c < C; ++c) acc.P[c] = fma2(gam[c], wz, acc.P[c]);
-}
-
-// The float32 grid path: the work units of bwd_grid_kernel, a lane taking two
-// neighbouring hit points at a time. A row's pairs may reach one point past
-// either end, which is left out: over empty cells it may belong to another row
-// of the same Gaussian. A small Gaussian runs on a lane
-// unless the warp does better to take it as it takes the large ones, one by one
-// (lane_limit).
-//
-// Hit points up to which a small Gaussian stays on its lane, of this warp's 32.
-// The lanes go as long as the longest of them, a pair each a round, and their
-// loads go to 32 places (kLaneRound); a Gaussian that the whole warp takes costs
-// 1/32 of its rounds, of coalesced loads, and kWholeRounds more for its rows and
-// the reduction. So a few long ones among short ones (many views of one place)
-// leave the lanes, and 32 that are alike stay up to some 130 points: the
-// doubling limit with the least cost is taken. Pair loop over 1M Gaussians with
-// query cells of 0.031 and 0.062: 0.74 and 1.11 ms at a fixed limit of 192
-// points, 0.69 and 1.65 at 768; kLaneRound 1, 2, 3, 5: 0.68, 0.62, 0.58, 0.57
-// and 1.67, 1.09, 1.09, 1.10 ms.
-constexpr uint32_t kLanePoints = 96, kLaneRound = 5, kWholeRounds = 8;
-__device__ __forceinline__ uint32_t lane_limit(uint32_t points) {
-  uint32_t limit = kLanePoints, best = 0xffffffffu, t = kLanePoints;
-  for (;;) {
-    const bool stays = points <= t;
-    const uint32_t rounds =
-        kLaneRound * (__reduce_max_sync(kFullMask, stays ? points : 0u) >> 1) +
-        __reduce_add_sync(kFullMask, stays ? 0u : (points >> 6) + kWholeRounds);
-    if (rounds < best) {
-      best = rounds;
-      limit = t;
-    }
-    if (__all_sync(kFullMask, stays)) return limit;
-    t *= 2;
-  }
-}
-// Resident blocks: the loads of the hit points are what the warps wait for, so
-// more warps win over fewer spills up to four channels (1M Gaussians, 3
-// channels: 5, 6, 7, 8 blocks per SM give a training step of 1.97, 1.90, 1.85,
-// 1.82 ms; 8 channels: 4.74, 4.86, 5.17, 6.02 ms).
-constexpr int bwd_blocks(int C) { return C <= 3 ? 8 : C == 4 ? 6 : 5; }
-// u / d for inv = 1 / d in float32: exact for u below 2^19 and d up to 1024 (the
-// quotient's error stays below half of 1 / d). An integer division by a run-time
-// value is a call that costs the pair loop's registers.
-__device__ __forceinline__ uint32_t quotient(uint32_t u, float inv) {
-  return (uint32_t)(((float)u + 0.5f) * inv);
-}
-// Units that a huge Gaussian is split into: up to kSplitWays. Halving the
-// longest unit (a Gaussian over all n_active points: 0.3 us per 64 of them)
-// costs another 4 us of loads and reduction per huge Gaussian over the 4,864
-// resident warps, so the best number is the square root of their ratio (11 K
-// points and 2,901 huge Gaussians: 4 units each take 60 us, 16 take 107).
-__device__ __forceinline__ int split_ways(const DeviceHeader* h) {
-  const float ratio = 6.0f * (float)h->n_active / (float)max(h->n_huge, 1u);
-  int ways = 1;
-  while (ways < kSplitWays && (float)((ways + 1) * (ways + 1)) <= ratio) ++ways;
-  return ways;
-}
-template <int C, bool PSI>
-__global__ void __launch_bounds__(kBwdThreads, bwd_blocks(C))
-bwd_pairs_kernel(const __grid_constant__ BwdArgs a) {
-  constexpr int NS = Acc2<C>::NS;
-  // per warp: first pair minus flattened start of each non-empty row, and the
-  // row's first and last + 1 hit point
-  __shared__ uint32_t s_base[kBwdWarps][kWarp];
-  __shared__ uint2 s_row[kBwdWarps][kWarp];
-  // ids and bounds: heavy small Gaussians by lane, then the large ones of a grab
-  __shared__ uint4 s_unit[kBwdWarps][kWarp + kGrab];
-  __shared__ uint2 s_small[kBwdWarps][4][kWarp];   // the rows of each lane's small Gaussian
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  if (index_unusable(a.header)) return;
-  const Grid& Gd = a.grid;
-  const bool guard = (a.header->wild_grad | a.header->wild_field) != 0u;
-  const uint32_t n_small = a.header->n_small;
-  const uint32_t small_warps = (n_small + kWarp - 1) / kWarp;
-  const uint32_t n_split = min(a.header->n_huge, (uint32_t)kSplitMax);
-  const uint32_t ways = (uint32_t)split_ways(a.header);
-  const uint32_t n_parts = n_split * ways;            // below 2^19
-  const float inv_ways = 1.0f / (float)ways;
-  const uint32_t n_whole = a.header->n_live - n_small - n_split;
-  const uint32_t units = small_warps + n_parts + n_whole;
-  const uint32_t fine_end = small_warps + n_parts + min(n_whole, (uint32_t)kFineLarge);
-  for (;;) {
-  uint32_t w0 = 0, grab = 0;
-  if (lane == 0) {
-    const uint32_t seen = (uint32_t)*(volatile unsigned long long*)a.next_work;
-    grab = seen + (uint32_t)kGrab > small_warps && seen < fine_end ? 1u : (uint32_t)kGrab;
-    w0 = (uint32_t)atomicAdd(a.next_work, (unsigned long long)grab);
-  }
-  w0 = __shfl_sync(kFullMask, w0, 0);
-  grab = __shfl_sync(kFullMask, grab, 0);
-  if (w0 >= units) break;
-  const uint32_t w_end = min(w0 + grab, units);
-  // the large Gaussians of these units, a unit per lane: their ids and bounds
-  // are on their way together instead of one chain of loads per unit
-  if (w0 + lane < w_end && w0 + lane >= small_warps) {
-    const uint32_t u = w0 + lane - small_warps;
-    const uint32_t gi =
-        a.order[n_small + (u < n_parts ? quotient(u, inv_ways) : n_split + (u - n_parts))];
-    const uint2 qb = a.qbox[gi];
-    s_unit[wib][kWarp + lane] = make_uint4(gi, qb.x, qb.y, 0u);
-  }
-  __syncwarp();
-  for (uint32_t w = w0; w < w_end; ++w) {
-    // the Gaussians that the whole warp takes: s_unit[base + l] for every bit l
-    uint32_t todo = 1u, base = kWarp + (w - w0);
-    int split_at = -1;                         // slot of the split sums, or none
-    uint32_t part = 0, parts = 1;              // this unit's share of the row blocks
-    if (w < small_warps) {
-      const uint32_t idx = w * kWarp + lane;
-      uint32_t mine = 0, points = 0;
-      uint2 box = make_uint2(0u, 0u);
-      // at most 2 x 2 rows
-      uint2 row[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) row[r] = make_uint2(0u, 0u);
-      if (idx < n_small) {
-        mine = a.order[idx];
-        box = a.qbox[mine];
-        uint32_t lo[3], hi[3];
-        unpack_qbox(box, lo, hi);
-        const uint32_t nx = hi[0] - lo[0] + 1;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const uint32_t iy = lo[1] + (r & 1), iz = lo[2] + (r >> 1);
-          if (iy <= hi[1] && iz <= hi[2]) {
-            const uint32_t key = qkey_of(Gd, lo[0], iy, iz);
-            row[r] = make_uint2(a.qstart[key], a.qstart[key + nx]);
-            points += row[r].y - row[r].x;
-          }
-        }
-      }
-      const bool heavy = points > lane_limit(points);
-      if (idx < n_small) {
-        if (heavy) {
-          s_unit[wib][lane] = make_uint4(mine, box.x, box.y, 0u);
-        } else {
-          PairG2<C> P;
-          load_gaussian2<C>(a, mine, P);
-          Acc2<C> acc;
-          acc.zero();
-          // one loop over the pairs of all rows: the lanes change rows each on
-          // its own, so the warp takes the longest lane's pairs, not the sum of
-          // each row's longest
-#pragma unroll
-          for (int r = 0; r < 4; ++r) s_small[wib][r][lane] = row[r];
-          int r = -1;
-          uint2 rw = make_uint2(0u, 0u);
-          uint32_t p = 0, end = 0;
-          for (;;) {
-            while (p >= end && ++r < 4) {
-              rw = s_small[wib][r][lane];
-              p = rw.x >> 1;
-              end = rw.x < rw.y ? (rw.y + 1) >> 1 : p;
-            }
-            if (p >= end) break;
-            bwd_pair2<C, PSI>(P, p, 2 * p < rw.x ? -1.0f : a.cut2,
-                              2 * p + 1 >= rw.y ? -1.0f : a.cut2, a, guard, acc);
-            ++p;
-          }
-          float v[NS];
-          acc.to_array(v);
-          store_sums<NS, float>(static_cast<float*>(a.gacc) + (int64_t)mine * NS, v);
-        }
-      }
-      todo = __ballot_sync(kFullMask, heavy);
-      base = 0;
-      __syncwarp();
-    } else {
-      const uint32_t u = w - small_warps;
-      if (u < n_parts) {
-        const uint32_t q = quotient(u, inv_ways);
-        part = u - q * ways;
-        parts = ways;
-        split_at = (int)(q * kSplitWays + part);
-      }
-    }
-    for (; todo; todo &= todo - 1u) {
-      // (through shuffles: read from shared memory at one address for all lanes,
-      // they make the compiler take the rows' loops into uniform registers and
-      // spill 600 bytes of the pair loop's instead of 150)
-      const uint4 un = s_unit[wib][base + __ffs(todo) - 1];
-      const uint32_t gi = __shfl_sync(kFullMask, un.x, 0);
-      PairG2<C> P;
-      load_gaussian2<C>(a, gi, P);
-      uint32_t lo[3], hi[3];
-      unpack_qbox(make_uint2(__shfl_sync(kFullMask, un.y, 0), __shfl_sync(kFullMask, un.z, 0)), lo, hi);
-      const int lx = (int)lo[0], ly = (int)lo[1], lz = (int)lo[2];
-      const int nx = (int)hi[0] - lx + 1, ny = (int)hi[1] - ly + 1, nz = (int)hi[2] - lz + 1;
-      const float inv_ny = 1.0f / (float)ny;
-      const float cut_keep = a.cut * 1.0001f;
-      const float cellK = Gd.cell0 * (float)(1u << Gd.qlevel);
-      const float half = 0.5f * cellK * 1.001f;
-      // the cells lx..hx of one (iy, iz) row have consecutive keys, so the row's
-      // hit points are one contiguous range of the sorted order
-      const bool xborder = lx == 0 || lx + nx - 1 == Gd.dx - 1;
-      const float rcx = Gd.ox + (lx + 0.5f * nx) * cellK, rhx = 0.5f * nx * cellK * 1.001f;
-      Acc2<C> acc;
-      acc.zero();
-      // rows of the z slabs that hold a hit point between their first and last
-      // row: hit points lie on surfaces, and most slabs of a large box are empty
-      // (up to 32 rows go without the look)
-      uint32_t block = 0;
-      for (int zb = 0; zb < nz; zb += kWarp) {
-      bool has = zb + lane < nz;
-      if (has && ny * nz > kWarp)
-        has = a.qstart[qkey_of(Gd, lx, ly, lz + zb + lane)] <
-              a.qstart[qkey_of(Gd, lx + nx - 1, ly + ny - 1, lz + zb + lane) + 1];
-      const uint32_t slabs = __ballot_sync(kFullMask, has);
-      const int rows = __popc(slabs) * ny;
-      for (int rb = 0; rb < rows; rb += kWarp) {
-        if (parts > 1) {                       // every parts-th block, from the part-th
-          const bool ours = block == part;
-          block = block + 1 == parts ? 0 : block + 1;
-          if (!ours) continue;
-        }
-        const int ri = rb + lane;
-        uint32_t qs = 0, qe = 0;
-        if (ri < rows) {
-          const int sl = (int)quotient((uint32_t)ri, inv_ny);
-          const int iy = ly + ri - sl * ny;
-          const int iz = lz + zb + (int)nth_bit(slabs, (uint32_t)sl);
-          const uint32_t key = qkey_of(Gd, lx, iy, iz);
-          qs = a.qstart[key];
-          qe = a.qstart[key + nx];
-          // border cells also hold the clamped points outside the grid: no cull
-          const bool border = xborder || iy == 0 || iz == 0 || iy == Gd.dy - 1 || iz == Gd.dz - 1;
-          if (qe > qs && !border) {
-            float M[9], nmx, nmy, nmz, t;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) unpack2(P.M[i], M[i], t);
-            unpack2(P.nmx, nmx, t);
-            unpack2(P.nmy, nmy, t);
-            unpack2(P.nmz, nmz, t);
-            const float lb = box_distance(M, rcx + nmx, Gd.oy + (iy + 0.5f) * cellK + nmy,
-                                          Gd.oz + (iz + 0.5f) * cellK + nmz, rhx, half, half);
-            if (lb > cut_keep) qe = qs;
-          }
-        }
-        // flatten the pairs of these (up to 32) rows over the lanes
-        const uint32_t cnt = qe > qs ? ((qe + 1) >> 1) - (qs >> 1) : 0u;
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
-          if (lane >= o) incl += t;
-        }
-        const uint32_t tot = __shfl_sync(kFullMask, incl, 31);
-        const uint32_t excl = incl - cnt;
-        // item f of the flattened rows belongs to the non-empty row with the
-        // largest start excl <= f. The non-empty rows, ranked in lane order, keep
-        // (first pair - start) in shared memory; a chunk's owner ranks come
-        // from the starts that fall inside it (a bit per start, OR-reduced over
-        // the warp) counted up to each lane, on top of the rank of the row that
-        // holds the chunk's first item.
-        const bool ne = cnt > 0;
-        const uint32_t ne_mask = __ballot_sync(kFullMask, ne);
-        if (ne) {
-          const int r = __popc(ne_mask & lanemask_lt());
-          s_base[wib][r] = (qs >> 1) - excl;
-          s_row[wib][r] = make_uint2(qs, qe);
-        }
-        __syncwarp();
-        const uint32_t le = lanemask_lt() | (1u << lane);
-        for (uint32_t f0 = 0; f0 < tot; f0 += kWarp) {
-          const uint32_t f = f0 + lane;
-          const uint32_t starts = __reduce_or_sync(
-              kFullMask, ne && excl > f0 && excl < f0 + kWarp ? 1u << (excl - f0) : 0u);
-          const int r0 = __popc(__ballot_sync(kFullMask, ne && excl <= f0)) - 1;
-          if (f < tot) {
-            const int r = r0 + __popc(starts & le);
-            const uint32_t p = s_base[wib][r] + f;     // modulo 2^32: the base may wrap
-            const uint2 rw = s_row[wib][r];
-            bwd_pair2<C, PSI>(P, p, 2 * p < rw.x ? -1.0f : a.cut2,
-                              2 * p + 1 >= rw.y ? -1.0f : a.cut2, a, guard, acc);
-          }
-        }
-        __syncwarp();
-      }
-      }
-      float v[NS];
-      acc.to_array(v);
-      int slot;
-      const float sum = reduce_scatter<NS, float>(v, lane, &slot);
-      float* dst = split_at >= 0 ? static_cast<float*>(a.bpart) + (int64_t)split_at * NS
-                                 : static_cast<float*>(a.gacc) + (int64_t)gi * NS;
-      if (NS == 32 || (lane & 1) == 0) dst[slot] = sum;
-    }
   }
   }  // work loop
 }
@@ -1178,10 +845,9 @@ __global__ void bwd_split_combine_kernel(BwdArgs a) {
   if (s >= n_split) return;
   const int64_t gi = a.order[(int64_t)a.header->n_small + s];
   const T* p = static_cast<const T*>(a.bpart) + s * kSplitWays * NS + i;
-  const int ways = sizeof(T) == 4 ? split_ways(a.header) : kSplitWays;
   T part[kSplitWays];
 #pragma unroll
-  for (int b = 0; b < kSplitWays; ++b) part[b] = b < ways ? p[b * NS] : T(0);
+  for (int b = 0; b < kSplitWays; ++b) part[b] = p[b * NS];
   T v = part[0];
 #pragma unroll
   for (int b = 1; b < kSplitWays; ++b) v += part[b];
@@ -1236,18 +902,9 @@ cudaError_t launch_ct(const BwdArgs& a, const IndexDims& d, bool psi, const Kern
     note_launches(1);
     return cudaGetLastError();
   }
-  const bool pairs = sizeof(T) == 4 && !a.nbrange && !d.brute;
-  cudaError_t e;
-  // the work counter and the flag of the packed hit points' values
-  if (!a.nbrange && !d.brute &&
-      (e = cudaMemsetAsync(a.next_work, 0, sizeof(unsigned long long) + sizeof(uint32_t),
-                           stream)) != cudaSuccess)
-    return e;
-  if (pairs)
-    pack_pairs_kernel<C><<<(unsigned)(((a.m + 1) / 2 + 255) / 256), 256, 0, stream>>>(a);
-  else
-    pack_qrec_kernel<C><<<(unsigned)((a.m + 255) / 256), 256, 0, stream>>>(a);
+  pack_qrec_kernel<C><<<(unsigned)((a.m + 255) / 256), 256, 0, stream>>>(a);
   note_launches(1);
+  cudaError_t e;
   if (a.nbrange) {
     // the hybrid neighbourhood: a warp per Gaussian over its selected pairs
     const int64_t want = (a.n * kWarp + kBwdThreads - 1) / kBwdThreads;
@@ -1265,18 +922,15 @@ cudaError_t launch_ct(const BwdArgs& a, const IndexDims& d, bool psi, const Kern
   // brute force: a warp per Gaussian; grid: up to n / 32 lane warps + n warps
   const int64_t warps = d.brute ? a.n : a.n + (a.n + kWarp - 1) / kWarp;
   const unsigned blocks = (unsigned)((warps + kBwdWarps - 1) / kBwdWarps);
+  if (!d.brute &&
+      (e = cudaMemsetAsync(a.next_work, 0, sizeof(unsigned long long), stream)) != cudaSuccess)
+    return e;
   if (ev.start && (e = cudaEventRecord(ev.start, stream)) != cudaSuccess) return e;
   if (d.brute) {
     if (psi) bwd_brute_kernel<C, true, T><<<blocks, kBwdThreads, 0, stream>>>(a);
     else bwd_brute_kernel<C, false, T><<<blocks, kBwdThreads, 0, stream>>>(a);
-  } else if constexpr (sizeof(T) == 4) {
-    // persistent: as many blocks as can be resident at once
-    const void* kfn = psi ? reinterpret_cast<const void*>(&bwd_pairs_kernel<C, true>)
-                          : reinterpret_cast<const void*>(&bwd_pairs_kernel<C, false>);
-    const unsigned gblocks = (unsigned)persistent_blocks(kfn, kBwdThreads, blocks);
-    if (psi) bwd_pairs_kernel<C, true><<<gblocks, kBwdThreads, 0, stream>>>(a);
-    else bwd_pairs_kernel<C, false><<<gblocks, kBwdThreads, 0, stream>>>(a);
   } else {
+    // persistent: as many blocks as can be resident at once
     const void* kfn = psi ? reinterpret_cast<const void*>(&bwd_grid_kernel<C, true, T>)
                           : reinterpret_cast<const void*>(&bwd_grid_kernel<C, false, T>);
     const unsigned gblocks = (unsigned)persistent_blocks(kfn, kBwdThreads, blocks);
@@ -1315,17 +969,14 @@ cudaError_t launch_backward(const IndexDims& d, const IndexBuffers& b, const gpf
   BwdArgs a;
   a.grid = d.grid;
   a.header = b.header;
-  a.qval = b.qval[b.qsorted];
   a.qpos = b.qpos;
   a.qstart = b.qstart;
-  a.x = q.x;
   a.albedo = q.albedo;
   a.grad_out = grad_out;
   a.out = out;
   a.z = z;
   a.m = q.m;
   a.qrec = b.qrec;
-  a.qtail = b.qrec + (q.m + 1) / 2 * 8;
   a.gacc = b.gacc;
   a.glive = b.glive;
   a.qbox = b.qbox;

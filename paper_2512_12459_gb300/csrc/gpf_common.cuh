@@ -35,15 +35,12 @@ struct DeviceHeader {
   unsigned long long n_heavy;         // forward: tiles deferred to the second launch
   unsigned long long next_tile;       // forward: next tile of 32 hit points
   unsigned long long next_work;       // backward: next work item
-  uint32_t wild_grad;    // backward: 1 if a packed hit point holds a non-finite value
-  uint32_t wild_field;   // 1 if a coordinate or 1/scale is so large that a pair's
-                         // u = M (x - mu) could overflow
   uint32_t nonfinite;    // 1 if a Gaussian parameter or an active hit point is not finite
   uint32_t nb_pairs;     // (hit point, Gaussian) pairs of the last hybrid backward
   uint32_t n_xunits;     // work units of the split forward tiles (<= GPF_MAX_SPLIT_UNITS)
   uint32_t n_hunits;     // work units of the split hybrid forward tiles (same limit)
   unsigned long long split_cost;  // estimated work of all forward tiles
-  uint32_t pad[40];
+  uint32_t pad[42];
 };
 static_assert(sizeof(DeviceHeader) == 256, "header is one 256-byte block");
 
@@ -112,22 +109,11 @@ __host__ __device__ constexpr int rec_stride(int channels) {
 // Packed hit point of the backward, float32, stride qrec_stride(C):
 //   [0..2] x, [3] zeta = 1/max(Z,eps) (1 in SUM mode),
 //   [4] kappa = sum_c g_c O_c (0 in SUM mode or when Z <= eps),
-//   [5..] gamma_c = g_c rho_c, then zero padding to a multiple of 4 floats
+//   [5..] gamma_c = g_c rho_c, then zero padding to a multiple of 8 floats (whole
+//   32-byte loads)
 __host__ __device__ constexpr int qrec_stride(int channels) {
-  return 4 * ((5 + channels + 3) / 4);
+  return 8 * ((5 + channels + 7) / 8);
 }
-// The float32 backward's packed hit points: two neighbours of the sorted order
-// interleaved value by value, so that each value of both is one operand of the
-// packed arithmetic. Their positions and zeta (8 floats) lie in one array, read
-// by every test, kappa and gamma (padded to 8 floats) in a second one, read by
-// the pairs that pass.
-__host__ __device__ constexpr int pair_tail(int channels) {
-  return 8 * ((2 * (1 + channels) + 7) / 8);
-}
-__host__ __device__ constexpr int pair_stride(int channels) { return 8 + pair_tail(channels); }
-// Above these a float32 pair could overflow on the way (kWildInvScale * 2
-// kWildCoord stays below the largest float).
-constexpr float kWildCoord = 1e8f, kWildInvScale = 1e29f;
 // Per-Gaussian sums of the backward (A 6, B 3, D 3, dPhi C), zero padded.
 __host__ __device__ constexpr int gacc_stride(int channels) {
   return 12 + channels <= 16 ? 16 : 32;

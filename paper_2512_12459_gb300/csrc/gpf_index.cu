@@ -232,10 +232,10 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
   const int64_t n = f.n;
   const int64_t n_groups = group_count(n, (int)blockDim.x);
   uint32_t level_bits = 0;
-  uint32_t v[4] = {0u, 0u, 0u, 0u};    // live, small, huge, (bad, wild << 16) of this thread
+  uint32_t v[4] = {0u, 0u, 0u, 0u};    // live, small, huge, bad of this thread
   for (int64_t group = blockIdx.x; group < n_groups; group += gridDim.x) {
   const int64_t g = group * blockDim.x + threadIdx.x;
-  bool live = false, small = false, huge = false, bad = false, wild = false;
+  bool live = false, small = false, huge = false, bad = false;
   uint32_t order_key = 0, entries = 0;
   if (g < n) {
     const float* mean = static_cast<const float*>(f.mean);
@@ -359,17 +359,12 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
       rec[g * rs + c] = sv;
     }
     bad = nf != 0u;
-    float big = 0.0f;
-#pragma unroll
-    for (int v = 4; v < 13; ++v) big = fmaxf(big, fabsf(rv[v]));
-    wild = big > kWildInvScale ||
-           fmaxf(fabsf(mu[0]), fmaxf(fabsf(mu[1]), fabsf(mu[2]))) > kWildCoord;
   }
   count_digits(order_key, g < n, passes, s_digits);
   v[0] += live;
   v[1] += small;
   v[2] += huge;
-  v[3] |= (bad ? 1u : 0u) | (wild ? 0x10000u : 0u);
+  v[3] |= bad;
   if (gpart) {
     const uint32_t ent = __reduce_add_sync(kFullMask, entries);
     if ((threadIdx.x & 31) == 0 && ent) {
@@ -391,8 +386,7 @@ preprocess_kernel(gpf_field f, Grid grid, float cutoff, int brute,
     if (v[0]) atomicAdd(&header->n_live, v[0]);
     if (v[1]) atomicAdd(&header->n_small, v[1]);
     if (v[2]) atomicAdd(&header->n_huge, v[2]);
-    if (v[3] & 0xffffu) atomicExch(&header->nonfinite, 1u);
-    if (v[3] >> 16) atomicExch(&header->wild_field, 1u);
+    if (v[3]) atomicExch(&header->nonfinite, 1u);
   }
   flush_digits(s_digits, passes, digit_counts);
 }
@@ -407,11 +401,11 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
   __shared__ uint32_t s_digits[kSortMaxPasses * kSortBins];   // of the sort keys
   for (int d = threadIdx.x; d < passes * kSortBins; d += blockDim.x) s_digits[d] = 0;
   __syncthreads();
-  uint32_t v[4] = {0u, 0u, 0u, 0u};      // active, bad, wild hit points of this thread
+  uint32_t v[4] = {0u, 0u, 0u, 0u};            // active, bad hit points of this thread
   const int64_t chunks = (m + kThreads - 1) / kThreads;
   for (int64_t chunk = blockIdx.x; chunk < chunks; chunk += gridDim.x) {
   const int64_t i = chunk * kThreads + threadIdx.x;
-  bool active = false, bad = false, wild = false;
+  bool active = false, bad = false;
   uint32_t k = grid.key_inactive;  // sort key
   uint32_t c0[3] = {0u, 0u, 0u};   // level-0 cell of an active hit point
   if (i < m) {
@@ -435,7 +429,6 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
     active = facing && (valid == nullptr || valid[i] != 0);
     if (active) {
       bad = !(isfinite(x[i]) && isfinite(x[m + i]) && isfinite(x[2 * m + i]));
-      wild = fmaxf(fabsf(x[i]), fmaxf(fabsf(x[m + i]), fabsf(x[2 * m + i]))) > kWildCoord;
       const uint32_t cx = coord0(x[i], grid.ox, grid.inv_cell0, grid.max0x);
       const uint32_t cy = coord0(x[m + i], grid.oy, grid.inv_cell0, grid.max0y);
       const uint32_t cz = coord0(x[2 * m + i], grid.oz, grid.inv_cell0, grid.max0z);
@@ -496,14 +489,12 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
   count_digits(k, i < m, passes, s_digits);
   v[0] += active;
   v[1] |= bad;
-  v[2] |= wild;
   }  // chunks
   __shared__ uint32_t s_cnt[kBlockWarps][4];
   block_counts(v, s_cnt);     // its __syncthreads also orders s_digits
   flush_digits(s_digits, passes, digit_counts);
   if (threadIdx.x == 0 && v[0]) atomicAdd(&header->n_active, v[0]);
   if (threadIdx.x == 0 && v[1]) atomicExch(&header->nonfinite, 1u);
-  if (threadIdx.x == 0 && v[2]) atomicExch(&header->wild_field, 1u);
 }
 
 // One (bucket, Gaussian) entry per occupied cell of every Gaussian's level

@@ -1,0 +1,57 @@
+"""Values and sizes at which a branch of the build or of the pair loops changes
+its mind, beside those of test_gpu_paths.py."""
+
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpf():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2512_12459_gb300 as g
+    return g
+
+
+@pytest.mark.parametrize("channels", [3, 4, 8])
+@pytest.mark.parametrize("cell", [0.02, 0.3])
+def test_products_that_overflow_reach_their_own_gaussians_only(gpf, channels, cell):
+    """A finite upstream value whose product with a spectrum is infinite: the
+    Gaussians that include that hit point get it, the others nothing of it."""
+    import torch
+    from paper_2512_12459_gb300.setup_index import make_index
+    fnp, qnp = synth.config1_random(seed=78, n=1500, m=3001, channels=channels)
+    fnp.spectrum = (fnp.spectrum + 10.0).astype(np.float32)
+    field, queries = gpf.Field.from_numpy(fnp), gpf.Queries.from_numpy(qnp)
+    act = np.flatnonzero(np.sum(qnp.n.astype(np.float64) * qnp.wo, axis=0) > 0)
+    p = int(act[len(act) // 2])
+    ref = oracle.radiance_fwd(fnp.mean, fnp.quat, fnp.logscale, fnp.spectrum, qnp.x[:, [p]],
+                              qnp.n[:, [p]], qnp.wo[:, [p]], mode=oracle.GPF_SUM, r_max=math.inf,
+                              cutoff_sigma=3.0)
+    assert not ref["near_cutoff"][0]
+    G = torch.randn((channels, qnp.m), generator=torch.Generator("cuda").manual_seed(4),
+                    device="cuda")
+    idx = make_index(field, queries, query_cell=cell)
+    idx.build(field, queries)
+    grads = []
+    for v in (0.0, 2e38):
+        H = G.clone()
+        H[:, p] = v
+        grads.append(gpf.gpf_radiance_bwd(idx, field, queries, H, mode=gpf.GPF_SUM))
+    bad = ~torch.isfinite(grads[1].logscale[0])
+    d = qnp.x[:, [p]].astype(np.float64) - fnp.mean
+    assert 0 < int(bad.sum()) <= int((np.linalg.norm(d, axis=0)
+                                      <= 3.0 * np.exp(fnp.logscale.max(axis=0)) * 1.001).sum())
+    # (a Gaussian may include the point with a finite term: those that change at all)
+    near = torch.from_numpy(np.linalg.norm(d, axis=0)
+                            <= 3.0 * np.exp(fnp.logscale.max(axis=0)) * 1.001).cuda()
+    for a, b in zip(grads[0].tensors(), grads[1].tensors()):
+        assert torch.equal(a[:, ~near], b[:, ~near])
