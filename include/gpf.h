@@ -222,15 +222,15 @@ typedef struct gpf_grid_config {
                             neighbourhoods hold more pairs sets the capacity
                             flag and leaves its gradients untouched.         */
   int32_t split_items;   /* forward load balance: 0 = every tile of 32 hit
-                            points is one work unit; > 0 = the build
-                            estimates each tile's work (the list entries its
-                            points walk) and splits a tile above this many
-                            (and above its share of all tiles' work) into up
-                            to GPF_MAX_TILE_PARTS units over disjoint chunks
-                            of its lists, whose partial sums a final
-                            kernel adds in part order (results still
-                            deterministic; they differ from the unsplit sums
-                            by summation order only)                         */
+                            points is summed whole by one warp; > 0 = the
+                            build estimates each tile's work (the list
+                            entries its points walk), a tile above this many
+                            has up to GPF_MAX_TILE_PARTS parts over disjoint
+                            chunks of its lists, added in part order, and a
+                            tile above its share of all tiles' work is given
+                            to several warps, some parts each (results
+                            still deterministic; they differ from the unsplit
+                            sums by summation order only)                    */
   int32_t tile_order;    /* order of the hit points inside each query-level
                             cell, which shapes the forward's 32-point tiles:
                             0 = hit point index order; b = 1 or 2 = by the

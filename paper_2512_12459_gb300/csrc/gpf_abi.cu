@@ -114,6 +114,8 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
     if (d.grid.fwords)
       t.focc = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * focc_words(d.grid)));
   }
+  if (d.split_items > 0)
+    t.xpart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tile_groups(tiles) + 1)));
   t.clear_bytes = off;
   t.rec = reinterpret_cast<float*>(take(sizeof(float) * N * rec_stride(d.channels)));
   t.vet = reinterpret_cast<VetRec*>(take(sizeof(VetRec) * N));
@@ -144,6 +146,7 @@ size_t layout(const gpf_index* ix, char* base, IndexBuffers* b) {
   t.dec = d.bf16 ? reinterpret_cast<float*>(take(sizeof(float) * (10 + d.channels) * N)) : nullptr;
   if (d.split_items > 0) {
     t.tparts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
+    t.tcost = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.xunit = reinterpret_cast<uint4*>(take(sizeof(uint4) * GPF_MAX_SPLIT_UNITS));
     t.xheavy = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (tiles + 1)));
     t.xsum = reinterpret_cast<float*>(

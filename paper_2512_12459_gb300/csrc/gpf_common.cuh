@@ -37,10 +37,11 @@ struct DeviceHeader {
   unsigned long long next_work;       // backward: next work item
   uint32_t nonfinite;    // 1 if a Gaussian parameter or an active hit point is not finite
   uint32_t nb_pairs;     // (hit point, Gaussian) pairs of the last hybrid backward
-  uint32_t n_xunits;     // work units of the split forward tiles (<= GPF_MAX_SPLIT_UNITS)
+  uint32_t n_xunits;     // units of the forward tiles that several warps take
   uint32_t n_hunits;     // work units of the split hybrid forward tiles (same limit)
   unsigned long long split_cost;  // estimated work of all forward tiles
-  uint32_t pad[42];
+  uint32_t n_xslots;     // slots of their parts' sums
+  uint32_t pad[41];
 };
 static_assert(sizeof(DeviceHeader) == 256, "header is one 256-byte block");
 
@@ -184,35 +185,35 @@ __host__ __device__ __forceinline__ uint32_t qkey_of(const Grid& g, uint32_t ix,
   return (iz * (uint32_t)g.dy + iy) * (uint32_t)g.dx + ix;
 }
 
-// Hash of the cell (ix, iy, iz) of level L: an odd multiple of each coordinate,
-// summed, through the 32-bit finaliser of MurmurHash3 (Appleby 2011; one to
-// one, so different sums never share both bucket and tag by chance of the
-// mixing). The top hash_bits bits pick the bucket; the low bits, shifted above
-// the id bits, tag the entry words so that entries of other cells sharing the
-// bucket are told apart without a memory access (a false match is caught by
-// the box test). 12 instructions against about 35 of a 64-bit mixer: the build
-// hashes every level of every hit point and every cell of every box.
+// Hash of the cell (ix, iy, iz) of level L: the 64-bit packed cell through
+// the splitmix64 finaliser (Steele, Lea and Flood 2014). The top hash_bits
+// bits pick the bucket; the low bits, shifted above the id bits, tag the
+// entry words so that entries of other cells sharing the bucket are told
+// apart without a memory access (a false match is caught by the box test).
+// Which cells share a bucket decides on which lane a pooled entry is summed,
+// so the hash is part of the order of the forward's sums.
 struct CellHash {
   uint32_t bucket;
   uint32_t tag;     // entry word bits above id_bits
 };
 // Salt of the centre-cell keys (one entry per Gaussian, in the cell of its
 // mean on the centre level): a key space apart from the box entries'.
-constexpr uint32_t kCentreSalt = 0xd192ed03u;
+constexpr uint64_t kCentreSalt = 0xd1b54a32d192ed03ull;
 
 __host__ __device__ __forceinline__ CellHash cell_hash(const Grid& g, int L, uint32_t ix,
                                                        uint32_t iy, uint32_t iz,
-                                                       uint32_t salt = 0) {
-  uint32_t z = ix * 0x9e3779b1u + iy * 0x85ebca77u + iz * 0xc2b2ae3du + (uint32_t)L * 0x27d4eb2fu +
-               salt;
-  z = (z ^ (z >> 16)) * 0x85ebca6bu;
-  z = (z ^ (z >> 13)) * 0xc2b2ae35u;
-  z ^= z >> 16;
+                                                       uint64_t salt = 0) {
+  uint64_t z = ((uint64_t)ix | ((uint64_t)iy << 20) | ((uint64_t)iz << 40) |
+                ((uint64_t)L << 60)) ^ salt;
+  z += 0x9e3779b97f4a7c15ull;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+  z ^= z >> 31;
   CellHash h;
-  h.bucket = z >> (32 - g.hash_bits);
+  h.bucket = (uint32_t)(z >> (64 - g.hash_bits));
   // (a centre entry and a box entry of one Gaussian in one bucket never have the
   // same tag: the highest bit tells them apart)
-  h.tag = ((z << g.id_bits) & 0x7fffffffu) | (salt ? 0x80000000u : 0u);
+  h.tag = (((uint32_t)z << g.id_bits) & 0x7fffffffu) | (salt ? 0x80000000u : 0u);
   return h;
 }
 // [start, end) of a bucket's list ([0, 0): it has none).

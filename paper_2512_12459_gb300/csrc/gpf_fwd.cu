@@ -13,8 +13,8 @@
 //     lower bound of their Mahalanobis distance to the box, staged in shared
 //     memory, and every lane evaluates all of them at its own hit point.
 //   * levels with many distinct cells (the Gaussians are small next to the
-//     spacing of the hit points) are pooled: the lanes' own lists, of all these
-//     levels, are laid end to end and taken 32 (hit point, entry) items at a
+//     spacing of the hit points) are pooled: the lanes' own lists are laid end to
+//     end, a level after the other, and taken 32 (hit point, entry) items at a
 //     time, one per lane; a segmented sum over the lanes returns each hit
 //     point's share to its lane.
 // Every lane applies the exact predicate Q <= k^2, so the result equals the
@@ -36,6 +36,7 @@ constexpr int kFwdWarps = 4;
 constexpr int kFwdThreads = kFwdWarps * kWarp;
 // Units of a tile's estimated work (tile_cost_kernel).
 constexpr uint32_t kCostPerEntry = 8, kCostPerTile = 8 * 32 * 10;
+constexpr uint32_t kTileUnits = 0x80000000u;   // of a tile's parts: taken by several units
 constexpr int kQueue = 128;   // vetted ids of a warp that wait for their records
 
 struct FwdArgs {
@@ -60,11 +61,11 @@ struct FwdArgs {
   float* out;              // [C,M]
   float* z;                // [M] or null
   unsigned long long* counts;  // count mode: [candidates, included]
-  const uint32_t* tparts;  // split forward: parts of each tile (null: no splitting)
-  uint4* xunit;            // split forward: (tile, part, parts, valid) of each split unit
-  uint32_t* xheavy;        // split forward: tiles deferred to the second launch
+  const uint32_t* tparts;  // split forward: parts of each tile, kTileUnits (null: no splitting)
+  const uint4* xunit;      // split forward: (tile, unit of units and parts, first slot) of each unit
+  uint32_t* xheavy;        // disk kernel: tiles deferred to the second launch
   int late;                // 1: the second launch, over the deferred tiles
-  float* xsum;             // split forward: [unit][C + 1][32] partial sums
+  float* xsum;             // split forward: [slot][C + 1][32] partial sums
 };
 
 __device__ __forceinline__ float warp_min(float v) {
@@ -160,14 +161,16 @@ __host__ __device__ constexpr int stage_fields(int C) { return 12 + C; }
 
 // Every staged record of the walked levels at this lane's hit point, four at a
 // time as straight-line code, two records to an instruction: the evaluation is
-// bound by the instructions it issues, about 23 per record packed and 40 not.
+// bound by the instructions it issues, about 25 per record packed and 40 not.
 // Every value is rounded as in pair_weight. nk is a multiple of 4: the slots
 // past the last record hold a NaN mean, which fails Q <= k^2, and finite Phi,
-// so their weight is 0. L and Z keep the even and the odd records' sums apart.
+// so their weight is 0. The sums take the records in turn, a scalar operation
+// each: sums of the even and the odd records apart would save 2 of 25
+// instructions a record and change the order.
 template <int C, int KERN>
 __device__ __forceinline__ void eval_staged(const float* __restrict__ st, int nk, float px,
                                             float py, float pz, const FwdArgs& a,
-                                            f32x2 (&L)[C], f32x2& Z) {
+                                            float (&L)[C], float& Z) {
   const f32x2 px2 = pack2(px, px), py2 = pack2(py, py), pz2 = pack2(pz, pz);
   const f32x2 c_e = pack2(-kNegHalfLog2e, -kNegHalfLog2e);
   const f32x2 c_neg = pack2(-1.0f, -1.0f), c_half = pack2(0.5f, 0.5f);
@@ -227,12 +230,15 @@ __device__ __forceinline__ void eval_staged(const float* __restrict__ st, int nk
         }
       }
     }
+    float v[4];
+    unpack2(w[0], v[0], v[1]);
+    unpack2(w[1], v[2], v[3]);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      const ulonglong2 phi = field(12 + c);
-      L[c] = fma2(w[1], phi.y, fma2(w[0], phi.x, L[c]));
+      const float4 phi = *reinterpret_cast<const float4*>(st + (12 + c) * kWarp + s);
+      L[c] = fmaf(v[3], phi.w, fmaf(v[2], phi.z, fmaf(v[1], phi.y, fmaf(v[0], phi.x, L[c]))));
     }
-    Z = add2(add2(Z, w[0]), w[1]);
+    Z = ((Z + v[0]) + v[1]) + v[2] + v[3];
   }
 }
 
@@ -344,8 +350,9 @@ struct WarpShared {
                            // (centre.z, half extents)
   uint2* range;            // [levels][32]
   unsigned long long* cell;  // [segments + 3] pack_cell
-  uint4* seg;              // [segments] entries before it, first entry of its list - those,
-                           // tag, level | first segment of that level << 8
+  uint4* seg;              // [segments + 1] where it begins in the stream, first entry of its
+                           // list - that, tag, level | first segment of that level << 8 |
+                           // entries of its last chunk - 1 << 16
   uint32_t* queue;         // [kQueue]
 };
 __host__ __device__ constexpr int stage_words(int C) {
@@ -354,7 +361,7 @@ __host__ __device__ constexpr int stage_words(int C) {
 __host__ __device__ constexpr int warp_shared_words(int C, int levels, int coop) {
   // (the cells' count rounded up to even, for 16-byte pieces)
   return stage_words(C) + (C + 1) * kWarp + 12 + 2 * levels * kWarp +
-         (levels * coop + 4) / 2 * 2 * 2 + levels * coop * 4 + kQueue;
+         (levels * coop + 4) / 2 * 2 * 2 + (levels * coop + 1) * 4 + kQueue;
 }
 template <int C>
 __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int levels, int coop) {
@@ -371,7 +378,7 @@ __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int leve
   w.cell = reinterpret_cast<unsigned long long*>(p);
   p += (levels * coop + 4) / 2 * 2 * 2;
   w.seg = reinterpret_cast<uint4*>(p);
-  p += levels * coop * 4;
+  p += (levels * coop + 1) * 4;
   w.queue = reinterpret_cast<uint32_t*>(p);
   return w;
 }
@@ -381,17 +388,26 @@ __device__ __forceinline__ WarpShared warp_shared(float* base, int wib, int leve
 // resident warps, long and short scoreboard the largest stalls, DRAM 5 %). So
 // the lists of a tile are walked as one stream of full chunks, whatever level
 // and cell they belong to, an entry is rejected on one 32-byte load, and only
-// survivors load their record; the same view took 433 M instructions and 620 us
-// with a chunk loop per cell and level, 327 M and 520 us so. 5 blocks of 4 warps
-// per SM: at 6 (80 registers) the spills cost 5 % more than the warps bring.
-// A tile of a split forward that turns out longer than its estimate (eight
+// survivors load their record. 5 blocks of 4 warps per SM: at 6 (80 registers)
+// the spills cost 5 % more than the warps bring.
+//
+// The order of the sums is part of the result (a training step's last bits
+// decide which pairs the next one includes), so what is free is only who takes
+// a sum, not how it is made up: a tile's walked sums take the entries level by
+// level, cell by cell, in list order; its pooled sums take each level's items
+// 32 at a time, a lane each; and a tile of P parts (Grid: split_items) adds P
+// such sums, each over every P-th chunk of 32 of every list. One warp takes all
+// the parts, one after the other, on one look-up of the lists; only a tile that
+// would keep a warp too long is given to several, some parts each
+// (tile_parts_kernel). Two cases choose their own order: calls of few tiles,
+// whose lists a team of warps shares, and the disk kernel, which nothing
+// differentiates: there a tile that turns out longer than its estimate (eight
 // sampled points may miss the one in a dense cell) is deferred, before its lists
 // are walked, to a second launch, which splits it kHeavyParts ways: one such tile
 // begun late kept its warp for 290 us after all the others of a 215 us density
-// estimate had ended, and 690 us of a 1,860 us forward over eight views. Longer
-// means an eighth of what every warp has to do; nothing is deferred below
-// kHeavyChunks chunks (16, 48, 144: the estimate 799, 812, 883 us a pass, but a
-// training step over 1M Gaussians 1.79 ms at 16 and 1.73 at 48). If they were too many for the list of units, the second
+// estimate had ended. Longer means an eighth of what every warp has to do;
+// nothing is deferred below kHeavyChunks chunks (16, 48, 144: the estimate 799,
+// 812, 883 us a pass). If they were too many for the list of units, the second
 // launch takes them whole (all of them, so that the sums do not depend on which
 // warp came first).
 constexpr uint32_t kHeavyParts = 8, kHeavyChunks = 48;
@@ -401,7 +417,7 @@ __device__ __forceinline__ uint32_t heavy_chunks(const DeviceHeader* h) {
   return max(kHeavyChunks, (uint32_t)min(share / 8, 1ull << 20));
 }
 __device__ __forceinline__ bool heavy_fits(const DeviceHeader* h) {
-  return h->n_xunits + kHeavyParts * h->n_heavy <= (unsigned long long)GPF_MAX_SPLIT_UNITS;
+  return h->n_xslots + kHeavyParts * h->n_heavy <= (unsigned long long)GPF_MAX_SPLIT_UNITS;
 }
 
 // COUNT: count the evaluated and included pairs instead of summing radiance.
@@ -412,6 +428,8 @@ __global__ void __launch_bounds__(TEAM > 4 ? TEAM * kWarp : kFwdThreads,
                                   TEAM > 4 ? 1 : C <= 4 ? 5 : 4)
 fwd_kernel(const __grid_constant__ FwdArgs a) {
   constexpr int RS = rec_stride(C);
+  constexpr bool kOrdered = TEAM == 1 && KERN != kKernDisk;   // sums in the order stated above
+  constexpr bool kDefer = KERN == kKernDisk && !BRUTE && !COUNT;
   extern __shared__ __align__(16) float s_mem[];
   __shared__ unsigned long long s_unit;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -422,15 +440,14 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
   for (int i = lane; i < stage_words(C); i += kWarp) ws.stage[i] = 0.0f;
   const int64_t n_act = a.header->n_active;
   const int64_t n_tiles = (a.m + kWarp - 1) / kWarp;
-  // split tiles (heavy ones, when the index asks for it) come first as
-  // n_x units, one per part; then every tile as one unit (a split tile's is
-  // skipped)
+  // the units of the tiles that several warps take come first, then every tile
+  // as one unit (those tiles' are skipped)
   const int64_t n_x = a.tparts ? (int64_t)a.header->n_xunits : 0;
-  const bool late = !COUNT && a.late;
+  const bool late = kDefer && a.late;
   const bool late_split = late && heavy_fits(a.header);
   const int64_t n_units =
       late ? (int64_t)a.header->n_heavy * (late_split ? (int64_t)kHeavyParts : 1) : n_x + n_tiles;
-  const uint32_t limit = !COUNT && !late && a.tparts ? heavy_chunks(a.header) : 0xffffffffu;
+  const uint32_t limit = kDefer && !late && a.tparts ? heavy_chunks(a.header) : 0xffffffffu;
   unsigned long long* const next_unit = late ? &a.header->next_heavy : &a.header->next_tile;
   const uint32_t lmask = a.header->level_mask;
   uint32_t n_eval = 0, n_inc = 0;
@@ -450,32 +467,36 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
     unit = (int64_t)__shfl_sync(kFullMask, unit_u, 0);
   }
   if (unit >= n_units) break;
+  // this unit's tile, its parts [p0, p1) of `parts`, and, where other units have
+  // the tile's other parts, the slot of part 0
   int64_t tile;
-  uint32_t part = 0, parts = 1;
+  uint32_t p0 = 0, p1 = 1, parts = 1, slot = 0;
+  bool split = false;
   if (late) {
-    if (late_split) {
-      unit += n_x;
-      const uint4 xu = a.xunit[unit];
-      tile = xu.x;
-      part = xu.y;
+    split = late_split;
+    tile = a.xheavy[split ? unit / kHeavyParts : unit];
+    if (split) {
       parts = kHeavyParts;
-    } else {
-      tile = a.xheavy[unit];
+      p0 = (uint32_t)(unit % kHeavyParts);
+      p1 = p0 + 1;
+      slot = a.header->n_xslots + (uint32_t)unit - p0;
     }
   } else if (unit < n_x) {
     const uint4 xu = a.xunit[unit];
-    if (!xu.w) continue;                      // a slot left over at the capacity edge
+    const uint32_t i = xu.y & 0xffu, of = (xu.y >> 8) & 0xffu;
     tile = xu.x;
-    part = xu.y;
-    parts = xu.z;
+    slot = xu.z;
+    split = true;
+    parts = kOrdered ? xu.y >> 16 : of;
+    p0 = kOrdered ? i * parts / of : i;
+    p1 = kOrdered ? (i + 1) * parts / of : i + 1;
   } else {
     tile = unit - n_x;
-    if (n_x && a.tparts[tile] > 1) continue;  // done by its parts
-  }
-  const bool split = parts > 1;
-  if (TEAM > 1) {
-    part = part * TEAM + wib;
-    parts *= TEAM;
+    if (a.tparts) {
+      const uint32_t tp = a.tparts[tile];
+      if (tp & kTileUnits) continue;          // taken by its units
+      if (kOrdered) p1 = parts = tp;
+    }
   }
   const int64_t base = tile * kWarp;
   const int64_t k = base + lane;
@@ -498,37 +519,19 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
     pz = p.z;
     q = __float_as_uint(p.w);
   }
-  f32x2 L2[C], Z2 = 0;
-#pragma unroll
-  for (int c = 0; c < C; ++c) L2[c] = 0;
-#pragma unroll
-  for (int c = 0; c <= C; ++c) ws.acc[c][lane] = 0.0f;
-  __syncwarp();
 
-  if (BRUTE) {
-    float L[C], Z = 0.0f;
-#pragma unroll
-    for (int c = 0; c < C; ++c) L[c] = 0.0f;
-    float* my_rec = ws.stage;
-    for (int64_t g0 = (int64_t)part * kWarp; g0 < a.n; g0 += (int64_t)parts * kWarp) {
-      const int64_t g = g0 + lane;
-      const int cnt = (int)min((int64_t)kWarp, a.n - g0);
-      if (g < a.n) {
-        const float4* src = reinterpret_cast<const float4*>(a.rec + g * RS);
-        float4* dst = reinterpret_cast<float4*>(my_rec + lane * RS);
-#pragma unroll
-        for (int v = 0; v < RS / 4; ++v) dst[v] = src[v];
-      }
-      __syncwarp();
-      if (active)
-        for (int s = 0; s < cnt; ++s)
-          eval_pair<C, KERN, COUNT>(my_rec + s * RS, px, py, pz, a, L, Z, n_eval, n_inc);
-      __syncwarp();
-    }
-#pragma unroll
-    for (int c = 0; c < C; ++c) L2[c] = pack2(L[c], 0.0f);
-    Z2 = pack2(Z, 0.0f);
-  } else {
+  // ---- walked levels: their distinct cells' lists as segments, end to end;
+  // pooled levels: each lane's lists of a level end to end, a level after the
+  // other (range[p] of the p-th pooled level: first entry - items before, items
+  // up to and with this lane's). The pooled levels are the finest ones: a
+  // coarser level has no more distinct cells.
+  int n_seg = 0, n_pool = 0;
+  uint32_t total = 0;                     // entries of the segments
+  uint32_t pool_chunks = 0;               // chunks of the pooled levels
+  unsigned long long pool_levels = 0;     // 4 bits per pooled level
+  // parts take whole chunks of each list, so their segments begin with a chunk
+  const bool pad = kOrdered && parts > 1;
+  if (!BRUTE) {
     const uint32_t c0x = coord0(px, G.ox, G.inv_cell0, G.max0x);
     const uint32_t c0y = coord0(py, G.oy, G.inv_cell0, G.max0y);
     const uint32_t c0z = coord0(pz, G.oz, G.inv_cell0, G.max0z);
@@ -564,14 +567,6 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
                               0.5f * (bz1 - bz0));
     }
     __syncwarp();
-
-    // ---- walked levels: their distinct cells' lists as segments, end to end;
-    // pooled levels: each lane's lists end to end (range[p] of the p-th pooled
-    // level becomes (first entry - items before, items up to and with it))
-    int n_seg = 0, n_pool = 0;
-    uint32_t total = 0;                     // entries of the segments
-    uint32_t len = 0;                       // this lane's pooled items
-    unsigned long long pool_levels = 0;     // 4 bits per pooled level
     for (int lev = 0; lev < G.levels; ++lev) {
       if (!((lmask >> lev) & 1u)) continue;
       const uint32_t lx = c0x >> lev, ly = c0y >> lev, lz = c0z >> lev;
@@ -581,53 +576,82 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
       const uint32_t uniq = __ballot_sync(kFullMask, leader);
       const int nu = __popc(uniq);
       const uint2 rg = ws.range[lev * kWarp + lane];    // (0, 0) for inactive lanes
-      if (nu <= G.coop) {
-        // (a cell without a list holds no Gaussian that another cell repeats)
-        const bool has = leader && rg.y > rg.x;
-        const uint32_t hm = __ballot_sync(kFullMask, has);
-        uint32_t incl = has ? rg.y - rg.x : 0u;
+      const bool walked = nu <= G.coop;
+      // (a cell without a list holds no Gaussian that another cell repeats)
+      const uint32_t len = walked && !leader ? 0u : rg.y - rg.x;
+      const uint32_t room = walked && pad ? (len + kWarp - 1) / kWarp * kWarp : len;
+      uint32_t incl = room;
 #pragma unroll
-        for (int o = 1; o < kWarp; o <<= 1) {
-          const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
-          if (lane >= o) incl += t;
-        }
-        if (has) {
-          const int slot = n_seg + __popc(hm & lanemask_lt());
-          const uint32_t before = total + incl - (rg.y - rg.x);
-          ws.cell[slot] = packed;
-          ws.seg[slot] = make_uint4(before, rg.x - before, cell_hash(G, lev, lx, ly, lz).tag,
-                                    (uint32_t)lev | ((uint32_t)n_seg << 8));
+      for (int o = 1; o < kWarp; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const uint32_t all = __shfl_sync(kFullMask, incl, kWarp - 1);
+      if (walked) {
+        const uint32_t hm = __ballot_sync(kFullMask, len > 0u);
+        if (len > 0u) {
+          const int s = n_seg + __popc(hm & lanemask_lt());
+          const uint32_t before = total + incl - room;
+          ws.cell[s] = packed;
+          ws.seg[s] = make_uint4(before, rg.x - before, cell_hash(G, lev, lx, ly, lz).tag,
+                                 (uint32_t)lev | ((uint32_t)n_seg << 8) |
+                                     (((len - 1u) & 31u) << 16));
         }
         n_seg += __popc(hm);
-        total += __shfl_sync(kFullMask, incl, kWarp - 1);
+        total += all;
       } else {
         // (slot n_pool <= lev: the ranges of this and later levels are read first)
-        ws.range[n_pool * kWarp + lane] = make_uint2(rg.x - len, len + (rg.y - rg.x));
-        len += rg.y - rg.x;
+        ws.range[n_pool * kWarp + lane] = make_uint2(rg.x - (incl - len), incl);
+        pool_chunks += (all + kWarp - 1) / kWarp;
         pool_levels |= (unsigned long long)lev << (4 * n_pool);
         ++n_pool;
       }
     }
+    if (lane == 0) ws.seg[n_seg].x = total;
     __syncwarp();
+  }
+  const uint32_t n_chunks = (total + kWarp - 1) / kWarp;
+  if (kDefer && !split && n_chunks + pool_chunks > limit) {
+    if ((TEAM == 1 || wib == 0) && lane == 0)
+      a.xheavy[atomicAdd(&a.header->n_heavy, 1ull)] = (uint32_t)tile;
+    continue;
+  }
 
-    // a split tile's part, and a team's warp, take every parts-th chunk of 32
-    // entries, then of 32 items
-    const uint32_t n_chunks = (total + kWarp - 1) / kWarp;
-    if (!split && n_chunks + __reduce_add_sync(kFullMask, len) / kWarp > limit) {
-      if (TEAM == 1 || wib == 0) {
-        uint32_t slot = 0;
-        if (lane == 0) {
-          slot = (uint32_t)atomicAdd(&a.header->n_heavy, 1ull);
-          a.xheavy[slot] = (uint32_t)tile;
-        }
-        const int64_t first =
-            n_x + (int64_t)kHeavyParts * __shfl_sync(kFullMask, slot, 0);
-        if (first + kHeavyParts <= GPF_MAX_SPLIT_UNITS && lane < kHeavyParts)
-          a.xunit[first + lane] = make_uint4((uint32_t)tile, lane, kHeavyParts, 1u);
+  float L[C], Z = 0.0f;                   // this hit point's sums over the unit's parts
+#pragma unroll
+  for (int c = 0; c < C; ++c) L[c] = 0.0f;
+  for (uint32_t pt = p0; pt < p1; ++pt) {
+  // chunk c of the unit's lists, the pooled levels' first, is taken for
+  // c mod of == part
+  const uint32_t part = TEAM > 1 ? pt * TEAM + wib : pt;
+  const uint32_t of = TEAM > 1 ? parts * TEAM : parts;
+  float W[C], V = 0.0f;                   // the walked sums of this part
+#pragma unroll
+  for (int c = 0; c < C; ++c) W[c] = 0.0f;
+#pragma unroll
+  for (int c = 0; c <= C; ++c) ws.acc[c][lane] = 0.0f;
+  __syncwarp();
+
+  if (BRUTE) {
+    float* my_rec = ws.stage;
+    for (int64_t g0 = (int64_t)part * kWarp; g0 < a.n; g0 += (int64_t)of * kWarp) {
+      const int64_t g = g0 + lane;
+      const int cnt = (int)min((int64_t)kWarp, a.n - g0);
+      if (g < a.n) {
+        const float4* src = reinterpret_cast<const float4*>(a.rec + g * RS);
+        float4* dst = reinterpret_cast<float4*>(my_rec + lane * RS);
+#pragma unroll
+        for (int v = 0; v < RS / 4; ++v) dst[v] = src[v];
       }
-      continue;
+      __syncwarp();
+      if (active)
+        for (int s = 0; s < cnt; ++s)
+          eval_pair<C, KERN, COUNT>(my_rec + s * RS, px, py, pz, a, W, V, n_eval, n_inc);
+      __syncwarp();
     }
-    if (n_chunks > 0) {
+  } else {
+    uint32_t chunk = (part + of - pool_chunks % of) % of;
+    if (chunk < n_chunks) {
       const float cut_keep = a.cut * 1.0001f;
       int top = 1;                          // the segment search's first step
       while (2 * top < n_seg) top *= 2;
@@ -637,12 +661,14 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
       const uint32_t seg_at =
           few && lane < n_seg ? ws.seg[lane].x : 0xffffffffu;
       const uint32_t le = lanemask_lt() | (1u << lane);
-      // entry e of the stream: its segment (the first whose inclusive count
-      // exceeds e) and entry word, with the previous word of its list
+      // entry e of the stream: its segment (the last that begins at or before e)
+      // and entry word (all ones, which no cell has: none), with the previous
+      // word of its list
       auto fetch = [&](uint32_t chunk, int& seg, uint32_t& v, uint32_t& vprev, bool& first) {
         const uint32_t e = chunk * kWarp + lane;
         seg = 0;
-        v = vprev = 0u;
+        v = 0xffffffffu;
+        vprev = 0u;
         first = true;
         if (few) {
           const uint32_t c0 = chunk * kWarp;
@@ -654,6 +680,10 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
           if (!few)
             for (int st = top; st > 0; st >>= 1)
               if (seg + st <= n_seg - 1 && ws.seg[seg + st].x <= e) seg += st;
+          // (a padded list's last chunk)
+          if (pad && ws.seg[seg + 1].x == (chunk + 1) * kWarp &&
+              (uint32_t)lane > (ws.seg[seg].w >> 16))
+            return;
           const uint2 sg = *reinterpret_cast<const uint2*>(ws.seg + seg);
           const uint32_t* p = a.gval + (sg.y + e);         // modulo 2^32
           v = __ldg(p);
@@ -661,7 +691,6 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
           if (!first && lane == 0) vprev = __ldg(p - 1);   // (else the lane to the left has it)
         }
       };
-      uint32_t chunk = part;
       int qn = 0;                            // queued ids
       for (;;) {
         // vet entries until the queue may overflow; the entry words of the
@@ -673,16 +702,15 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
         while (chunk < n_chunks && qn <= kQueue - kWarp) {
           const int seg = seg_n;
           const uint32_t v = v_n;
-          const bool live = chunk * kWarp + lane < total;
           const uint32_t left = __shfl_up_sync(kFullMask, v, 1);
           // a Gaussian listed twice in a bucket sits on consecutive entries
           const bool again = !first_n && v == (lane == 0 ? vp_n : left);
           const uint2 sl = reinterpret_cast<const uint2*>(ws.seg + seg)[1];   // tag, level
-          bool keep = live && (v & ~G.id_mask) == sl.x && !again;
+          bool keep = (v & ~G.id_mask) == sl.x && !again;
           const uint32_t g = v & G.id_mask;
           VetRec r;
           if (keep) r = load_vet(a.vet + g);
-          chunk += parts;
+          chunk += of;
           fetch(chunk, seg_n, v_n, vp_n, first_n);
           if (keep) {
             // sphere test: distance from mu to the tile box vs k * max s
@@ -694,7 +722,7 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
             // have been taken from an earlier cell of this tile
             keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= r.radius * r.radius &&
                    rec_level(r.radius) == (sl.y & 0xffu) && cell_in(r, ws.cell[seg]);
-            for (int j = (int)(sl.y >> 8); j < seg && keep; j += 2)      // two loads at a time
+            for (int j = (int)((sl.y >> 8) & 0xffu); j < seg && keep; j += 2)   // two loads at a time
               keep = !(cell_in(r, ws.cell[j]) || (j + 1 < seg && cell_in(r, ws.cell[j + 1])));
           }
           const uint32_t kb = __ballot_sync(kFullMask, keep);
@@ -730,7 +758,7 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
           if (COUNT) {
             if (active) count_staged<C>(ws.stage, nk, px, py, pz, a, n_eval, n_inc);
           } else {
-            eval_staged<C, KERN>(ws.stage, nk, px, py, pz, a, L2, Z2);
+            eval_staged<C, KERN>(ws.stage, nk, px, py, pz, a, W, V);
           }
           __syncwarp();
         }
@@ -746,81 +774,87 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
 
     // ---- pooled levels: 32 (hit point, entry) items at a time, one per lane.
     // A lane sums what it evaluates for one owner at a time and hands the
-    // sum over (pooled_flush) when the owner of its item slot changes, so
-    // no lane waits for the longest list and every sum has a fixed order.
-    // The cell-box test is not needed here: an entry that reached this
+    // sum over (pooled_flush) when the owner of its item slot, or the level,
+    // changes, so no lane waits for the longest list and every sum has a fixed
+    // order. The cell-box test is not needed here: an entry that reached this
     // bucket from another cell on the same level has a box that misses
     // this hit point, so Q > k^2 rejects it; the level test and the
     // duplicate test keep any Gaussian from being counted twice.
-    if (n_pool > 0) {
-      uint32_t incl = len;  // inclusive prefix sum of the lanes' items
-#pragma unroll
-      for (int o = 1; o < kWarp; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const uint32_t items = __shfl_sync(kFullMask, incl, kWarp - 1);
-      // the lanes that have items, in order: (lane, first item); the owners of a
-      // chunk follow from the first items inside it
-      const uint32_t has = __ballot_sync(kFullMask, len > 0u);
-      const uint32_t own_at = len > 0u ? incl - len : 0xffffffffu;
-      uint2* owners = reinterpret_cast<uint2*>(ws.queue);
-      if (len > 0u)
-        owners[__popc(has & lanemask_lt())] = make_uint2((uint32_t)lane, incl - len);
-      __syncwarp();
+    if (part < pool_chunks) {
+      // the level that is fetched: its chunks [lbeg, lend) of the pooled ones, its
+      // items, where this lane's begin, and the lanes that have items, in order:
+      // (lane, first item, tag, first entry - first item)
+      int pl = -1, lev_f = 0;
+      uint32_t lbeg = 0, lend = 0, items = 0, own_at = 0xffffffffu;
+      uint4* owners = reinterpret_cast<uint4*>(ws.queue);
+      static_assert(sizeof(uint4) * kWarp <= sizeof(uint32_t) * kQueue, "room for every lane");
       const uint32_t le = lanemask_lt() | (1u << lane);
-      // item i: its owner (the first lane whose inclusive end exceeds i; kWarp:
-      // none), level, entry word and the previous word of its list
-      auto fetch = [&](uint32_t i, int& own, int& lev, uint32_t& v, uint32_t& vprev, bool& first) {
-        const uint32_t i0 = i - lane;
+      // item of this lane in chunk c: its owner (kWarp: none), the owner's tag,
+      // level, entry word and the previous word of its list
+      auto fetch = [&](uint32_t c, int& own, int& lev, uint32_t& tag, uint32_t& v,
+                       uint32_t& vprev, bool& first) {
+        own = kWarp;
+        lev = lev_f;
+        tag = v = vprev = 0u;
+        first = true;
+        if (c >= pool_chunks) return;
+        if (c >= lend) {
+          do {
+            ++pl;
+            items = ws.range[pl * kWarp + kWarp - 1].y;
+            lbeg = lend;
+            lend += (items + kWarp - 1) / kWarp;
+          } while (c >= lend);
+          lev = lev_f = (int)((pool_levels >> (4 * pl)) & 15u);
+          const uint2 rg = ws.range[pl * kWarp + lane];
+          uint32_t excl = __shfl_up_sync(kFullMask, rg.y, 1);
+          if (lane == 0) excl = 0;
+          const bool any = rg.y > excl;
+          own_at = any ? excl : 0xffffffffu;
+          const uint32_t has = __ballot_sync(kFullMask, any);
+          if (any)
+            owners[__popc(has & lanemask_lt())] =
+                make_uint4((uint32_t)lane, excl,
+                           cell_hash(G, lev_f, coord0(px, G.ox, G.inv_cell0, G.max0x) >> lev_f,
+                                     coord0(py, G.oy, G.inv_cell0, G.max0y) >> lev_f,
+                                     coord0(pz, G.oz, G.inv_cell0, G.max0z) >> lev_f).tag,
+                           rg.x);
+          __syncwarp();
+        }
+        const uint32_t i0 = (c - lbeg) * kWarp, i = i0 + lane;
         const uint32_t inside = __reduce_or_sync(
             kFullMask, own_at > i0 && own_at - i0 < kWarp ? 1u << (own_at - i0) : 0u);
         const uint32_t begun = __ballot_sync(kFullMask, own_at <= i0);
-        own = kWarp;
-        lev = 0;
-        v = vprev = 0u;
-        first = true;
         if (i < items) {
-          const uint2 ow = owners[__popc(begun) - 1 + __popc(inside & le)];
-          const uint32_t o = ow.x, kk = i - ow.y;
-          own = (int)o;
-          uint32_t before = 0;
-          int p = 0;
-          uint2 rg = ws.range[o];
-          while (rg.y <= kk) {
-            before = rg.y;
-            ++p;
-            rg = ws.range[p * kWarp + o];
-          }
-          lev = (int)((pool_levels >> (4 * p)) & 15u);
-          const uint32_t at = rg.x + kk;               // modulo 2^32
+          const uint4 ow = owners[__popc(begun) - 1 + __popc(inside & le)];
+          own = (int)ow.x;
+          tag = ow.z;
+          const uint32_t at = ow.w + i;                // modulo 2^32
           v = __ldg(a.gval + at);
-          first = kk == before;
+          first = i == ow.y;
           if (!first && lane == 0) vprev = __ldg(a.gval + (at - 1u));
         }
+        __syncwarp();                                  // (before the next level's owners)
       };
-      int cur = -1;  // owner of this lane's item slot in the previous chunk
+      int cur = -1, cur_lev = -1;  // owner of this lane's item slot in the previous chunk
       float pc[C + 1];
 #pragma unroll
       for (int c = 0; c <= C; ++c) pc[c] = 0.0f;
       float qx = 0.0f, qy = 0.0f, qz = 0.0f;
-      const uint32_t step = parts * kWarp;
-      uint32_t b = (part + parts - n_chunks % parts) % parts * kWarp;
       int own_n, lev_n;
-      uint32_t v_n, vp_n;
+      uint32_t tag_n, v_n, vp_n;
       bool first_n;
-      fetch(b + lane, own_n, lev_n, v_n, vp_n, first_n);
-      for (; b < items; b += step) {
+      fetch(part, own_n, lev_n, tag_n, v_n, vp_n, first_n);
+      for (uint32_t b = part; b < pool_chunks; b += of) {
         const int own = own_n, lev = lev_n;
         const uint32_t v = v_n;
         const uint32_t left = __shfl_up_sync(kFullMask, v, 1);
-        // (by id: entries of two cells in one bucket may differ in their tags)
-        const bool again = !first_n && ((v ^ (lane == 0 ? vp_n : left)) & G.id_mask) == 0u;
-        const bool take = own < kWarp && !again;
+        const bool again = !first_n && v == (lane == 0 ? vp_n : left);
+        const bool take = own < kWarp && (v & ~G.id_mask) == tag_n && !again;
         float rr[RS];
         if (take) load_rec_head<RS>(a.rec, v & G.id_mask, rr);
-        fetch(b + step + lane, own_n, lev_n, v_n, vp_n, first_n);
-        const bool chg = own != cur;
+        fetch(b + of, own_n, lev_n, tag_n, v_n, vp_n, first_n);
+        const bool chg = own != cur || lev != cur_lev;
         if (__any_sync(kFullMask, chg)) {
           pooled_flush<C>(ws.acc, lane, cur, chg && cur >= 0 && cur < kWarp, pc);
           const int src = own & (kWarp - 1);
@@ -828,6 +862,7 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
           qy = __shfl_sync(kFullMask, py, src);
           qz = __shfl_sync(kFullMask, pz, src);
           cur = own;
+          cur_lev = lev;
         }
         // the rest of the record only where its bounding sphere holds the point
         bool near = take && rec_level(rr[3]) == (uint32_t)lev;
@@ -851,48 +886,49 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
   }
 
   if (!COUNT) {
-    // the staged sums and the pooled sums of this lane's hit point
+    // the walked and the pooled sums of this lane's hit point
     __syncwarp();
-    float L[C], Z;
 #pragma unroll
-    for (int c = 0; c <= C; ++c) {
-      float lo, hi;
-      unpack2(c < C ? L2[c < C ? c : 0] : Z2, lo, hi);
-      const float s = (lo + hi) + ws.acc[c][lane];
-      if (c < C) L[c < C ? c : 0] = s;
-      else Z = s;
-    }
+    for (int c = 0; c < C; ++c) W[c] += ws.acc[c][lane];
+    V += ws.acc[C][lane];
     if (TEAM > 1) {
       // the team's sums, added in warp order by warp 0
 #pragma unroll
-      for (int c = 0; c < C; ++c) ws.acc[c][lane] = L[c];
-      ws.acc[C][lane] = Z;
+      for (int c = 0; c < C; ++c) ws.acc[c][lane] = W[c];
+      ws.acc[C][lane] = V;
       __syncthreads();
-      if (wib > 0) continue;
+      if (wib > 0) continue;      // (a team's unit has one part)
       for (int w = 1; w < TEAM; ++w) {
         const WarpShared o = warp_shared<C>(s_mem, w, G.levels, G.coop);
 #pragma unroll
-        for (int c = 0; c < C; ++c) L[c] += o.acc[c][lane];
-        Z += o.acc[C][lane];
+        for (int c = 0; c < C; ++c) W[c] += o.acc[c][lane];
+        V += o.acc[C][lane];
       }
     }
     if (split) {
       // this part's sums; fwd_split_combine_kernel adds the parts in order
-      float* xs = a.xsum + (size_t)unit * (C + 1) * kWarp;
+      float* xs = a.xsum + (size_t)(slot + pt) * (C + 1) * kWarp;
 #pragma unroll
-      for (int c = 0; c < C; ++c) xs[c * kWarp + lane] = L[c];
-      xs[C * kWarp + lane] = Z;
-    } else if (active) {
-      float scale = 1.0f;
-      if (a.mode == GPF_NORMALIZED) scale = 1.0f / fmaxf(Z, a.eps);
-      else if (a.mode == GPF_DISK_KDE) scale = a.kde_scale;
+      for (int c = 0; c < C; ++c) xs[c * kWarp + lane] = W[c];
+      xs[C * kWarp + lane] = V;
+    } else {
 #pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const float rho = a.albedo ? a.albedo[(int64_t)c * a.m + q] : 1.0f;
-        a.out[(int64_t)c * a.m + q] = rho * (L[c] * scale);
-      }
-      if (a.z) a.z[q] = Z;
+      for (int c = 0; c < C; ++c) L[c] += W[c];
+      Z += V;
     }
+  }
+  }  // parts
+
+  if (!COUNT && !split && active && (TEAM == 1 || wib == 0)) {
+    float scale = 1.0f;
+    if (a.mode == GPF_NORMALIZED) scale = 1.0f / fmaxf(Z, a.eps);
+    else if (a.mode == GPF_DISK_KDE) scale = a.kde_scale;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const float rho = a.albedo ? a.albedo[(int64_t)c * a.m + q] : 1.0f;
+      a.out[(int64_t)c * a.m + q] = rho * (L[c] * scale);
+    }
+    if (a.z) a.z[q] = Z;
   }
   }  // tile loop
 
@@ -909,25 +945,35 @@ fwd_kernel(const __grid_constant__ FwdArgs a) {
   }
 }
 
-// The split tiles' outputs: one warp per split unit of part 0, adding the
-// tile's parts in part order, then the epilogue of fwd_kernel.
+// The split tiles' outputs: one warp per tile that several units took, adding
+// its parts in part order, then the epilogue of fwd_kernel. ordered: the units
+// wrote the tile's own parts (else a part each).
 template <int C>
-__global__ void fwd_split_combine_kernel(FwdArgs a) {
+__global__ void fwd_split_combine_kernel(FwdArgs a, bool ordered, bool deferred) {
   const int lane = threadIdx.x & 31;
   const int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t n_heavy = heavy_fits(a.header) ? (int64_t)a.header->n_heavy : 0;
-  if (index_unusable(a.header) ||
-      u >= (int64_t)a.header->n_xunits + (int64_t)kHeavyParts * n_heavy)
-    return;
-  const uint4 xu = a.xunit[u];
-  if (!xu.w || xu.y != 0u) return;
-  const int64_t k = (int64_t)xu.x * kWarp + lane;
+  if (index_unusable(a.header)) return;
+  const int64_t n_x = a.header->n_xunits;
+  uint32_t tile, slot, parts;
+  if (u < n_x) {
+    const uint4 xu = a.xunit[u];
+    if ((xu.y & 0xffu) != 0u) return;
+    tile = xu.x;
+    slot = xu.z;
+    parts = ordered ? xu.y >> 16 : (xu.y >> 8) & 0xffu;
+  } else {
+    if (!deferred || !heavy_fits(a.header) || u - n_x >= (int64_t)a.header->n_heavy) return;
+    tile = a.xheavy[u - n_x];
+    slot = a.header->n_xslots + kHeavyParts * (uint32_t)(u - n_x);
+    parts = kHeavyParts;
+  }
+  const int64_t k = (int64_t)tile * kWarp + lane;
   float L[C], Z = 0.0f;
 #pragma unroll
   for (int c = 0; c < C; ++c) L[c] = 0.0f;
 #pragma unroll 4
-  for (uint32_t p = 0; p < xu.z; ++p) {
-    const float* xs = a.xsum + (size_t)(u + p) * (C + 1) * kWarp;
+  for (uint32_t p = 0; p < parts; ++p) {
+    const float* xs = a.xsum + (size_t)(slot + p) * (C + 1) * kWarp;
 #pragma unroll
     for (int c = 0; c < C; ++c) L[c] += xs[c * kWarp + lane];
     Z += xs[C * kWarp + lane];
@@ -946,20 +992,25 @@ __global__ void fwd_split_combine_kernel(FwdArgs a) {
   if (a.z) a.z[q] = active ? Z : 0.0f;
 }
 
-// Estimated work of every tile of 32 hit points, from a sample of eight of its
+// Two estimates for every tile of 32 hit points, from a sample of eight of its
 // points (every fourth: neighbouring points of the cell order see similar
-// lists), on every used level: where the sample falls in at most Grid::coop
-// cells, the distinct cells' lists, walked by the whole warp; else the points'
-// own lists, and four times as many for the points not sampled. 32 entries of
-// either kind cost a warp about the same (a least-squares fit over the units of
-// a 1M-Gaussian view: 1.5 us per 32 walked, 1.6 us per 32 pooled entries, and
-// 17 us a unit; weighting the pooled ones an eighth left single units of up to
-// 690 us at the end of a 1.8 ms forward). And the sum over all tiles. Four tiles
-// per warp, eight lanes each.
+// lists), over every used level: where the sample falls in at most Grid::coop
+// cells, from the distinct cells' lists, walked by the whole warp; else from the
+// points' own lists, times four for the points not sampled.
+//  * The parts of its sums (parts, and by group of tiles in xpart): a walked
+//    entry counts 8 and a pooled one 1, and a tile of more than split_items has
+//    one part per split_items. They fix the order of the sums, so this count is
+//    not an estimate to be improved.
+//  * The work of a warp (cost, and the sum over all tiles): 32 entries of either
+//    kind cost it about the same (a least-squares fit over the units of a
+//    1M-Gaussian view: 1.5 us per 32 walked, 1.6 us per 32 pooled entries, and
+//    17 us a unit).
+// Four tiles per warp, eight lanes each.
 __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
                                  const float4* __restrict__ qpos, int64_t m,
                                  const uint2* __restrict__ brange,
-                                 const uint32_t* __restrict__ listed,
+                                 const uint32_t* __restrict__ listed, uint32_t split_items,
+                                 uint32_t* __restrict__ tparts, uint32_t* __restrict__ xpart,
                                  uint32_t* __restrict__ tcost, unsigned long long* total) {
   const int lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -984,7 +1035,7 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
     if (active && lev < grid.levels && ((lmask >> lev) & 1u))
       rg[lev] = bucket_list(listed, brange, bucket_of(grid, lev, c0x >> lev, c0y >> lev, c0z >> lev));
   }
-  uint32_t cost = 0;
+  uint32_t walked = 0, pooled = 0;       // entries, of this sampled point
 #pragma unroll
   for (int lev = 0; lev < kMaxLevels; ++lev) {
     if (lev >= grid.levels || !((lmask >> lev) & 1u)) continue;
@@ -997,14 +1048,27 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
     const int nu = __popc(__ballot_sync(kFullMask, leader) & group);
     const uint32_t len = rg[lev].y - rg[lev].x;
     // (eight samples see at most 8 cells: all 8 distinct reads as more than 8)
-    cost += kCostPerEntry * (nu <= min(grid.coop, 7) ? (leader ? len : 0u) : 4u * len);
+    if (nu > min(grid.coop, 7)) pooled += len;
+    else if (leader) walked += len;
   }
   // the eight lanes of a tile are consecutive: sum them
-  cost += __shfl_xor_sync(kFullMask, cost, 1);
-  cost += __shfl_xor_sync(kFullMask, cost, 2);
-  cost += __shfl_xor_sync(kFullMask, cost, 4);
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    walked += __shfl_xor_sync(kFullMask, walked, o);
+    pooled += __shfl_xor_sync(kFullMask, pooled, o);
+  }
+  const uint32_t items = 8u * walked + 4u * pooled;
+  uint32_t cost = kCostPerEntry * (walked + 4u * pooled);
   if (tile < n_tiles && tile * kWarp < n_act) cost += kCostPerTile;
-  if ((lane & 7) == 0 && tile < n_tiles) tcost[tile] = cost;
+  if ((lane & 7) == 0 && tile < n_tiles) {
+    const uint32_t parts = items <= split_items
+                               ? 1u
+                               : min((items + split_items - 1) / split_items,
+                                     (uint32_t)GPF_MAX_TILE_PARTS);
+    tparts[tile] = parts;
+    tcost[tile] = cost;
+    if (parts > 1) atomicAdd(&xpart[tile / kTileGroup], parts);
+  }
   __shared__ uint32_t s_sum;
   if (threadIdx.x == 0) s_sum = 0;
   __syncthreads();
@@ -1014,53 +1078,77 @@ __global__ void tile_cost_kernel(Grid grid, const DeviceHeader* header,
   if (threadIdx.x == 0 && s_sum) atomicAdd(total, (unsigned long long)s_sum);
 }
 
-// Parts of every tile from its cost, and the split units. A tile is split when
-// its cost exceeds both split_items and 1 / kSplitShare of all tiles' (a
-// quarter of what a resident warp has to do anyway: splitting the ordinary
-// tiles of a large batch only repeats their lookups; 22 K tiles of a 1M field
-// were 35 K units). The second bound also keeps the units below
-// GPF_MAX_SPLIT_UNITS: a split tile has at most 2 cost / bound parts. Which
-// slots a tile's units get depends on the order of the blocks; its sums do not.
-constexpr uint32_t kSplitShare = 152 * 24 * 4;
-static_assert(2 * kSplitShare <= GPF_MAX_SPLIT_UNITS, "room for every split unit");
+// The parts' slots and the units. Each part of a split tile has a slot, after
+// those of the split tiles before it (a block adds up the groups before its
+// own: there is one word per 256 tiles, and most of them are zero); a tile
+// whose slots would not all fit under GPF_MAX_SPLIT_UNITS has one part. A tile
+// is given to several units, some of its parts each, when its work exceeds 1 /
+// kSplitShare of all tiles' (a quarter of what a resident warp has to do
+// anyway): a unit of its own for every part repeats the tile's look-ups, 17 us
+// each (22 K tiles of a 1M field were 33 K units). Which place in the list a
+// tile's units get depends on the order of the blocks; its sums do not.
+constexpr uint32_t kSplitShare = 152 * 20 * 4;
 __global__ void __launch_bounds__(kTileGroup)
-tile_parts_kernel(int64_t n_tiles, int split_items, uint32_t* __restrict__ tparts,
+tile_parts_kernel(int64_t n_tiles, uint32_t split_items, uint32_t* __restrict__ tparts,
+                  const uint32_t* __restrict__ xpart, const uint32_t* __restrict__ tcost,
                   const unsigned long long* total, uint4* __restrict__ xunit,
-                  uint32_t* n_units) {
-  __shared__ uint32_t s_warp[kTileGroup / kWarp], s_first;
+                  uint32_t* n_units, uint32_t* n_slots) {
+  __shared__ uint32_t s_before[kTileGroup / kWarp], s_parts[kTileGroup / kWarp],
+      s_units[kTileGroup / kWarp], s_first;
+  const bool last = blockIdx.x == gridDim.x - 1;
+  if (xpart[blockIdx.x] == 0u && !last) return;      // one part each, as written
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t t = (int64_t)blockIdx.x * kTileGroup + threadIdx.x;
-  const unsigned long long bound =
-      max((unsigned long long)split_items, *total / kSplitShare + 1ull);
-  uint32_t parts = 1;
-  if (t < n_tiles) {
-    const unsigned long long cost = min(tparts[t], 1u << 26);     // as summed
-    if (cost > bound)
-      parts = (uint32_t)min((cost + bound - 1) / bound, (unsigned long long)GPF_MAX_TILE_PARTS);
-    tparts[t] = parts;
-  }
-  uint32_t incl = parts > 1 ? parts : 0u;
+  uint32_t before = 0;
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kTileGroup) before += xpart[i];
+  before = __reduce_add_sync(kFullMask, before);
+  uint32_t parts = t < n_tiles ? tparts[t] : 1u;
+  auto scan = [&](uint32_t v) {                      // inclusive, over the warp
 #pragma unroll
-  for (int o = 1; o < kWarp; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(kFullMask, incl, o);
-    if (lane >= o) incl += v;
+    for (int o = 1; o < kWarp; o <<= 1) {
+      const uint32_t u = __shfl_up_sync(kFullMask, v, o);
+      if (lane >= o) v += u;
+    }
+    return v;
+  };
+  const uint32_t mine = parts > 1 ? parts : 0u, incl = scan(mine);
+  if (lane == 0) s_before[warp] = before;
+  if (lane == kWarp - 1) s_parts[warp] = incl;
+  __syncthreads();
+  uint32_t slot = incl - mine, slots = 0;
+  for (int w = 0; w < kTileGroup / kWarp; ++w) {
+    slot += s_before[w] + (w < warp ? s_parts[w] : 0u);
+    slots += s_before[w] + s_parts[w];
   }
-  if (lane == kWarp - 1) s_warp[warp] = incl;
+  if (last && threadIdx.x == 0) *n_slots = min(slots, (uint32_t)GPF_MAX_SPLIT_UNITS);
+  uint32_t units = 1;
+  if (parts > 1) {
+    if ((uint64_t)slot + parts > (uint64_t)GPF_MAX_SPLIT_UNITS) {
+      parts = 1;
+    } else {
+      const unsigned long long share =
+          max((unsigned long long)split_items, *total / kSplitShare + 1ull);
+      units = (uint32_t)min((tcost[t] + share - 1) / share, (unsigned long long)parts);
+    }
+    tparts[t] = parts | (units > 1 ? kTileUnits : 0u);
+  }
+  const uint32_t my_units = units > 1 ? units : 0u, uincl = scan(my_units);
+  if (lane == kWarp - 1) s_units[warp] = uincl;
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t sum = 0;
-    for (int w = 0; w < kTileGroup / kWarp; ++w) sum += s_warp[w];
+    for (int w = 0; w < kTileGroup / kWarp; ++w) sum += s_units[w];
     s_first = sum ? atomicAdd(n_units, sum) : 0u;
   }
   __syncthreads();
-  if (parts <= 1) return;
-  uint32_t o = s_first + incl - parts;
-  for (int w = 0; w < warp; ++w) o += s_warp[w];
-  for (uint32_t p = 0; p < parts && o + p < (uint32_t)GPF_MAX_SPLIT_UNITS; ++p)
-    xunit[o + p] = make_uint4((uint32_t)t, p, parts, 1u);
+  if (units <= 1) return;
+  uint32_t o = s_first + uincl - units;              // no more units than slots: they fit
+  for (int w = 0; w < warp; ++w) o += s_units[w];
+  for (uint32_t i = 0; i < units; ++i)
+    xunit[o + i] = make_uint4((uint32_t)t, i | (units << 8) | (parts << 16), slot, 0u);
 }
 
-// The split units: a split tile's parts follow those of the split tiles before
+// The hybrid forward's split units: a split tile's parts follow those of the split tiles before
 // it (a block adds up the groups before its own: there is one word per 256
 // tiles, and most of them are zero); a tile whose units would not all fit
 // under GPF_MAX_SPLIT_UNITS runs unsplit, and its slots below the limit are
@@ -1114,9 +1202,11 @@ cudaError_t launch_tile_split(const IndexDims& d, const IndexBuffers& b, const g
                               cudaStream_t stream) {
   const int64_t n_tiles = (q.m + kWarp - 1) / kWarp;
   tile_cost_kernel<<<(unsigned)((n_tiles * 8 + 255) / 256), 256, 0, stream>>>(
-      d.grid, b.header, b.qpos, q.m, b.brange, b.listed, b.tparts, &b.header->split_cost);
+      d.grid, b.header, b.qpos, q.m, b.brange, b.listed, (uint32_t)d.split_items, b.tparts,
+      b.xpart, b.tcost, &b.header->split_cost);
   tile_parts_kernel<<<(unsigned)tile_groups(n_tiles), kTileGroup, 0, stream>>>(
-      n_tiles, d.split_items, b.tparts, &b.header->split_cost, b.xunit, &b.header->n_xunits);
+      n_tiles, (uint32_t)d.split_items, b.tparts, b.xpart, b.tcost, &b.header->split_cost,
+      b.xunit, &b.header->n_xunits, &b.header->n_xslots);
   note_launches(2);
   return cudaGetLastError();
 }
@@ -1165,7 +1255,7 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
   a.z = z;
   a.counts = counts;
   a.late = 0;
-  const bool split = d.split_items > 0 && !d.brute;
+  const bool split = d.split_items > 0 && !d.brute && n > 0;
   a.tparts = split ? b.tparts : nullptr;
   a.xunit = split ? b.xunit : nullptr;
   a.xheavy = split ? b.xheavy : nullptr;
@@ -1192,7 +1282,7 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
     const unsigned blocks = (unsigned)persistent_blocks(                                     \
         reinterpret_cast<const void*>(kernel), warps * kWarp, want, smem);                   \
     kernel<<<blocks, warps * kWarp, smem, stream>>>(a);                                      \
-    if (split && !CN) {                                                                      \
+    if (split && !CN && PS == kKernDisk) {                                                   \
       FwdArgs late = a;                                                                      \
       late.late = 1;                                                                         \
       kernel<<<blocks, warps * kWarp, smem, stream>>>(late);                                 \
@@ -1220,7 +1310,8 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
     }                                                                                 \
     note_launches(1);                                                                 \
     if (split && !counts) {                                                           \
-      fwd_split_combine_kernel<CC><<<GPF_MAX_SPLIT_UNITS / 4, 128, 0, stream>>>(a);   \
+      fwd_split_combine_kernel<CC><<<GPF_MAX_SPLIT_UNITS / 4, 128, 0, stream>>>(      \
+          a, team == 1 && kern != kKernDisk, kern == kKernDisk);                      \
       note_launches(1);                                                               \
     }                                                                                 \
     break;

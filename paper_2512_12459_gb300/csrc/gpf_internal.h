@@ -100,9 +100,11 @@ struct IndexBuffers {
   void* nbsort_ws;
   int nbsorted;
   // forward tile splitting (split_items > 0)
-  uint32_t* tparts;     // [tiles_max] cost, then parts of each tile (1 = not split)
-  uint4* xunit;         // [GPF_MAX_SPLIT_UNITS] (tile, part, parts, valid) of every split unit
-  float* xsum;          // [GPF_MAX_SPLIT_UNITS * (C + 1) * 32] partial sums of split units
+  uint32_t* tparts;     // [tiles_max] parts of each tile's sums, a bit where several units have it
+  uint32_t* xpart;      // [tiles_max / 256 + 1] parts of the split tiles of 256 tiles
+  uint32_t* tcost;      // [tiles_max] estimated work of each tile
+  uint4* xunit;         // [GPF_MAX_SPLIT_UNITS] the units of those tiles
+  float* xsum;          // [GPF_MAX_SPLIT_UNITS * (C + 1) * 32] sums of split tiles' parts
   uint32_t* xheavy;     // [tiles_max] tiles deferred to the forward's second launch
   // a centre level (ball_radius > 0): occupancy bits of the centre cells'
   // coarse cells (Grid::cshift), and the hybrid forward's tile splitting
