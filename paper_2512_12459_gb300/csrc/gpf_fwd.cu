@@ -1275,10 +1275,16 @@ cudaError_t launch_forward(const IndexDims& d, const IndexBuffers& b, const gpf_
     const int smem =                                                                         \
         (int)sizeof(float) * warps * warp_shared_words(CC, d.grid.levels, d.grid.coop);      \
     const auto kernel = fwd_kernel<CC, BR, PS, CN, TM>;                                      \
-    cudaError_t e = cudaSuccess;                                                             \
-    if (smem > 48 * 1024)                                                                    \
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);   \
-    if (e != cudaSuccess) return e;                                                          \
+    /* the limit belongs to the kernel, which other indexes launch from other threads: */    \
+    /* always the same value, the most any index needs */                                    \
+    constexpr int most =                                                                     \
+        (int)sizeof(float) * warps * warp_shared_words(CC, GPF_MAX_LEVELS, GPF_MAX_COOP_CELLS); \
+    static_assert(most <= 227 * 1024, "a block's shared memory");                            \
+    if (most > 48 * 1024) {                                                                  \
+      const cudaError_t e =                                                                  \
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);   \
+      if (e != cudaSuccess) return e;                                                        \
+    }                                                                                        \
     const unsigned blocks = (unsigned)persistent_blocks(                                     \
         reinterpret_cast<const void*>(kernel), warps * kWarp, want, smem);                   \
     kernel<<<blocks, warps * kWarp, smem, stream>>>(a);                                      \

@@ -55,3 +55,42 @@ def test_products_that_overflow_reach_their_own_gaussians_only(gpf, channels, ce
                             <= 3.0 * np.exp(fnp.logscale.max(axis=0)) * 1.001).cuda()
     for a, b in zip(grads[0].tensors(), grads[1].tensors()):
         assert torch.equal(a[:, ~near], b[:, ~near])
+
+
+def test_two_threads_with_indexes_of_different_levels(gpf):
+    """Small queries through one kernel from two host threads, each on a stream
+    and an index of its own, whose warps need different shared memory."""
+    import threading
+
+    import torch
+    from paper_2512_12459_gb300.setup_index import make_index
+    fnp, qnp = synth.config1_random(seed=5, n=300, m=640)
+    field, queries = gpf.Field.from_numpy(fnp), gpf.Queries.from_numpy(qnp)
+    work = []
+    for levels, coop in ((16, 8), (6, 8), (10, 8)):
+        grid = gpf.grid_for_bounds([0.0] * 3, [1.0] * 3, 0.01, 3, 300, 640, 200_000,
+                                   levels=levels, query_level=2, hash_bits=14)
+        grid.coop_cells = coop
+        idx = make_index(field, queries, grid=grid)
+        idx.build(field, queries)
+        out, _ = gpf.gpf_radiance_fwd(idx, field, queries, gpf.GPF_SUM)
+        work.append((idx, out, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    errors = []
+
+    def run(idx, out, stream):
+        try:
+            with torch.cuda.stream(stream):
+                for _ in range(2000):
+                    o, _ = gpf.gpf_radiance_fwd(idx, field, queries, gpf.GPF_SUM)
+                stream.synchronize()
+                assert torch.equal(o, out)
+        except Exception as e:              # noqa: BLE001 (reported by the main thread)
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=run, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
