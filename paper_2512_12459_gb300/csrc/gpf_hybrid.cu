@@ -303,24 +303,34 @@ __device__ int warp_knn(const HybArgs& a, bool need, float px, float py, float p
       // the occupancy cells under a slice, and the fine bits' words of its rows
       const int cs = G.cshift - Lb;
       const int ux0 = fx0 >> cs, uy0 = fy0 >> cs;
-      const int unx = (fx1 >> cs) - ux0 + 1, nu = unx * ((fy1 >> cs) - uy0 + 1);
+      const int unx = (fx1 >> cs) - ux0 + 1, uny = (fy1 >> cs) - uy0 + 1;
       const int fw0 = fx0 >> 5, fnw = (fx1 >> 5) - fw0 + 1;
       const int per_slice = fnw * (fy1 - fy0 + 1);
       for (int zb = max(z0, 0); zb <= fz1; zb += kWarp) {
-        // the slices that hold a mean, by the coarse bits, one slice per lane
-        uint32_t any = 0u;
-        if (zb + lane <= fz1) {
-          const uint32_t uz = (uint32_t)((zb + lane) >> cs) * G.cdy;
-          for (int u = 0, ux = 0, uy = 0; u < nu; ++u) {
-            const uint32_t bit = (uz + (uint32_t)(uy0 + uy)) * G.cdx + (uint32_t)(ux0 + ux);
-            any |= (__ldg(a.cocc + (bit >> 5)) >> (bit & 31u)) & 1u;
-            if (++ux == unx) {
-              ux = 0;
-              ++uy;
+        // the slices that hold a mean, by the coarse bits: a lane takes a row of
+        // coarse cells along x, whose bits are consecutive, of any of the layers
+        // under the 32 slices (a slice per lane, each reading all the cells under
+        // it, left the other lanes waiting where a field is a few cells high)
+        const int uz0 = zb >> cs, zl = min(zb + kWarp - 1, fz1);
+        const int crows = ((zl >> cs) - uz0 + 1) * uny;
+        uint32_t layers = 0u;
+        for (int t = lane; t < crows; t += kWarp) {
+          const int l = t / uny, uy = uy0 + t - l * uny;
+          const uint32_t b0 = ((uint32_t)(uz0 + l) * G.cdy + (uint32_t)uy) * G.cdx + (uint32_t)ux0;
+          const uint32_t b1 = b0 + (uint32_t)unx - 1u;      // the row's first and last bit
+          for (uint32_t w = b0 >> 5; w <= b1 >> 5; ++w) {
+            uint32_t m = __ldg(a.cocc + w);
+            if (w == b0 >> 5) m &= 0xffffffffu << (b0 & 31u);
+            if (w == b1 >> 5) m &= 0xffffffffu >> (31u - (b1 & 31u));
+            if (m) {
+              layers |= 1u << l;
+              break;
             }
           }
         }
-        const uint32_t slices = __ballot_sync(kFullMask, any != 0u);
+        layers = __reduce_or_sync(kFullMask, layers);
+        const uint32_t slices = __ballot_sync(
+            kFullMask, zb + lane <= fz1 && ((layers >> (((zb + lane) >> cs) - uz0)) & 1u));
         // their rows' words, one per lane: the occupied cells of the ring
         const int words = __popc(slices) * per_slice;
         for (int wb = 0; wb < words; wb += kWarp) {

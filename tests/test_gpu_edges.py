@@ -94,3 +94,31 @@ def test_two_threads_with_indexes_of_different_levels(gpf):
     for t in threads:
         t.join()
     assert not errors, errors[0]
+
+
+@pytest.mark.parametrize("n", [40, 400, 4000])
+@pytest.mark.parametrize("height", [0.0, 0.05, 0.7])
+def test_nearest_means_of_a_field_a_few_cells_high(gpf, n, height):
+    """Means and hit points on a floor (and up to a height above it): rings of
+    many coarse cells in one or a few layers. The nearest means are summed by
+    distance, so cells of another size give the same sums bit for bit."""
+    from paper_2512_12459_gb300.setup_index import make_index
+    rng = np.random.default_rng(n)
+    fnp, qnp = synth.config1_random(seed=n, n=n, m=1500)
+    fnp.mean = np.concatenate([rng.uniform(0, 2, (2, n)), rng.uniform(0, 1, (1, n)) * height]
+                              ).astype(np.float32)
+    qnp.x = np.concatenate([rng.uniform(0, 2, (2, 1500)), rng.uniform(0, 1, (1, 1500)) * height]
+                           ).astype(np.float32)
+    field, queries = gpf.Field.from_numpy(fnp), gpf.Queries.from_numpy(qnp)
+    outs = []
+    for ball in (0.02, 0.05, 0.4):
+        idx = make_index(field, queries, query_cell=0.05, ball_radius=ball)
+        idx.build(field, queries)
+        assert idx.stats()["flags"] == 0
+        outs.append(gpf.gpf_radiance_fwd(idx, field, queries, gpf.GPF_SUM, r_max=0.5,
+                                         neighbourhood=gpf.GPF_NB_BALL_KNN, ball_r=0.0,
+                                         k_min=4)[0].cpu().numpy())
+    assert outs[0].any()
+    for o in outs[1:]:
+        np.testing.assert_array_equal(o, outs[0])
+
