@@ -122,3 +122,85 @@ def test_nearest_means_of_a_field_a_few_cells_high(gpf, n, height):
     for o in outs[1:]:
         np.testing.assert_array_equal(o, outs[0])
 
+
+
+# two float32 sums of the same positive terms, at most 2000 of them, in
+# different orders: below 2000 * 2^-24 apart relative to the sum
+SUM_RTOL = 1.2e-4
+
+
+def _on_and_by_brute_force(gpf, fnp, qnp, mode, r, **kw):
+    """(out, z) on a grid, twice, and by brute force; the pairs agree."""
+    from paper_2512_12459_gb300.setup_index import make_index
+    field, queries = gpf.Field.from_numpy(fnp), gpf.Queries.from_numpy(qnp)
+    res, counts = [], []
+    for k in (kw, {"brute_force": True}):
+        idx = make_index(field, queries, cutoff_sigma=3.0, **k)
+        idx.build(field, queries)
+        assert idx.stats()["flags"] == 0
+        for _ in range(1 if "brute_force" in k else 2):
+            out, z = gpf.gpf_radiance_fwd(idx, field, queries, mode, r_max=r)
+            res.append((out.cpu().numpy(), z.cpu().numpy()))
+        counts.append(gpf.gpf_count_pairs(idx, field, queries)["included"])
+    assert counts[0] == counts[1]
+    return res
+
+
+@pytest.mark.parametrize("tiles,every", [(1000, 1), (3000, 1), (6000, 3), (5000, 1)])
+def test_density_estimate_whose_samples_miss_a_dense_cell(gpf, tiles, every):
+    """A photon gather in which one unsampled point of (every third of) the tiles
+    stands in a dense cell of 1,600 photons, so that these tiles are put off to the
+    second launch: with teams of 16 and of 4 warps, one warp, and more tiles than
+    the second launch has room to split."""
+    m, per, r = 32 * tiles, 1600, 0.02
+    a = np.array([1.1, 1.1, 1.1])
+    x = np.tile(a + 0.12, (m, 1))                 # (one query-level cell: index order)
+    x[1::32 * every] = a
+    mean = np.concatenate([np.tile(a, (per, 1)), np.tile(a + 0.12, (5, 1)), [[0.0] * 3, [4.0] * 3]])
+    fnp, qnp = synth.config1_random(seed=tiles, n=len(mean), m=m)
+    fnp.mean = np.ascontiguousarray(mean.T.astype(np.float32))
+    fnp.logscale[:] = math.log(r / 3.0)
+    qnp.x = np.ascontiguousarray(x.T.astype(np.float32))
+    qnp.n[:], qnp.valid = qnp.wo, np.ones_like(qnp.valid)
+    (o, z), (o2, z2), (ob, zb) = _on_and_by_brute_force(gpf, fnp, qnp, gpf.GPF_DISK_KDE, r,
+                                                        query_cell=0.85, split_items=64)
+    np.testing.assert_array_equal(z, np.where(np.arange(m) % (32 * every) == 1, per, 5))
+    np.testing.assert_array_equal(z, zb)
+    np.testing.assert_array_equal(o, o2)
+    np.testing.assert_array_equal(z, z2)
+    np.testing.assert_allclose(o, ob, rtol=SUM_RTOL, atol=1e-30)
+
+
+@pytest.mark.parametrize("m", [32, 32 * 152 * 32 + 32])
+@pytest.mark.parametrize("split", [0, 64])
+def test_tiles_of_more_than_32_walked_lists(gpf, m, split):
+    """Hit points in eight cells on each of six levels: 48 lists a tile."""
+    rng = np.random.default_rng(m)
+    at = 0.1 + 0.25 * np.stack(np.meshgrid(range(4), range(4), [0], indexing="ij"), -1).reshape(-1, 3)[:8]
+    x = at[np.arange(m) % 8] + 1e-4 * rng.standard_normal((m, 3))
+    k = np.repeat(np.arange(8), 6 * 40)
+    fnp, qnp = synth.config1_random(seed=m % 1000, n=len(k), m=m)
+    fnp.mean = (at[k] + 1e-4 * rng.standard_normal((len(k), 3))).T.astype(np.float32).copy()
+    fnp.logscale = np.tile(np.log(3e-4 * 2.0 ** (np.arange(len(k)) % 6)), (3, 1)).astype(np.float32)
+    qnp.x = np.ascontiguousarray(x.T.astype(np.float32))
+    qnp.n[:], qnp.valid = qnp.wo, np.ones_like(qnp.valid)
+    grid = gpf.grid_for_bounds([0.0] * 3, [1.0] * 3, 8e-4, 3, len(k), m, 100_000, levels=6,
+                               query_level=10, hash_bits=16)
+    grid.coop_cells = 8
+    (o, z), (o2, _), (ob, zb) = _on_and_by_brute_force(gpf, fnp, qnp, gpf.GPF_SUM, math.inf,
+                                                       grid=grid, split_items=split)
+    np.testing.assert_array_equal(o, o2)
+    np.testing.assert_allclose(z, zb, rtol=SUM_RTOL, atol=1e-30)
+    np.testing.assert_allclose(o, ob, rtol=SUM_RTOL, atol=1e-30)
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 16383, 16384, 16385])
+@pytest.mark.parametrize("span", [3, 9])
+def test_edges_of_the_groups_that_list_their_entries(gpf, n, span):
+    """Every Gaussian of the last, partly filled group of 256 and super-group of
+    64 groups."""
+    fnp, qnp = synth.config1_random(seed=n, n=n, m=2000)
+    fnp.logscale = (fnp.logscale - 0.33 * math.log(n / 64.0)).astype(np.float32)
+    (_, z), _, (_, zb) = _on_and_by_brute_force(gpf, fnp, qnp, gpf.GPF_SUM, math.inf,
+                                                max_span=span)
+    np.testing.assert_allclose(z, zb, rtol=SUM_RTOL, atol=1e-30)
