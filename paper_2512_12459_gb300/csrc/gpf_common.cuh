@@ -200,20 +200,31 @@ struct CellHash {
 // mean on the centre level): a key space apart from the box entries'.
 constexpr uint64_t kCentreSalt = 0xd1b54a32d192ed03ull;
 
+// The cell as the hash takes it: the next cell in x, y and z is 1, 2^20 and 2^40
+// more, so the words of a box's cells differ by constants.
+__host__ __device__ __forceinline__ uint64_t cell_word(int L, uint32_t ix, uint32_t iy,
+                                                       uint32_t iz) {
+  return (uint64_t)ix | ((uint64_t)iy << 20) | ((uint64_t)iz << 40) | ((uint64_t)L << 60);
+}
+__host__ __device__ __forceinline__ uint64_t mix_word(uint64_t z) {
+  z += 0x9e3779b97f4a7c15ull;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  return (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+}
+// (the finaliser's last step, z ^ (z >> 31), leaves the top 31 bits as they are, and
+// a bucket is at most 28)
+__host__ __device__ __forceinline__ uint32_t bucket_of_word(const Grid& g, uint64_t word) {
+  return (uint32_t)(mix_word(word) >> 32) >> (32 - g.hash_bits);
+}
 __host__ __device__ __forceinline__ CellHash cell_hash(const Grid& g, int L, uint32_t ix,
                                                        uint32_t iy, uint32_t iz,
                                                        uint64_t salt = 0) {
-  uint64_t z = ((uint64_t)ix | ((uint64_t)iy << 20) | ((uint64_t)iz << 40) |
-                ((uint64_t)L << 60)) ^ salt;
-  z += 0x9e3779b97f4a7c15ull;
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-  z ^= z >> 31;
+  const uint64_t z = mix_word(cell_word(L, ix, iy, iz) ^ salt);
   CellHash h;
-  h.bucket = (uint32_t)(z >> (64 - g.hash_bits));
+  h.bucket = (uint32_t)(z >> 32) >> (32 - g.hash_bits);
   // (a centre entry and a box entry of one Gaussian in one bucket never have the
   // same tag: the highest bit tells them apart)
-  h.tag = (((uint32_t)z << g.id_bits) & 0x7fffffffu) | (salt ? 0x80000000u : 0u);
+  h.tag = (((uint32_t)(z ^ (z >> 31)) << g.id_bits) & 0x7fffffffu) | (salt ? 0x80000000u : 0u);
   return h;
 }
 // [start, end) of a bucket's list ([0, 0): it has none).
@@ -224,7 +235,7 @@ __device__ __forceinline__ uint2 bucket_list(const uint32_t* __restrict__ listed
 }
 __host__ __device__ __forceinline__ uint32_t bucket_of(const Grid& g, int L, uint32_t ix,
                                                        uint32_t iy, uint32_t iz) {
-  return cell_hash(g, L, ix, iy, iz).bucket;
+  return bucket_of_word(g, cell_word(L, ix, iy, iz));
 }
 
 // What the pair loops vet an entry by, one 32-byte load: the mean, the radius

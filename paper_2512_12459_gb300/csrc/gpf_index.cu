@@ -199,11 +199,12 @@ __device__ __forceinline__ unsigned long long small_box_mask(
     const Grid& grid, const uint32_t* __restrict__ occ, int L, uint32_t lx, uint32_t ly,
     uint32_t lz, uint32_t sx, uint32_t sy, uint32_t sz) {
   unsigned long long mask = 0;
-  for (uint32_t dz = 0; dz <= sz; ++dz) {
+  uint64_t cell = cell_word(L, lx, ly, lz);
+  for (uint32_t dz = 0; dz <= sz; ++dz, cell += uint64_t(1) << 40) {
     uint32_t bkt[N * N], word[N * N];
 #pragma unroll
     for (int j = 0; j < N * N; ++j) {
-      bkt[j] = bucket_of(grid, L, lx + j % N, ly + j / N, lz + dz);
+      bkt[j] = bucket_of_word(grid, cell + (uint64_t)(j % N) + ((uint64_t)(j / N) << 20));
       word[j] = (uint32_t)(j % N) <= sx && (uint32_t)(j / N) <= sy ? __ldg(occ + (bkt[j] >> 5)) : 0u;
     }
     uint32_t bits = 0;
@@ -500,8 +501,8 @@ __global__ void query_keys_kernel(Grid grid, const float* __restrict__ x,
 // One (bucket, Gaussian) entry per occupied cell of every Gaussian's level
 // box, in the box's cell order, at the Gaussian's offset (the entries of the
 // Gaussians before it). A Gaussian whose cells share a bucket appears there on
-// consecutive entries; the pair loops take only the first. A block takes one
-// group of preprocess and adds up the counts before it; a warp lays the
+// consecutive entries; the pair loops take only the first. A block takes the
+// groups of preprocess in strides and adds up the counts before each; a warp lays the
 // entries of its 32 Gaussians end to end and writes 32 at a time, so that the
 // stores are coalesced and no lane waits for the Gaussian with the most cells
 // (a thread per Gaussian: 53 us and scattered 4-byte stores at 3.8 M entries).
