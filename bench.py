@@ -136,23 +136,37 @@ def measured_peaks():
 
 
 # DRAM bytes (read + write) per launch of the pair-loop kernels on this
-# workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum,
-# third warm-up step of `python bench.py --steps 3 --warmup 3
-# --no-cpu-baseline --grid 0.0307543,3,8,4096`; the forward's two launches
-# together), with the SHA-256 of the sources the kernel was built from;
-# reported only while those sources are unchanged.
-PROFILED_TRAFFIC = {
-    "fwd_kernel": {"bytes": 247116800 + 18750720, "sources": {
-        "paper_2512_12459_gb300/csrc/gpf_fwd.cu":
-            "10dc4679b2ae84a450f8f043b7406a70a993c165a25df7cfcc282dd3de3cfc74",
+# workload, each from an ncu capture (dram__bytes_read.sum +
+# dram__bytes_write.sum, third warm-up step of `python bench.py --steps 3
+# --warmup 3 --no-cpu-baseline --grid G`), with the grid G and the SHA-256 of the
+# sources the kernel was built from; reported only for that grid and while those
+# sources are unchanged.
+_FWD = {"paper_2512_12459_gb300/csrc/gpf_fwd.cu":
+            "35f32490a7e93ebd0324f0210b4e8408a91008d13787d1ccef3529cb6b04ba8a",
         "paper_2512_12459_gb300/csrc/gpf_common.cuh":
-            "4f754dc2ca658c27f73638001642c474908868ab0c7d454b2cb2031f4d3b6d5b"}},
-    "bwd_pairs_kernel": {"bytes": 156698112 + 59414016, "sources": {
-        "paper_2512_12459_gb300/csrc/gpf_bwd.cu":
-            "02fa41568274384cbaeabc01ade438a7d3306c9541daac70182ffda0b07d28de",
+            "691856f88615e12068bca80fd0caaf8836792ec62c86acf0a1115c38bbd3a606"}
+_BWD = {"paper_2512_12459_gb300/csrc/gpf_bwd.cu":
+            "ae6c55dafef5aa3bb0e7e066c485a8e3cf124680dbbbaaa7e67d79be9ea21632",
         "paper_2512_12459_gb300/csrc/gpf_common.cuh":
-            "4f754dc2ca658c27f73638001642c474908868ab0c7d454b2cb2031f4d3b6d5b"}},
-}
+            "691856f88615e12068bca80fd0caaf8836792ec62c86acf0a1115c38bbd3a606"}
+PROFILED_TRAFFIC = [
+    {"kernel": kernel, "sources": sources, "grid": (cell, 3, 8, split), "bytes": read + written}
+    for kernel, sources, cell, split, read, written in (
+        ("fwd_kernel", _FWD, 0.03075434, 4096, 147423744, 12975872),
+        ("fwd_kernel", _FWD, 0.03075434, 0, 130246912, 11461376),
+        ("fwd_kernel", _FWD, 0.01537717, 4096, 148023296, 13519104),
+        ("fwd_kernel", _FWD, 0.01537717, 0, 129993216, 11306496),
+        ("bwd_grid_kernel", _BWD, 0.03075434, 4096, 151176960, 48704768),
+        ("bwd_grid_kernel", _BWD, 0.03075434, 0, 151159296, 49044480),
+        ("bwd_grid_kernel", _BWD, 0.01537717, 4096, 177943808, 48784896),
+        ("bwd_grid_kernel", _BWD, 0.01537717, 0, 178549760, 48850944))]
+
+
+def grid_key(grid):
+    """What a kernel's traffic depends on besides the scene: query cell, max
+    span, cooperative cells, split items."""
+    return (grid.cell_size * (1 << grid.query_level), grid.max_span, grid.coop_cells,
+            grid.split_items)
 
 
 def _sha256(path: str) -> str:
@@ -161,13 +175,15 @@ def _sha256(path: str) -> str:
         return hashlib.sha256(fh.read()).hexdigest()
 
 
-def profiled_traffic(kernel: str):
-    rec = PROFILED_TRAFFIC.get(kernel)
-    if rec is None:
-        return None
-    if any(_sha256(p) != h for p, h in rec["sources"].items()):
-        return None
-    return rec["bytes"]
+def profiled_traffic(kernel: str, grid):
+    """The captured bytes of `kernel` on the grid of this run (query cell, max
+    span, cooperative cells, split items), or None."""
+    for rec in PROFILED_TRAFFIC:
+        if rec["kernel"] != kernel or any(_sha256(p) != h for p, h in rec["sources"].items()):
+            continue
+        if rec["grid"][1:] == tuple(grid[1:]) and abs(rec["grid"][0] - grid[0]) < 1e-4 * grid[0]:
+            return rec["bytes"]
+    return None
 
 
 def fp32_peak_tflops(sm_mhz_max: float, sms: int = 152) -> float:
@@ -981,7 +997,7 @@ def main():
         per["step"].append(mk[0].elapsed_time(mk[5]))
     ms = {k: float(np.mean(v)) for k, v in per.items()}
     kernel_ms = {"fwd_kernel": float(np.mean([mk[6].elapsed_time(mk[7]) for mk in all_marks])),
-                 "bwd_pairs_kernel": float(np.mean([mk[8].elapsed_time(mk[9]) for mk in all_marks]))}
+                 "bwd_grid_kernel": float(np.mean([mk[8].elapsed_time(mk[9]) for mk in all_marks]))}
     step_ms = sharding.max_over_ranks(ms["step"], device="cuda")
     total_q = float(n_total)
     value = total_q / (step_ms / 1000.0)
@@ -1063,12 +1079,12 @@ def main():
         fwd_flops = inc * (25 + 2 * C)       # per included pair, FMA = 2 flops
         bwd_flops = inc * (55 + 4 * C)
         fwd_ach = fwd_flops / (kernel_ms["fwd_kernel"] / 1e3) / 1e12
-        bwd_ach = bwd_flops / (kernel_ms["bwd_pairs_kernel"] / 1e3) / 1e12
-        dom = "bwd_pairs_kernel" if kernel_ms["bwd_pairs_kernel"] >= kernel_ms["fwd_kernel"] \
+        bwd_ach = bwd_flops / (kernel_ms["bwd_grid_kernel"] / 1e3) / 1e12
+        dom = "bwd_grid_kernel" if kernel_ms["bwd_grid_kernel"] >= kernel_ms["fwd_kernel"] \
             else "fwd_kernel"
-        ach = bwd_ach if dom == "bwd_pairs_kernel" else fwd_ach
+        ach = bwd_ach if dom == "bwd_grid_kernel" else fwd_ach
         roof = {"bound": "alu", "kernel": dom, "achieved": ach, "peak": fp32_peak,
-                "unit": "TFLOP/s", "frac": ach / fp32_peak, "traffic": profiled_traffic(dom),
+                "unit": "TFLOP/s", "frac": ach / fp32_peak, "traffic": profiled_traffic(dom, grid_key(idx.grid)),
                 "peak_source": "measured FP32 FMA rate of this GPU (gpf_measure_alu_peak); "
                                f"nominal 152 SMs x 128 lanes x 2 x {smax:.0f} MHz = "
                                f"{nominal_fp32:.1f}",
@@ -1077,7 +1093,7 @@ def main():
         extra = {"included_pairs": inc, "candidate_pairs": pairs["candidates"],
                  "fwd_alu_frac": fwd_ach / fp32_peak, "bwd_alu_frac": bwd_ach / fp32_peak,
                  "fwd_sfu_frac": inc / (kernel_ms["fwd_kernel"] / 1e3) / 1e12 / ex2_peak,
-                 "bwd_sfu_frac": inc / (kernel_ms["bwd_pairs_kernel"] / 1e3) / 1e12 / ex2_peak}
+                 "bwd_sfu_frac": inc / (kernel_ms["bwd_grid_kernel"] / 1e3) / 1e12 / ex2_peak}
 
     cpu, err = None, None
     if pool is not None:
